@@ -455,7 +455,10 @@ static rw_status build_factors(rw_context* ctx, std::vector<MatBuild>& mbs, uint
         }
         wb.nmat = nmat;
         wb.total = total;
-        for (const auto& mb : mbs) wb.table_bytes += table_bytes(mb.T);
+        for (const auto& mb : mbs) {
+            wb.table_bytes += table_bytes(mb.T);
+            wb.huge = wb.huge || has_huge_nodes(mb.T);
+        }
         wb.nrows = (int32_t)rows;
         if (nmat == 1) {
             wb.m0 = hmats[0];
@@ -507,7 +510,7 @@ static rw_status build_factors(rw_context* ctx, std::vector<MatBuild>& mbs, uint
         }
         WalkLaunch wl;
         wl.max_steps = ctx->opt.max_steps;
-        wl.record_lengths = ctx->opt.record_lengths;
+        wl.record_lengths = ctx->opt.record_lengths ? 1 : 0;
         const int64_t launches0 = g_launches;
         if (reuse) {
             wl.record_lengths = 0;

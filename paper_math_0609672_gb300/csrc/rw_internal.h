@@ -96,27 +96,34 @@ inline int grid_for(int64_t work, int block, int max_blocks) {
 //         order) form ng = ceil((1 + deg) / 4) groups; slot j lives in group
 //         j / 4, word j % 4 its threshold (0 for the header slot: always
 //         passed), word 4 + j % 4 its successor word (the successor's node
-//         index in bits 27..0, in bits 31..28 its class: 0 without a
-//         summary, ng for 3 <= ng <= 8, 15 above; deg for the header slot,
-//         0 for padding).
+//         index in bits 27..0, in bits 31..28 its class: ng up to 8, 15
+//         above; deg for the header slot, kGroundWord for padding: a draw
+//         past every threshold lands on it, or past the last group).
 //           sectors [0, 2n): node j's groups at 2j, 2j + 1 when ng <= 2;
-//           sectors [2n, 3n): node j's summary at 2n + j when ng > 2 -- deg in
-//             word 0, in words 1..7 the last threshold of groups 0..6
-//             (0xFFFFFFFF past the last);
+//           sectors [2n, 3n): node j's summary, 16 bytes at byte 64n + 16j,
+//             when ng > 2 -- the upper halves of the last thresholds of
+//             groups 0..6 (0xFFFF past the last);
 //           sectors [3n, 11n): node j's groups at 3n + 8j when 2 < ng <= 8
 //             (a fixed stride, so that a group's address needs no load);
 //           sectors [11n, 11n + G): the groups of the nodes with more than
 //             eight, at gbase[j] (a prefix over those nodes).
-//         The summaries (32 bytes per node, dense) stay in L2 on large
+//         The summaries (16 bytes per node, dense) stay in L2 on large
 //         matrices, so a hop to a node with a summary costs one DRAM sector
-//         (its group) besides one L2 read (two, with gbase, above eight
-//         groups); a node of at most seven neighbours costs one or two
-//         sectors of group 0/1.  Sectors [3n, 11n) are allocated for every
-//         node but touched only by the nodes that use it.
+//         (its group) besides one L2 read (three above eight groups).  A
+//         draw passes every group whose half threshold is below its own upper
+//         half; where the two are equal (7 draws in 65,536) the walk reads
+//         that group and goes on to the next if it is passed.  A node of at
+//         most seven neighbours costs one or two sectors of group 0/1.
+//         Sectors [3n, 11n) are allocated for every node but touched only by
+//         the nodes that use it.
 //  gbase: [n] the sector of each node's group 0.
 //  fthr:  per walk row a block [updeg, lowdeg, ft_0 .. ft_{updeg-1}, pad].
 // The walk works with node indices throughout (home: below the start row,
 // return: equal to it).  Padding thresholds are 0xFFFFFFFF.
+constexpr uint32_t kNodeMask = 0x0FFFFFFFu;
+constexpr uint32_t kHugeClass = 15u;
+constexpr uint32_t kGroundWord = kNodeMask;  // never a node: n < 2^28
+
 struct Tables {
     int32_t n = 0;
     uint32_t* tab = nullptr;
@@ -154,6 +161,8 @@ rw_status build_chunk_rows(rw_context* ctx, int32_t nw, const int64_t* wbase, in
 
 struct WalkLaunch {
     uint64_t max_steps = 1ull << 24;
+    // what a walk's record holds besides its end node: 0 its returns, 1 its
+    // length in hops; 2: length and returns, without the end node
     int record_lengths = 0;
 };
 
@@ -170,6 +179,7 @@ struct MatWalk {
 struct WalkBatch {
     int nmat = 1;
     uint64_t table_bytes = 0;      // walk-table bytes of all matrices
+    bool huge = false;             // some node has more than eight groups
     int32_t nrows = 0;             // walk rows of all matrices
     MatWalk m0{};                  // the single matrix (nmat == 1)
     const MatWalk* mats = nullptr; // [nmat] device (nmat > 1)
@@ -182,6 +192,7 @@ struct WalkBatch {
 };
 
 inline uint64_t table_bytes(const Tables& T) { return T.sectors * 32u + (uint64_t)T.n * 4u; }
+inline bool has_huge_nodes(const Tables& T) { return T.sectors > 11u * (uint64_t)T.n; }
 
 inline MatWalk mat_walk(const Tables& T, uint64_t seed, uint32_t matrix_index, uint32_t kind) {
     return MatWalk{T.tab, T.gbase, T.fthr, (uint32_t)seed, (uint32_t)(seed >> 32),

@@ -751,6 +751,7 @@ static rw_status pilot_run(rw_context* ctx, const rw_csr* A, uint32_t walks, uin
     WalkBatch wb;
     wb.m0 = mat_walk(T, seed, 0, 1);  // kind 1: pilot walks
     wb.table_bytes = table_bytes(T);
+    wb.huge = has_huge_nodes(T);
     wb.nrows = T.n_walk_rows;
     wb.wrow = T.wrow;
     wb.wbase = ws.wbase;

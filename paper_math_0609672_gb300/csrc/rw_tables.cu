@@ -203,22 +203,23 @@ __global__ void k_fill_tables(int32_t n, const int32_t* __restrict__ rp,
             w[0] = cumulative_threshold(c, dg);
             const int32_t jc = col[p];
             const uint32_t ngc = (uint32_t)(deg[jc] + 4) / 4u;
-            // bits 31..28: the successor's group class (0: no summary, 3..8:
-            // its ng, 15: more than eight groups)
-            const uint32_t cls = ngc <= 2u ? 0u : ngc <= 8u ? ngc : 15u;
+            // bits 31..28: the successor's group class (1..8: its ng, 15:
+            // more than eight groups)
+            const uint32_t cls = ngc <= 8u ? ngc : kHugeClass;
             w[4] = (uint32_t)jc | (cls << 28);
             ++j;
         }
         for (; j < ng * 4u; ++j) {
             uint32_t* w = word(j);
             w[0] = 0xFFFFFFFFu;
-            w[4] = 0u;
+            w[4] = kGroundWord;
         }
         if (big) {
-            // summary: deg, then the threshold of the last slot of groups 0..6
-            uint32_t* sw = tab + (2u * (uint64_t)n + (uint64_t)l) * 8u;
-            sw[0] = (uint32_t)d;
-            for (uint64_t g = 0; g < 7u; ++g) sw[1 + g] = g < ng ? *word(4u * g + 3u) : 0xFFFFFFFFu;
+            // summary: the upper halves of the last thresholds of groups 0..6
+            uint32_t hi[8];
+            for (uint32_t g = 0; g < 8u; ++g) hi[g] = g < 7u && g < ng ? *word(4u * g + 3u) >> 16 : 0xFFFFu;
+            *reinterpret_cast<uint4*>(tab + (size_t)n * 16u + (size_t)l * 4u) =
+                make_uint4(hi[0] | hi[1] << 16, hi[2] | hi[3] << 16, hi[4] | hi[5] << 16, hi[6] | hi[7] << 16);
         }
         const int32_t up = d - lo;
         double cu = 0.0;
