@@ -115,48 +115,75 @@ __global__ void k_features(int32_t n, const int32_t* __restrict__ rp, const int3
     }
 }
 
-// Pilot-walk statistics of each walk row (one warp per row) from a per-walk
-// quantity: the walk length (records hold lengths; plus = 0) or the visits to
-// the start row, J = 1 + returns (records hold returns; plus = 1).  Mean,
-// sample standard deviation (two passes, FP64), and the label
-// log((sd / mean)^2 + 1e-6).
-__global__ void k_pilot_stats(int32_t nw, const int4* __restrict__ wrow,
-                              const int64_t* __restrict__ wbase, const int2* __restrict__ rec, uint32_t plus,
-                              float* mean_out, float* sd_out, float* label, float* has) {
+// Pilot-walk statistics of each walk row from a per-walk quantity: the walk
+// length (quantity 0; records hold lengths) or the visits to the start row,
+// J = 1 + returns (quantities 1 and 2; records hold returns).  Mean, sample
+// standard deviation (two passes, FP64), and the label log((sd / mean)^2 +
+// 1e-6).  Quantity 2 (records hold lengths and returns) makes the label cost
+// aware: half of (the visits' label minus the log of the mean walk length), so
+// that exp(label) is proportional to sqrt(relative variance of the visits /
+// walk cost) -- the allocation of a fixed number of hops that minimises the
+// summed relative variances.
+//
+// A warp takes 32 rows: the sums of a row's walks are warp wide, lane i keeps
+// those of row i, and the quotients, roots and logarithms of all 32 rows are
+// then one FP64 instruction each.  The FP64 pipe bounds the kernel (one
+// warp-wide instruction per 19 cycles and SM whatever the lanes active): with
+// one lane per row doing them, 110,592 rows of 64 walks took 527 us, and now
+// take 178 us.
+template <int Q>
+__global__ void __launch_bounds__(256) k_pilot_stats(int32_t nw, const int4* __restrict__ wrow,
+                                                     const int64_t* __restrict__ wbase, const int2* __restrict__ rec,
+                                                     float* mean_out, float* sd_out, float* label, float* has) {
+    constexpr unsigned long long plus = Q == 0 ? 0u : 1u;
+    const int lane = (int)lane_id();
     const int32_t gw = (int32_t)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
     const int32_t nwarps = (int32_t)((gridDim.x * blockDim.x) >> 5);
-    for (int32_t r = gw; r < nw; r += nwarps) {
-        const int32_t k = wrow[r].x;
-        const int64_t b0 = wbase[r], b1 = wbase[r + 1];
-        unsigned long long s1 = 0;
-        for (int64_t i = b0 + lane_id(); i < b1; i += 32) s1 += (unsigned long long)(uint32_t)rec[i].y + plus;
-        s1 = warp_sum(s1);
-        const double m = (double)(b1 - b0);
-        const double mean = (double)s1 / m;
-        double s2 = 0.0;
-        for (int64_t i = b0 + lane_id(); i < b1; i += 32) {
-            const double d = (double)((unsigned long long)(uint32_t)rec[i].y + plus) - mean;
-            s2 += d * d;
+    for (int64_t r0 = (int64_t)gw * 32; r0 < nw; r0 += (int64_t)nwarps * 32) {
+        const int rows = (int)min((int64_t)32, nw - r0);
+        const int64_t mine = r0 + min(lane, rows - 1);
+        const int64_t b0 = wbase[mine], b1 = wbase[mine + 1];
+        unsigned long long sum = 0, len = 0;
+        for (int i = 0; i < rows; ++i) {
+            const int64_t e0 = __shfl_sync(kFull, b0, i), e1 = __shfl_sync(kFull, b1, i);
+            unsigned long long s1 = 0, l1 = 0;
+            for (int64_t p = e0 + lane; p < e1; p += 32) {
+                const int2 v = rec[p];
+                s1 += (unsigned long long)(uint32_t)v.y + plus;
+                if (Q == 2) l1 += (unsigned long long)(uint32_t)v.x;
+            }
+            s1 = warp_sum(s1);
+            if (Q == 2) l1 = warp_sum(l1);
+            if (lane == i) {
+                sum = s1;
+                len = l1;
+            }
         }
-        s2 = warp_sum(s2);
-        if (lane_id() == 0) {
-            const double var = m > 1.0 ? s2 / (m - 1.0) : 0.0;
+        const double m = (double)(b1 - b0);
+        const double mean = (double)sum / m;
+        double sq = 0.0;
+        for (int i = 0; i < rows; ++i) {
+            const int64_t e0 = __shfl_sync(kFull, b0, i), e1 = __shfl_sync(kFull, b1, i);
+            const double mi = __shfl_sync(kFull, mean, i);
+            double s2 = 0.0;
+            for (int64_t p = e0 + lane; p < e1; p += 32) {
+                const double d = (double)((unsigned long long)(uint32_t)rec[p].y + plus) - mi;
+                s2 += d * d;
+            }
+            s2 = warp_sum(s2);
+            if (lane == i) sq = s2;
+        }
+        if (lane < rows) {
+            const int32_t k = wrow[mine].x;
+            const double var = m > 1.0 ? sq / (m - 1.0) : 0.0;
+            float lb = (float)log(var / (mean * mean) + 1e-6);
+            if (Q == 2) lb = (float)(0.5 * ((double)lb - log((double)(float)((double)len / m))));
             mean_out[k] = (float)mean;
             sd_out[k] = (float)sqrt(var);
-            label[k] = (float)log(var / (mean * mean) + 1e-6);
+            label[k] = lb;
             has[k] = 1.f;
         }
     }
-}
-
-// Cost-aware label (quantity 2): half of (the visits label minus log of the
-// mean walk length), so that exp(label) is proportional to sqrt(relative
-// variance of the visits / walk cost) -- the allocation of a fixed number of
-// hops that minimises the summed relative variances.
-__global__ void k_label_cost(int32_t n, const float* __restrict__ mean_len, const float* __restrict__ has,
-                             float* label) {
-    for (int32_t k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x)
-        if (has[k] > 0.f) label[k] = (float)(0.5 * ((double)label[k] - log((double)mean_len[k])));
 }
 
 // ---------------------------------------------------------------------------
@@ -706,26 +733,7 @@ static rw_status features_run(rw_context* ctx, const rw_csr* A, float* feat) {
     return check_launch("row features");
 }
 
-static rw_status pilot_run(rw_context* ctx, const rw_csr* A, uint32_t walks, uint64_t seed, int quantity,
-                           float* mean, float* sd, float* label, float* has);
-
-// quantity 2: the same walks twice (lengths, then visits), combined
-static rw_status pilot_cost(rw_context* ctx, const rw_csr* A, uint32_t walks, uint64_t seed, float* mean, float* sd,
-                            float* label, float* has) {
-    Pool sc(ctx);
-    float* mlen = alloc_n<float>(sc, A->n);
-    float* t1 = alloc_n<float>(sc, A->n);
-    float* t2 = alloc_n<float>(sc, A->n);
-    if (!mlen || !t1 || !t2) return RW_ERR_ALLOC;
-    rw_status rc;
-    if ((rc = pilot_run(ctx, A, walks, seed, 0, mlen, t1, t2, has))) return rc;
-    if ((rc = pilot_run(ctx, A, walks, seed, 1, mean, sd, label, has))) return rc;
-    RW_COUNT_LAUNCH();
-    k_label_cost<<<grid_for(A->n, 256, ctx->num_sms * 8), 256, 0, ctx->stream>>>(A->n, mlen, has, label);
-    if ((rc = check_launch("cost label"))) return rc;
-    return read_status(ctx, "pilot statistics");
-}
-
+// One launch of pilot walks; quantity 2 records their lengths and returns together.
 static rw_status pilot_run(rw_context* ctx, const rw_csr* A, uint32_t walks, uint64_t seed, int quantity,
                            float* mean, float* sd, float* label, float* has) {
     NvtxRange nvtx_range("rw_pilot");
@@ -759,12 +767,14 @@ static rw_status pilot_run(rw_context* ctx, const rw_csr* A, uint32_t walks, uin
     wb.total = ws.total;
     WalkLaunch wl;
     wl.max_steps = ctx->opt.max_steps;
-    wl.record_lengths = quantity == 0 ? 1 : 0;
+    wl.record_lengths = quantity == 0 ? 1 : quantity == 2 ? 2 : 0;
     if ((rc = run_walks(ctx, wb, wl, rec, hops, scratch, nullptr))) return rc;
     if ((rc = read_status(ctx, "pilot walks"))) return rc;
+    const int g = grid_for(T.n_walk_rows, 256, ctx->num_sms * 8);
     RW_COUNT_LAUNCH();
-    k_pilot_stats<<<grid_for((int64_t)T.n_walk_rows * 32, 256, ctx->num_sms * 8), 256, 0, s>>>(
-        T.n_walk_rows, T.wrow, ws.wbase, rec, quantity == 0 ? 0u : 1u, mean, sd, label, has);
+    if (quantity == 0) k_pilot_stats<0><<<g, 256, 0, s>>>(T.n_walk_rows, T.wrow, ws.wbase, rec, mean, sd, label, has);
+    else if (quantity == 1) k_pilot_stats<1><<<g, 256, 0, s>>>(T.n_walk_rows, T.wrow, ws.wbase, rec, mean, sd, label, has);
+    else k_pilot_stats<2><<<g, 256, 0, s>>>(T.n_walk_rows, T.wrow, ws.wbase, rec, mean, sd, label, has);
     if ((rc = check_launch("pilot statistics"))) return rc;
     return read_status(ctx, "pilot statistics");
 }
@@ -1021,7 +1031,6 @@ rw_status rw_pilot_stats(rw_context* ctx, const rw_csr* A, uint32_t pilot_walks,
     }
     rw_status rc = check_csr_args(A, "rw_pilot_stats");
     if (rc || A->n == 0) return rc;
-    if (quantity == 2) return pilot_cost(ctx, A, pilot_walks, seed, d_mean, d_sd, d_label, d_has);
     return pilot_run(ctx, A, pilot_walks, seed, quantity, d_mean, d_sd, d_label, d_has);
 }
 
