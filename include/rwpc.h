@@ -101,7 +101,8 @@ typedef struct {
                                 right-hand sides, power of two <= 32); 0 = one row per warp;
                                 -1 = vector rows: one row per warp, each lane reads all
                                 right-hand sides of its entries (default -1) */
-    int32_t spmv_slices;     /* SpMV: entry slices per row, as wide_slices; 0 = one row per warp */
+    int32_t spmv_slices;     /* SpMV: entry slices per row (lanes per row = slices x right-hand sides, power
+                                of two <= 32); 0 = from the average row length (default 0) */
     int32_t cluster_width;   /* levels of at most this many rows (above the thin-run width) run on
                                 one thread-block cluster with hardware barriers; 0 = never */
     int32_t cluster_size;    /* CTAs of that cluster (2..16; 0 = 16) */
@@ -425,7 +426,7 @@ rw_status rw_row_features(rw_context* ctx, const rw_csr* A, float* d_feat);
  * "expected number of returns" that Sec. 5.1 names as an alternative
  * b-independent quantity; it sets D_kk in Eq. newz).  quantity 2: the
  * visits' statistics with the cost-aware label
- * (log((sd/mean)^2 + 1e-6) - log Xi'_k) / 2 from the same walks recorded twice:
+ * (log((sd/mean)^2 + 1e-6) - log Xi'_k) / 2 from one set of walks recorded with lengths and returns:
  * exp(label) is then the allocation of a fixed hop count (walks cost Xi'_k
  * hops each) that minimises the sum of the rows' relative variances
  * (M_k proportional to sd_k / (mean_k sqrt(Xi'_k))).  Outputs are device

@@ -749,7 +749,7 @@ rw_status factor_tune_target(const rw_factor* F, const rw_csr* A, TuneTarget* X)
         return RW_ERR_ARG;
     }
     const rw_factor_desc& d = F->desc;
-    *X = TuneTarget{A->n, A->row_ptr, A->col, A->val, nullptr, d.y_row_ptr, d.y_col, d.y_val, d.y_val32,
+    *X = TuneTarget{A->n, A->nnz, A->row_ptr, A->col, A->val, nullptr, d.y_row_ptr, d.y_col, d.y_val, d.y_val32,
                     d.yt_row_ptr, d.yt_col, d.yt_val, d.yt_val32, d.d, d.d32, &F->fwd_sched, &F->bwd_sched,
                     F->bar, d.nnz, std::max(d.fwd_levels, d.bwd_levels)};
     return RW_OK;
@@ -824,9 +824,9 @@ rw_status rw_spmv(rw_context* ctx, const rw_csr* A, const double* d_x, double* d
     rw_status rc = check_csr(A);
     if (rc) return rc;
     if (A->n == 0) return RW_OK;
-    if ((rc = reset_status(ctx))) return rc;
+    // (the kernel reports nothing through the device status: no reset, no read back)
     if ((rc = spmv_fp64(ctx, A, d_x, d_y, nrhs))) return rc;
-    return read_status(ctx, "spmv");
+    return check_cuda(cudaStreamSynchronize(ctx->stream), "spmv");
 }
 
 }  // extern "C"

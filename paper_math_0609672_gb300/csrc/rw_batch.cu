@@ -426,7 +426,7 @@ rw_status batch_tune_target(const rw_batch* B, TuneTarget* X) {
         set_error("autotune: NULL batch");
         return RW_ERR_ARG;
     }
-    *X = TuneTarget{B->N, B->a_rp, B->a_col, B->a_val, B->a_val32, B->y_rp, B->y_col, B->y_val, B->y_val32,
+    *X = TuneTarget{B->N, B->nnzA, B->a_rp, B->a_col, B->a_val, B->a_val32, B->y_rp, B->y_col, B->y_val, B->y_val32,
                     B->yt_rp, B->yt_col, B->yt_val, B->yt_val32, B->d, B->d32, &B->fwd_sched, &B->bwd_sched,
                     B->bar, B->nnzY, std::max(B->fwd_depth, B->bwd_depth)};
     return RW_OK;
@@ -510,7 +510,7 @@ rw_status pcg_batch_t(rw_context* ctx, rw_batch* B, const double* const* d_b, do
     // one iteration of Algorithm 1 for every system; every decision on the device
     auto iteration = [&]() -> rw_status {
         rw_status r2;
-        if ((r2 = spmv_launch<T>(ctx, N, B->a_rp, B->a_col, Aval, p, q, nrhs))) return r2;
+        if ((r2 = spmv_launch<T>(ctx, N, B->nnzA, B->a_rp, B->a_col, Aval, p, q, nrhs))) return r2;
         seg_dot<T, T>(nch, s, p, q, nrhs, B->chunk_row0, part);
         seg_scalars(wide, s, S, part, B->seg_chunk0, nmat, nrhs, kBOpAlpha, tol);
         RW_COUNT_LAUNCH();

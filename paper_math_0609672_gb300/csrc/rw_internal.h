@@ -347,7 +347,7 @@ rw_status csr_transpose(rw_context* ctx, const rw_csr* A, int32_t* rp, int32_t* 
 
 // y = A x (node-major, nrhs <= 16) for T = double or float.
 template <typename T>
-rw_status spmv_launch(rw_context* ctx, int32_t n, const int32_t* rp, const int32_t* col, const T* val,
+rw_status spmv_launch(rw_context* ctx, int32_t n, int64_t nnz, const int32_t* rp, const int32_t* col, const T* val,
                       const T* x, T* y, int nrhs);
 
 // Size and pointer checks of a matrix argument (RW_ERR_ARG / RW_ERR_NOT_RMATRIX).
@@ -357,6 +357,7 @@ rw_status check_csr(const rw_csr* A);
 // solve schedules (a single factor or a batch).
 struct TuneTarget {
     int32_t n;
+    int64_t nnz_a;
     const int32_t* a_rp;
     const int32_t* a_col;
     const double* a_val;

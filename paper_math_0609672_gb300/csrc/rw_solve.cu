@@ -20,9 +20,23 @@ namespace rw {
 constexpr int kDotParts = 1024;  // blocks of the dot-product producing kernels
 
 // ---------------------------------------------------------------------------
-// SpMV: y = A x for node-major vectors.  GS lanes per row, each lane keeps one
-// accumulator per right-hand side.  Optionally accumulates per-block partial
-// dot products x.y (per right-hand side) for the PCG step.
+// SpMV: y = A x for node-major vectors.  Optionally accumulates per-block
+// partial dot products x.y (per right-hand side) for the PCG step.
+//
+// A block takes rows_per_pass consecutive rows at a time: their entries are
+// one contiguous piece of the CSR arrays, copied to shared memory by all
+// threads (every column and value is read from memory once, coalesced); then a
+// group of G = NR * ES lanes per row sums it: lane (es, j) owns right-hand
+// side j and entries es, es + ES, ... .  What bounds it is the FP64 pipe (2
+// lane-FMAs per cycle and SM) and the gathers of x, one sector each, so a row
+// gets few lanes: a warp-wide FMA then carries entries of 32 / G rows, and
+// log2(ES) of the expensive FP64 additions across lanes serve them all.  With
+// 32 / NR lanes per row, rows loaded one dependent access after the other, a
+// call took 586 us on the 101 x 97 x 89 27-point grid with three right-hand
+// sides and 406 us with one; now 249 and 237 us (1.0e11 gathers/s).
+// Passes whose entries exceed the copy or that hold a row of more than
+// kLongRow entries per lane sum their rows with all 32 lanes each, straight
+// from memory.
 //
 // DIFF (the FP32 operator of the mixed mode): val holds A_ij (j != i) and, at
 // the diagonal position, the excess e_i = A_ii + sum_j A_ij, and the row is
@@ -31,52 +45,119 @@ constexpr int kDotParts = 1024;  // blocks of the dot-product producing kernels
 // so the operator keeps the near-null space of a weakly grounded matrix
 // (rounding A_ii itself would move a row sum by 2^-24 A_ii).
 // ---------------------------------------------------------------------------
+constexpr int kSpmvEntries = 2048;  // entries of a pass (24 KB of columns and FP64 values: eight blocks per SM)
+constexpr int kSpmvRows = 512;      // rows of a pass
+constexpr int kLongRow = 64;
+
 template <typename TA, typename TV, int NR, int ES, bool DIFF>
 __global__ void __launch_bounds__(256) k_spmv(int32_t n, const int32_t* __restrict__ rp,
                                               const int32_t* __restrict__ col,
                                               const TA* __restrict__ val, const TV* __restrict__ x,
-                                              TV* __restrict__ y, int nrhs, double* part) {
-    // a group of G = NR * ES lanes per row: lane (es, j) owns right-hand side j
-    // and entries s + es, s + es + ES, ... (one contiguous load of NR values per
-    // entry); the ES entry slices are summed across lanes
+                                              TV* __restrict__ y, int nrhs, int rows_per_pass, double* part) {
     constexpr int G = NR * ES;
-    constexpr int R = 32 / G;
     static_assert(G <= 32 && 32 % G == 0, "lane group");
-    __shared__ double sdot[8][R][NR];  // per (warp, row group, rhs): summed in a fixed order
-    const int lane = (int)lane_id();
-    const int gl = lane % G, j = gl % NR, es = gl / NR;
-    const unsigned gmask = G == 32 ? kFull : (((1u << G) - 1u) << (lane - gl));
-    const int64_t gid = (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * R + lane / G;
-    const int64_t ngroups = (((int64_t)gridDim.x * blockDim.x) >> 5) * R;
-    const bool jok = j < nrhs;
-    double mydot = 0.0;
-    for (int64_t row = gid; row < n; row += ngroups) {
-        const TV xi = (DIFF && jok) ? x[(size_t)row * nrhs + j] : TV(0);
-        TV acc = TV(0);
-        const int32_t s = rp[row], e = rp[row + 1];
-        for (int32_t p = s + es; p < e; p += ES) {
-            const int32_t c = col[p];
-            const TV a = (TV)val[p];
-            if (jok) {
-                if (DIFF) acc += (c == row) ? a * xi : a * (x[(size_t)c * nrhs + j] - xi);
-                else acc += a * x[(size_t)c * nrhs + j];
+    __shared__ __align__(16) TA sval[kSpmvEntries];
+    __shared__ int32_t scol[kSpmvEntries];
+    __shared__ int32_t srp[kSpmvRows + 1];
+    const int tid = (int)threadIdx.x, lane = (int)lane_id();
+    double mydot = 0.0, wdot = 0.0;
+    // lanes of right-hand side j, slice es of an ESX-lane row sum entries [s + es, e) of (c, a)
+    auto term = [&](int32_t c, TA av, int32_t row, int j, TV xi) -> TV {
+        const TV a = (TV)av;
+        const TV xc = x[(size_t)c * nrhs + j];
+        if (DIFF) return c == row ? a * xi : a * (xc - xi);
+        return a * xc;
+    };
+    const int64_t npass = ((int64_t)n + rows_per_pass - 1) / rows_per_pass;
+    for (int64_t ps = blockIdx.x; ps < npass; ps += gridDim.x) {
+        const int32_t base = (int32_t)(ps * rows_per_pass);
+        const int nr = min(rows_per_pass, n - base);
+        for (int i = tid; i <= nr; i += 256) srp[i] = rp[base + i];
+        __syncthreads();
+        int longest = 0;
+        for (int i = tid; i < nr; i += 256) longest = max(longest, srp[i + 1] - srp[i]);
+        const int32_t s0 = srp[0];
+        const int cnt = srp[nr] - s0;
+        const bool direct = __syncthreads_or(longest > kLongRow * ES || cnt > kSpmvEntries || cnt < 0);
+        if (!direct) {
+            for (int i = tid; i < cnt; i += 256) {
+                scol[i] = col[s0 + i];
+                sval[i] = val[s0 + i];
+            }
+            __syncthreads();
+            // one slice: nrhs lanes per row, no lane left over for a right-hand side past nrhs
+            const int lanes = ES == 1 ? nrhs : G, set = 256 / lanes, mine = tid / lanes;
+            const int j = ES == 1 ? tid - mine * lanes : tid % NR, es = ES == 1 ? 0 : (tid % G) / NR;
+            const bool jok = mine < set && j < nrhs;
+            for (int r0 = 0; r0 < nr; r0 += set) {
+                const int r = r0 + mine;
+                TV acc = TV(0);
+                if (r < nr && jok) {
+                    const int32_t row = base + r;
+                    const TV xi = DIFF ? x[(size_t)row * nrhs + j] : TV(0);
+                    const int e = srp[r + 1] - s0;
+                    for (int p = srp[r] - s0 + es; p < e; p += 4 * ES) {  // four gathers in flight
+                        TV t[4];
+                        int32_t c[4];
+#pragma unroll
+                        for (int u = 0; u < 4; ++u) {
+                            c[u] = p + u * ES < e ? scol[p + u * ES] : row;
+                            t[u] = x[(size_t)c[u] * nrhs + j];
+                        }
+#pragma unroll
+                        for (int u = 0; u < 4; ++u) {
+                            if (p + u * ES >= e) break;
+                            const TV a = (TV)sval[p + u * ES];
+                            if (DIFF) acc += c[u] == row ? a * xi : a * (t[u] - xi);
+                            else acc += a * t[u];
+                        }
+                    }
+                }
+                if constexpr (ES > 1) {
+#pragma unroll
+                    for (int o = NR; o < G; o <<= 1) acc += __shfl_xor_sync(kFull, acc, o);
+                }
+                if (r < nr && jok && es == 0) {
+                    const size_t at = (size_t)(base + r) * nrhs + j;
+                    y[at] = acc;
+                    if (part) mydot += (double)x[at] * (double)acc;
+                }
+            }
+        } else {
+            constexpr int EW = 32 / NR;
+            const int j = lane % NR, es = lane / NR;
+            const bool jok = j < nrhs;
+            for (int r = tid >> 5; r < nr; r += 8) {
+                const int32_t row = base + r;
+                const TV xi = (DIFF && jok) ? x[(size_t)row * nrhs + j] : TV(0);
+                TV acc = TV(0);
+                if (jok)
+                    for (int32_t p = srp[r] + es; p < srp[r + 1]; p += EW) acc += term(col[p], val[p], row, j, xi);
+#pragma unroll
+                for (int o = NR; o < 32; o <<= 1) acc += __shfl_xor_sync(kFull, acc, o);
+                if (es == 0 && jok) {
+                    const size_t at = (size_t)row * nrhs + j;
+                    y[at] = acc;
+                    if (part) wdot += (double)x[at] * (double)acc;
+                }
             }
         }
-#pragma unroll
-        for (int o = NR; o < G; o <<= 1) acc += __shfl_xor_sync(gmask, acc, o);
-        if (es == 0 && jok) {
-            y[(size_t)row * nrhs + j] = acc;
-            if (part) mydot += (double)x[(size_t)row * nrhs + j] * (double)acc;
-        }
+        __syncthreads();
     }
     if (part) {
-        if (es == 0) sdot[threadIdx.x >> 5][lane / G][j] = jok ? mydot : 0.0;
+        // per right-hand side, the threads that hold it in thread order: mydot in the copied passes, wdot
+        // (lanes l, l + NR, ... of a warp: right-hand side l % NR) in the others
+        static_assert(sizeof(sval) >= 512 * sizeof(double), "the copy's room holds the sums");
+        double* sdot = reinterpret_cast<double*>(sval);
+        sdot[tid] = mydot;
+        sdot[256 + tid] = wdot;
         __syncthreads();
-        if (threadIdx.x < NR) {
+        const int lanes = ES == 1 ? nrhs : NR;
+        if (tid < nrhs) {
             double t = 0.0;
-            for (int w = 0; w < (int)(blockDim.x >> 5); ++w)
-                for (int g = 0; g < R; ++g) t += sdot[w][g][threadIdx.x];
-            part[(size_t)blockIdx.x * 16 + threadIdx.x] = t;
+            for (int i = tid; i < 256; i += lanes) t += sdot[i];
+            for (int i = tid; i < 256; i += NR) t += sdot[256 + i];
+            part[(size_t)blockIdx.x * 16 + tid] = t;
         }
     }
 }
@@ -330,58 +411,83 @@ static int pow2_at_least(int v) {
 }
 
 template <typename TA, typename TV, int NR, int ES>
-static void launch_spmv_es(int32_t n, const int32_t* rp, const int32_t* col, const TA* val, const TV* x, TV* y,
-                           int nrhs, double* part, int blocks, cudaStream_t s) {
+static void launch_spmv_es(const rw_context* ctx, int32_t n, int64_t nnz, const int32_t* rp, const int32_t* col,
+                           const TA* val, const TV* x, TV* y, int nrhs, double* part, int* blocks_out, cudaStream_t s) {
     if constexpr (NR * ES <= 32) {
+        // rows of a pass: as many as the copy holds with a tenth to spare, in whole sets of row groups
+        const int set = 256 / (ES == 1 ? nrhs : NR * ES);
+        const double avg = n > 0 ? std::max(1.0, (double)nnz / (double)n) : 1.0;
+        int rows = std::max(1, std::min(kSpmvRows, (int)(0.9 * kSpmvEntries / avg)));
+        // (a small matrix: at least two passes per SM)
+        rows = std::max(std::min(rows, set), std::min(rows, n / (2 * ctx->num_sms)));
+        if (rows > set) rows -= rows % set;
+        const int64_t passes = ((int64_t)n + rows - 1) / rows;
+        static int per_sm = 0;
+        if (per_sm < 1) {
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_spmv<TA, TV, NR, ES, sizeof(TA) == 4>, 256, 0);
+            if (per_sm < 1) per_sm = 1;
+        }
+        int blocks = grid_for(passes, 1, ctx->num_sms * per_sm);
+        if (part && blocks > kDotParts) blocks = kDotParts;
+        if (blocks_out) *blocks_out = blocks;
         RW_COUNT_LAUNCH();
         // FP32 values are always the excess + difference form of the mixed mode
-        k_spmv<TA, TV, NR, ES, sizeof(TA) == 4><<<blocks, 256, 0, s>>>(n, rp, col, val, x, y, nrhs, part);
+        k_spmv<TA, TV, NR, ES, sizeof(TA) == 4><<<blocks, 256, 0, s>>>(n, rp, col, val, x, y, nrhs, rows, part);
     }
 }
 
+// Entry slices per row: the option, else one, doubled until the rows that the
+// block's threads hold at once fit the copy (27 entries a row and one
+// right-hand side: four slices; nine: one), and while the rows' lanes do not
+// fill the chip.
 template <typename TA, typename TV, int NR>
-static void launch_spmv_nr(const rw_context* ctx, int32_t n, const int32_t* rp, const int32_t* col,
-                           const TA* val, const TV* x, TV* y, int nrhs, double* part, cudaStream_t s) {
-    int es = ctx->opt.spmv_slices > 0 ? ctx->opt.spmv_slices : 32 / NR;
+static void launch_spmv_nr(const rw_context* ctx, int32_t n, int64_t nnz, const int32_t* rp, const int32_t* col,
+                           const TA* val, const TV* x, TV* y, int nrhs, double* part, int* blocks, cudaStream_t s) {
     int p = 1;
-    while (p * 2 <= es && p * 2 * NR <= 32) p *= 2;
-    const int rows_per_block = 8 * (32 / (NR * p));
-    const int blocks = part ? kDotParts : grid_for(((int64_t)n + rows_per_block - 1) / rows_per_block, 1,
-                                                   ctx->num_sms * 16);
+    if (ctx->opt.spmv_slices > 0) {
+        while (p * 2 <= ctx->opt.spmv_slices && p * 2 * NR <= 32) p *= 2;
+    } else {
+        const int64_t avg = n > 0 ? nnz / n : 0, lanes = (int64_t)ctx->num_sms * 1024;
+        while (p * 2 * NR <= 32 && (256 / (p == 1 ? nrhs : NR * p) * avg > kSpmvEntries * 3 / 2 ||
+                                    ((int64_t)n * NR * p < lanes && avg > 2 * p)))
+            p *= 2;
+    }
     switch (p) {
-        case 1: launch_spmv_es<TA, TV, NR, 1>(n, rp, col, val, x, y, nrhs, part, blocks, s); break;
-        case 2: launch_spmv_es<TA, TV, NR, 2>(n, rp, col, val, x, y, nrhs, part, blocks, s); break;
-        case 4: launch_spmv_es<TA, TV, NR, 4>(n, rp, col, val, x, y, nrhs, part, blocks, s); break;
-        case 8: launch_spmv_es<TA, TV, NR, 8>(n, rp, col, val, x, y, nrhs, part, blocks, s); break;
-        case 16: launch_spmv_es<TA, TV, NR, 16>(n, rp, col, val, x, y, nrhs, part, blocks, s); break;
-        default: launch_spmv_es<TA, TV, NR, 32>(n, rp, col, val, x, y, nrhs, part, blocks, s); break;
+        case 1: launch_spmv_es<TA, TV, NR, 1>(ctx, n, nnz, rp, col, val, x, y, nrhs, part, blocks, s); break;
+        case 2: launch_spmv_es<TA, TV, NR, 2>(ctx, n, nnz, rp, col, val, x, y, nrhs, part, blocks, s); break;
+        case 4: launch_spmv_es<TA, TV, NR, 4>(ctx, n, nnz, rp, col, val, x, y, nrhs, part, blocks, s); break;
+        case 8: launch_spmv_es<TA, TV, NR, 8>(ctx, n, nnz, rp, col, val, x, y, nrhs, part, blocks, s); break;
+        case 16: launch_spmv_es<TA, TV, NR, 16>(ctx, n, nnz, rp, col, val, x, y, nrhs, part, blocks, s); break;
+        default: launch_spmv_es<TA, TV, NR, 32>(ctx, n, nnz, rp, col, val, x, y, nrhs, part, blocks, s); break;
     }
 }
 
+// part: per-block dot products x.y of the right-hand sides ([blocks][16], at
+// most kDotParts blocks; *blocks receives their number).
 template <typename TA, typename TV>
-static rw_status launch_spmv(rw_context* ctx, int32_t n, const int32_t* rp, const int32_t* col,
-                             const TA* val, const TV* x, TV* y, int nrhs, double* part) {
+static rw_status launch_spmv(rw_context* ctx, int32_t n, int64_t nnz, const int32_t* rp, const int32_t* col,
+                             const TA* val, const TV* x, TV* y, int nrhs, double* part, int* blocks = nullptr) {
     cudaStream_t s = ctx->stream;
     const int nr = pow2_at_least(nrhs);
     switch (nr) {
-        case 1: launch_spmv_nr<TA, TV, 1>(ctx, n, rp, col, val, x, y, nrhs, part, s); break;
-        case 2: launch_spmv_nr<TA, TV, 2>(ctx, n, rp, col, val, x, y, nrhs, part, s); break;
-        case 4: launch_spmv_nr<TA, TV, 4>(ctx, n, rp, col, val, x, y, nrhs, part, s); break;
-        case 8: launch_spmv_nr<TA, TV, 8>(ctx, n, rp, col, val, x, y, nrhs, part, s); break;
-        default: launch_spmv_nr<TA, TV, 16>(ctx, n, rp, col, val, x, y, nrhs, part, s); break;
+        case 1: launch_spmv_nr<TA, TV, 1>(ctx, n, nnz, rp, col, val, x, y, nrhs, part, blocks, s); break;
+        case 2: launch_spmv_nr<TA, TV, 2>(ctx, n, nnz, rp, col, val, x, y, nrhs, part, blocks, s); break;
+        case 4: launch_spmv_nr<TA, TV, 4>(ctx, n, nnz, rp, col, val, x, y, nrhs, part, blocks, s); break;
+        case 8: launch_spmv_nr<TA, TV, 8>(ctx, n, nnz, rp, col, val, x, y, nrhs, part, blocks, s); break;
+        default: launch_spmv_nr<TA, TV, 16>(ctx, n, nnz, rp, col, val, x, y, nrhs, part, blocks, s); break;
     }
     return check_launch("spmv");
 }
 
 template <typename T>
-rw_status spmv_launch(rw_context* ctx, int32_t n, const int32_t* rp, const int32_t* col, const T* val,
+rw_status spmv_launch(rw_context* ctx, int32_t n, int64_t nnz, const int32_t* rp, const int32_t* col, const T* val,
                       const T* x, T* y, int nrhs) {
     NvtxRange nvtx_range("rw_spmv");
-    return launch_spmv<T, T>(ctx, n, rp, col, val, x, y, nrhs, nullptr);
+    return launch_spmv<T, T>(ctx, n, nnz, rp, col, val, x, y, nrhs, nullptr);
 }
-template rw_status spmv_launch<double>(rw_context*, int32_t, const int32_t*, const int32_t*, const double*,
+template rw_status spmv_launch<double>(rw_context*, int32_t, int64_t, const int32_t*, const int32_t*, const double*,
                                        const double*, double*, int);
-template rw_status spmv_launch<float>(rw_context*, int32_t, const int32_t*, const int32_t*, const float*,
+template rw_status spmv_launch<float>(rw_context*, int32_t, int64_t, const int32_t*, const int32_t*, const float*,
                                       const float*, float*, int);
 
 template <typename T>
@@ -447,7 +553,7 @@ void launch_to_fp32(const double* in, float* out, int64_t cnt, cudaStream_t s, i
 }
 
 rw_status spmv_fp64(rw_context* ctx, const rw_csr* A, const double* x, double* y, int nrhs) {
-    return launch_spmv<double, double>(ctx, A->n, A->row_ptr, A->col, A->val, x, y, nrhs, nullptr);
+    return launch_spmv<double, double>(ctx, A->n, A->nnz, A->row_ptr, A->col, A->val, x, y, nrhs, nullptr);
 }
 
 rw_status precond_fp64(rw_context* ctx, const FactorView& F, const double* r, double* z,
@@ -520,13 +626,14 @@ static rw_status pcg_t(rw_context* ctx, const rw_csr* A, const FactorView& F, co
     for (int it = 1; it <= max_iter && any_active; ++it) {
         done_iters = it;
         if (tm.on) cudaEventRecord(ctx->ev[2], s);
-        if ((rc = launch_spmv<T, T>(ctx, n, A->row_ptr, A->col, Aval, p, q, nrhs, part))) return rc;
+        int sb = 0;
+        if ((rc = launch_spmv<T, T>(ctx, n, A->nnz, A->row_ptr, A->col, Aval, p, q, nrhs, part, &sb))) return rc;
         if (tm.on) {
             cudaEventRecord(ctx->ev[3], s);
             tm.pending_spmv = true;
         }
         RW_COUNT_LAUNCH();
-        k_scalars<<<1, 256, 0, s>>>(S, part, kDotParts, nrhs, kOpAlpha, tol, it);
+        k_scalars<<<1, 256, 0, s>>>(S, part, sb, nrhs, kOpAlpha, tol, it);
         RW_COUNT_LAUNCH();
         k_update_xr<T><<<vb, 256, 0, s>>>(n, nrhs, S, x, r, p, q, w, z, part);
         if (mixed && it % refine == 0) {
@@ -711,7 +818,7 @@ rw_status bicgstab_run(rw_context* ctx, const rw_csr* A, const FactorView& F, co
         return r2 ? r2 : check_launch("bicgstab preconditioner");
     };
     auto spmv = [&](const double* in, double* out) -> rw_status {
-        return launch_spmv<double, double>(ctx, n, A->row_ptr, A->col, A->val, in, out, 1, nullptr);
+        return launch_spmv<double, double>(ctx, n, A->nnz, A->row_ptr, A->col, A->val, in, out, 1, nullptr);
     };
     cudaEventRecord(ctx->ev[8], s);
     double bb = 0.0;

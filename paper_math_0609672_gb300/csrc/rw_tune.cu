@@ -120,10 +120,10 @@ rw_status time_spmv(rw_context* ctx, const TuneTarget& X, const T* av, const T* 
                     float* ms) {
     cudaStream_t s = ctx->stream;
     rw_status rc;
-    if ((rc = spmv_launch<T>(ctx, X.n, X.a_rp, X.a_col, av, x, y, nrhs))) return rc;
+    if ((rc = spmv_launch<T>(ctx, X.n, X.nnz_a, X.a_rp, X.a_col, av, x, y, nrhs))) return rc;
     cudaEventRecord(ctx->ev[10], s);
     for (int i = 0; i < reps; ++i)
-        if ((rc = spmv_launch<T>(ctx, X.n, X.a_rp, X.a_col, av, x, y, nrhs))) return rc;
+        if ((rc = spmv_launch<T>(ctx, X.n, X.nnz_a, X.a_rp, X.a_col, av, x, y, nrhs))) return rc;
     cudaEventRecord(ctx->ev[11], s);
     if ((rc = check_cuda(cudaEventSynchronize(ctx->ev[11]), "sync"))) return rc;
     cudaEventElapsedTime(ms, ctx->ev[10], ctx->ev[11]);
@@ -220,7 +220,7 @@ rw_status tune_t(rw_context* ctx, const TuneTarget& X, int nrhs, const T* av, co
         }
     }
     if (X.a_rp) {
-        for (int es : slices) {
+        for (int es = 32 / nr; es >= 1; es /= 2) {
             ctx->opt.spmv_slices = es;
             float ms = 0.f;
             if ((rc = time_spmv<T>(ctx, X, av, r, z, nrhs, 5, &ms))) {
