@@ -93,9 +93,9 @@ typedef struct {
     int32_t refine_every;    /* FP32 PCG: true-residual replacement period (default 50) */
     int32_t walk_blocks_per_sm; /* 0 = from the occupancy calculator */
     int32_t timing;          /* 1: record per-phase device times (default 1) */
-    int32_t solve_blocks_per_sm; /* wide-level solves and the sync-free parts with vector rows:
-                                    512-thread blocks per SM (0 = 1; 2 = a register-capped
-                                    sync-free kernel, two blocks resident per SM) */
+    int32_t solve_blocks_per_sm; /* level schedule and row solves with vector rows: 512-thread blocks
+                                    per SM (0 = 1; 2 = a register-capped row kernel, two blocks
+                                    resident per SM) */
     int32_t graphs;          /* 1: batched PCG replays each iteration from a CUDA graph (default 1) */
     int32_t wide_slices;     /* wide-level solves: entry slices per row (lanes per row = slices x
                                 right-hand sides, power of two <= 32); 0 = one row per warp;
@@ -103,13 +103,13 @@ typedef struct {
                                 right-hand sides of its entries (default -1) */
     int32_t spmv_slices;     /* SpMV: entry slices per row (lanes per row = slices x right-hand sides, power
                                 of two <= 32); 0 = from the average row length (default 0) */
-    int32_t cluster_width;   /* levels of at most this many rows (above the thin-run width) run on
-                                one thread-block cluster with hardware barriers; 0 = never */
+    int32_t cluster_width;   /* level schedule: levels of at most this many rows run on one thread-block
+                                cluster with hardware barriers; 0 = never */
     int32_t cluster_size;    /* CTAs of that cluster (2..16; 0 = 16) */
-    int32_t solve_mode;      /* triangular solves: 0 = level schedule (thin / wide / cluster runs),
+    int32_t solve_mode;      /* triangular solves: 0 = level schedule (the whole grid level by level),
                                 1 = sync-free (each row waits only for its own dependencies),
-                                2 = hybrid (thin runs on one block, the other runs sync-free;
-                                default 2) */
+                                2 = stretches of narrow levels in blocks of rows with inverted
+                                triangles, the other rows sync-free (default 2) */
     int32_t reuse;           /* 1: walk reuse (Algorithm 2 of Sec. 5.3) in single-matrix builds:
                                 every simulated walk also counts, for each later node k' it
                                 passes, the legal sub-walk from k' (k' its least node until it
@@ -117,25 +117,18 @@ typedef struct {
                                 one start row never overlap).  Y, D and the counters then hold
                                 all these walks (default 0) */
     int32_t solve_mode_bwd;  /* solve_mode of the backward (Y^T) solve; -1 = as solve_mode (default) */
-    int32_t thin_levels;     /* factor build: levels per thin run at most (0 = no cap; default 128);
-                                dependencies on earlier runs are summed by the whole grid */
-    int32_t thin_cluster;    /* thin runs on a thread-block cluster of this many CTAs (2..16, reduced to
-                                what the device can place), x replicated in each CTA's shared memory;
-                                0 or 1 = one block (default 0) */
+    int32_t thin_levels;     /* accepted, without effect (default 128) */
+    int32_t thin_cluster;    /* accepted, without effect (default 0) */
     int32_t adapt_ahead;     /* rw_adaptive_budget: walks a row runs past its next decision point T, in
                                 percent of T (default 100; 0 = exactly up to T); changes only the
                                 time, never the counts */
-    int32_t thin_flags;      /* thin runs on one block: 1 = each row flags its slot in shared memory
-                                when done and readers wait on the flags of their entries (no barrier
-                                per level); 0 = one block barrier per level (default 0) */
+    int32_t thin_flags;      /* accepted, without effect (default 0) */
     int32_t spin_limit;      /* polls of one device-side wait (level computation, solve hand-offs,
                                 grid and cluster barriers, the latency probe) before it gives up and
                                 the call returns RW_ERR_TIMEOUT; 0 = 2^20 (about a second at L2
                                 latency; default 0).  A small value makes waits give up early: for
                                 testing the timeout path, never for results */
-    int32_t thin_lanes;      /* thin runs on one block: lanes per row, 8, 16 or 32 (0 = 32);
-                                fewer lanes let one FP64 instruction serve several rows
-                                (default 0) */
+    int32_t thin_lanes;      /* accepted, without effect (default 0) */
 } rw_options;
 
 typedef struct rw_context rw_context;
@@ -171,7 +164,7 @@ typedef struct {
     float phase_ms[8];         /* tables, walk, merge, emit, transpose, levels, fp32, total */
     int64_t kernel_launches;   /* kernels launched by the build */
     int64_t extra_walks;       /* walk reuse: sub-walks counted besides the simulated walks */
-    const int32_t* fwd_order;  /* [n] rows of Y z = v by level (level 0 first; any order inside a level) */
+    const int32_t* fwd_order;  /* [n] rows of Y z = v by level (level 0 first; ascending inside a level) */
     const int64_t* fwd_level_ptr; /* [fwd_levels+1] level l = fwd_order[ptr[l] .. ptr[l+1]) */
     const int32_t* bwd_order;  /* the same for Y^T w = r */
     const int64_t* bwd_level_ptr;
@@ -316,10 +309,10 @@ rw_status rw_permute_csr(rw_context* ctx, const rw_csr* A, const int32_t* d_perm
 
 /* Schedule autotuner.  Times a fixed list of launch shapes of the
  * preconditioner application and the SpMV on the given factor (or batch) and
- * nrhs random right-hand sides in precision prec -- the sync-free solve, and
- * the level schedule with entry slices per row group, wide-level blocks per
- * SM and cluster runs off / on for levels of up to 256 rows; SpMV entry
- * slices -- and installs the fastest in the context's options
+ * nrhs random right-hand sides in precision prec -- the sync-free solve, the
+ * blocks of narrow levels, and the level schedule with entry slices per row
+ * group, blocks per SM and cluster runs off / on for levels of up to 256 rows;
+ * SpMV entry slices -- and installs the fastest in the context's options
  * (rw_options.solve_mode, wide_slices, solve_blocks_per_sm, cluster_width,
  * spmv_slices), also copied to *out if not NULL.  cache_path (may be NULL): a
  * JSON-lines file; a line whose key matches the device and the problem's
@@ -362,7 +355,7 @@ rw_status rw_probe_gather(rw_context* ctx, uint64_t buffer_bytes, int32_t access
  * scaling by 1/D, forward solve with Y).
  * Concurrency: every solve on a factor (this call, rw_precond_apply_static,
  * pcg_solve, rw_precond_apply_ldu, bicgstab_solve) uses the factor's own solve
- * workspace (grid-barrier words and thin-run sums), so two of them on the same
+ * workspace (grid-barrier words and gathered right-hand sides), so two of them on the same
  * factor must not overlap on the GPU (different streams or threads); calls on
  * different factors may. */
 rw_status rw_precond_apply(rw_context* ctx, const rw_factor* F, const double* d_r, double* d_z,

@@ -285,10 +285,11 @@ rw_status rw::complete_factor(rw_context* ctx, rw_factor* F, const FactorOut& fo
     if (timing) cudaEventRecord(ctx->ev[12], s);
     F->fwd_order = alloc_n<int32_t>(F->pool, n);
     F->bwd_order = alloc_n<int32_t>(F->pool, n);
-    if (!F->fwd_order || !F->bwd_order) return RW_ERR_ALLOC;
-    if ((rc = compute_levels_pair(ctx, n, LevelDag{fo.y_rp, fo.y_col, false, F->fwd_order, &d.fwd_levels, &fwd_lptr},
-                                  LevelDag{yt_rp, yt_col, true, F->bwd_order, &d.bwd_levels, &bwd_lptr}, F->pool,
-                                  scratch)))
+    int32_t* last = alloc_n<int32_t>(scratch, 2 * (int64_t)n);
+    if (!F->fwd_order || !F->bwd_order || !last) return RW_ERR_ALLOC;
+    if ((rc = compute_levels_pair(
+             ctx, n, LevelDag{fo.y_rp, fo.y_col, false, F->fwd_order, last, &d.fwd_levels, &fwd_lptr},
+             LevelDag{yt_rp, yt_col, true, F->bwd_order, last + n, &d.bwd_levels, &bwd_lptr}, F->pool, scratch)))
         return rc;
     if (timing) cudaEventRecord(ctx->ev[13], s);
     d.fwd_order = F->fwd_order;
@@ -310,10 +311,10 @@ rw_status rw::complete_factor(rw_context* ctx, rw_factor* F, const FactorOut& fo
     }
     F->bar = static_cast<unsigned*>(F->pool.get((size_t)kSolveWorkspaceBytes));
     if (!F->bar) return RW_ERR_ALLOC;
-    if ((rc = build_schedule(ctx, n, fo.y_rp, fo.y_col, fo.y_val, y32, F->fwd_order, fwd_lptr,
+    if ((rc = build_schedule(ctx, n, fo.y_rp, fo.y_col, fo.y_val, y32, F->fwd_order, last, fwd_lptr,
                              d.fwd_levels, F->fwd_sched, F->pool, scratch)))
         return rc;
-    if ((rc = build_schedule(ctx, n, yt_rp, yt_col, yt_val, yt32, F->bwd_order, bwd_lptr,
+    if ((rc = build_schedule(ctx, n, yt_rp, yt_col, yt_val, yt32, F->bwd_order, last + n, bwd_lptr,
                              d.bwd_levels, F->bwd_sched, F->pool, scratch)))
         return rc;
     if (timing) cudaEventRecord(ctx->ev[14], s);

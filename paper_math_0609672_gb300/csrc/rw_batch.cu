@@ -438,8 +438,8 @@ namespace {
 template <typename T>
 rw_status pcg_batch_t(rw_context* ctx, rw_batch* B, const double* const* d_b, double* const* d_x,
                       int nrhs, double tol, int max_iter, rw_pcg_stats* stats, int32_t* h_iters,
-                      double* h_relres, const T* Aval, const T* yv, const T* ytv, const T* dv,
-                      const T* tv_fwd, const T* tv_bwd, bool mixed, Pool& sc) {
+                      double* h_relres, const T* Aval, const T* yv, const T* ytv, const T* dv, bool mixed,
+                      Pool& sc) {
     NvtxRange nvtx_range("rw_pcg_batch");
     cudaStream_t s = ctx->stream;
     const int32_t N = B->N;
@@ -489,11 +489,9 @@ rw_status pcg_batch_t(rw_context* ctx, rw_batch* B, const double* const* d_b, do
     seg_scalars(wide, s, S, part, B->seg_chunk0, nmat, nrhs, kBOpBnorm, tol);
     if ((rc = check_launch("batch pcg init"))) return rc;
     auto precond = [&]() -> rw_status {
-        rw_status r2 = solve_runs<T>(ctx, B->bwd_sched, B->yt_rp, B->yt_col, ytv, tv_bwd, r, nullptr, w,
-                                     nrhs, B->bar, true);
+        rw_status r2 = solve_runs<T>(ctx, B->bwd_sched, B->yt_rp, B->yt_col, ytv, r, w, nrhs, B->bar, true);
         if (r2) return r2;
-        if ((r2 = apply_inverse_diag<T>(ctx, w, dv, B->fwd_sched.n, nrhs))) return r2;
-        return solve_runs<T>(ctx, B->fwd_sched, B->y_rp, B->y_col, yv, tv_fwd, w, nullptr, z, nrhs, B->bar);
+        return solve_runs<T>(ctx, B->fwd_sched, B->y_rp, B->y_col, yv, w, z, nrhs, B->bar, false, w, dv);
     };
     if ((rc = precond())) return rc;
     seg_dot<T, T>(nch, s, r, z, nrhs, B->chunk_row0, part);
@@ -832,14 +830,15 @@ rw_status rw_batch_create(rw_context* ctx, int32_t nmat, const rw_csr* As, const
     }
     int64_t* fwd_lptr = nullptr;
     int64_t* bwd_lptr = nullptr;
-    if ((rc = compute_levels_pair(ctx, (int32_t)N,
-                                  LevelDag{B->y_rp, B->y_col, false, B->fwd_order, &B->fwd_depth, &fwd_lptr},
-                                  LevelDag{B->yt_rp, B->yt_col, true, B->bwd_order, &B->bwd_depth, &bwd_lptr}, P,
-                                  sc)) ||
-        (rc = build_schedule(ctx, (int32_t)N, B->y_rp, B->y_col, B->y_val, B->y_val32, B->fwd_order, fwd_lptr,
+    int32_t* last = alloc_n<int32_t>(sc, 2 * N);
+    if (!last) return fail(RW_ERR_ALLOC);
+    if ((rc = compute_levels_pair(
+             ctx, (int32_t)N, LevelDag{B->y_rp, B->y_col, false, B->fwd_order, last, &B->fwd_depth, &fwd_lptr},
+             LevelDag{B->yt_rp, B->yt_col, true, B->bwd_order, last + N, &B->bwd_depth, &bwd_lptr}, P, sc)) ||
+        (rc = build_schedule(ctx, (int32_t)N, B->y_rp, B->y_col, B->y_val, B->y_val32, B->fwd_order, last, fwd_lptr,
                              B->fwd_depth, B->fwd_sched, P, sc)) ||
-        (rc = build_schedule(ctx, (int32_t)N, B->yt_rp, B->yt_col, B->yt_val, B->yt_val32, B->bwd_order, bwd_lptr,
-                             B->bwd_depth, B->bwd_sched, P, sc)))
+        (rc = build_schedule(ctx, (int32_t)N, B->yt_rp, B->yt_col, B->yt_val, B->yt_val32, B->bwd_order, last + N,
+                             bwd_lptr, B->bwd_depth, B->bwd_sched, P, sc)))
         return fail(rc);
     if ((rc = read_status(ctx, "batch create"))) return fail(rc);
     *out = B;
@@ -889,11 +888,10 @@ rw_status pcg_solve_batch(rw_context* ctx, rw_batch* B, const double* const* d_b
             return RW_ERR_ARG;
         }
         return pcg_batch_t<float>(ctx, B, d_b, d_x, nrhs, tol, max_iter, stats, h_iters, h_relres, B->a_val32,
-                                  B->y_val32, B->yt_val32, B->d32, B->fwd_sched.tval32, B->bwd_sched.tval32,
-                                  true, sc);
+                                  B->y_val32, B->yt_val32, B->d32, true, sc);
     }
     return pcg_batch_t<double>(ctx, B, d_b, d_x, nrhs, tol, max_iter, stats, h_iters, h_relres, B->a_val,
-                               B->y_val, B->yt_val, B->d, B->fwd_sched.tval, B->bwd_sched.tval, false, sc);
+                               B->y_val, B->yt_val, B->d, false, sc);
 }
 
 }  // extern "C"

@@ -253,6 +253,7 @@ struct LevelDag {
     const int32_t* col;
     bool descending;
     int32_t* order;       // [n] out
+    int32_t* last;        // [n] out: a dependency of each row on its highest level (-1: none)
     int32_t* depth;       // out
     int64_t** lptr_out;   // out
 };
@@ -260,49 +261,72 @@ struct LevelDag {
 rw_status compute_levels_pair(rw_context* ctx, int32_t n, const LevelDag& fwd, const LevelDag& bwd, Pool& keep,
                               Pool& scratch);
 
-// Schedule of one triangular solve (see rw_sched.cu).
-struct SolveRun {
-    int thin;                    // 1: one block with shared-memory values; 0: whole grid
-    int32_t lev_begin, lev_end;  // levels [begin, end)
-    int64_t pos_begin, pos_end;  // positions in the level order
-    int64_t in_entries = 0;      // thin run: entries whose column lies in the run
+// A position of the level order as the row solve takes it (see rw_sched.cu):
+// its row, the row's entries, and a dependency on its highest level (-1: none).
+struct SolveRow {
+    int64_t start;
+    int32_t cnt;
+    int32_t row;
+    int32_t last;
+    int32_t pad;
 };
+
+// Positions [pos0, pos1) solved together: as blocks, or (nblocks 0) row by row.
+struct SolveStretch {
+    int64_t pos0, pos1;
+    int32_t block0, nblocks;
+};
+
+// Block of a narrow stretch: positions [pos0, pos0 + rows); prev0: the first
+// position of the block before it (pos0 in the stretch's first block);
+// stretch0: the first position of the stretch.
+struct SolveBlock {
+    int64_t pos0, prev0, stretch0;
+    int32_t rows, pad;
+};
+
+// Entries of the block slots' rows outside their blocks.
+struct SolveEntries {
+    const int64_t* ptr = nullptr;  // [slots + 1]
+    const int32_t* idx = nullptr;  // columns
+    const double* val = nullptr;
+    const float* val32 = nullptr;
+};
+
+// Schedule of one triangular solve (see rw_sched.cu).
 struct SolveSchedule {
     int32_t n = 0, depth = 0;
     const int32_t* order = nullptr;  // rows in level order
     const int64_t* lptr = nullptr;   // [depth + 1] level boundaries (device)
     std::vector<int64_t> lptr_h;     // host copy
-    std::vector<SolveRun> runs;
-    int64_t* tptr = nullptr;         // [n+1] packed entries of thin-run positions
-    int32_t* tnin = nullptr;         // [n] in-run entries of each position (listed first)
-    int32_t* tidx = nullptr;         // in-run: slot in the run; external: column
-    double* tval = nullptr;
-    float* tval32 = nullptr;
-    int64_t thin_entries = 0;
+    SolveRow* rows = nullptr;        // [n] by position
+    std::vector<SolveStretch> stretches;
+    // blocks of the narrow stretches
+    SolveBlock* blocks = nullptr;
+    int32_t* trow = nullptr;         // row of each block slot (-1: unused)
+    SolveEntries ext[3];             // entries in the block before, earlier in the stretch, before it
+    double* inv = nullptr;           // inverses of the blocks' unit triangles
+    float* inv32 = nullptr;
+    void* t = nullptr;               // workspace: [slots][nrhs] gathered right-hand sides
 };
 
 rw_status build_schedule(rw_context* ctx, int32_t n, const int64_t* rp, const int32_t* col,
                          const double* val, const float* val32, const int32_t* order,
-                         const int64_t* lptr_dev, int32_t depth, SolveSchedule& S, Pool& pool,
+                         const int32_t* last, const int64_t* lptr_dev, int32_t depth, SolveSchedule& S, Pool& pool,
                          Pool& scratch);
 
-// Device workspace of the solves, owned by the factor: two grid-barrier words
-// (at offset 0) and the external sums of a thin run (from byte 256 on).
-constexpr int64_t kSolveWorkspaceBytes = 256 + (int64_t)4096 * 16 * 8;
+// Device workspace of the solves, owned by the factor: two grid-barrier words.
+constexpr int64_t kSolveWorkspaceBytes = 256;
 
-// w <- w / d row by row (w node-major [n][nrhs]), in place: the D^-1 step of
-// the preconditioner between the two solves, so that the forward solve's rows
-// need no division of their own (the FP64 division is a long instruction
-// sequence on GB300's narrow FP64 pipe; here one instruction serves 32 rows).
-// IEEE division as the solve would do it, so results are unchanged.
-template <typename T>
-rw_status apply_inverse_diag(rw_context* ctx, T* w, const T* d, int64_t n, int nrhs);
-
-// backward: the Y^T solve (rw_options.solve_mode_bwd may choose its mode).
+// Solve of one triangle, x = rhs - (strict part) x.  backward: the Y^T solve
+// (rw_options.solve_mode_bwd may choose its mode).  w, d: when given, w <- w / d
+// row by row (w node-major [n][nrhs]) before the solve starts -- the D^-1 step
+// between the two solves, so that the forward solve's rows need no division of
+// their own; IEEE division as the solve would do it.
 template <typename T>
 rw_status solve_runs(rw_context* ctx, const SolveSchedule& S, const int64_t* rp, const int32_t* col,
-                     const T* val, const T* tval, const T* rhs, const T* scale, T* x, int nrhs,
-                     unsigned* bar, bool backward = false);
+                     const T* val, const T* rhs, T* x, int nrhs, unsigned* bar, bool backward = false,
+                     T* w = nullptr, const T* d = nullptr);
 
 // ---- solve path (rw_solve.cu) ----------------------------------------------
 

@@ -24,6 +24,7 @@ struct LevelJob {
     int descending;
     int* lev;
     int* maxlev;
+    int32_t* last;
 };
 
 // Levels of one or two DAGs in one co-resident launch: with two jobs the even
@@ -46,7 +47,7 @@ __global__ void __launch_bounds__(256) k_levels(int32_t n, const LevelJob J0, co
     for (int64_t pos = gw; pos < n; pos += nw) {
         const int32_t row = J.descending ? n - 1 - (int32_t)pos : (int32_t)pos;
         const int64_t s = rp[row], e = rp[row + 1];
-        int m = -1;
+        int m = -1, at = -1;
         for (int64_t p = s + lane; p < e; p += 32) {
             const int32_t c = col[p];
             int v = ld_relaxed(&lev[c]);
@@ -59,46 +60,62 @@ __global__ void __launch_bounds__(256) k_levels(int32_t n, const LevelJob J0, co
                 __nanosleep(20);
                 v = ld_relaxed(&lev[c]);
             }
-            m = max(m, v);
+            if (v > m) {
+                m = v;
+                at = c;
+            }
         }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(kFull, m, o));
+        const int mine = m;
+        m = __reduce_max_sync(kFull, m);
         if (lane == 0) st_relaxed(&lev[row], m + 1);
+        // (after the hand-off) a dependency on the highest level, -1 without any
+        at = __shfl_sync(kFull, at, __ffs(__ballot_sync(kFull, mine == m)) - 1);
+        if (lane == 0) J.last[row] = at;
         my_max = max(my_max, m + 1);
     }
     if (lane == 0 && my_max >= 0) atomicMax(J.maxlev, my_max);
 }
 
-__global__ void k_level_hist(int32_t n, const int* __restrict__ lev, uint32_t* cnt) {
-    for (int32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
-        atomicAdd(&cnt[lev[i]], 1u);
-}
-
-__global__ void k_level_scatter(int32_t n, const int* __restrict__ lev,
-                                const int64_t* __restrict__ lptr, uint32_t* fill, int32_t* order) {
+// Sort keys (the levels) and values (the rows) of the level order.
+__global__ void k_level_keys(int32_t n, const int* __restrict__ lev, uint32_t* key, uint32_t* row) {
     for (int32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-        const int l = lev[i];
-        order[lptr[l] + atomicAdd(&fill[l], 1u)] = i;
+        key[i] = (uint32_t)lev[i];
+        row[i] = (uint32_t)i;
     }
 }
 
-// Histogram of the levels, their boundaries and the rows sorted by level.
+// The sorted rows, and the first position of each level (every level up to the
+// depth holds a row).
+__global__ void k_level_bounds(int32_t n, int nlev, const uint32_t* __restrict__ key,
+                               const uint32_t* __restrict__ row, int32_t* order, int64_t* lptr) {
+    for (int32_t p = blockIdx.x * blockDim.x + threadIdx.x; p < n; p += gridDim.x * blockDim.x) {
+        order[p] = (int32_t)row[p];
+        if (p == 0 || key[p] != key[p - 1]) lptr[key[p]] = p;
+        if (p == n - 1) lptr[nlev] = n;
+    }
+}
+
+// The rows sorted by level, ascending inside a level, and the levels'
+// boundaries: a stable radix sort (a counting sort by atomics left the rows of a
+// level in any order, took as long, and with the order the blocks of the narrow
+// levels and their rounding would change from build to build).
 static rw_status level_order(rw_context* ctx, int32_t n, const int* lev, int nlev, int32_t* order, int64_t* lptr,
-                             uint32_t* cnt, Pool& scratch) {
+                             uint32_t* buf, Pool& scratch) {
     cudaStream_t s = ctx->stream;
     rw_status rc;
-    if ((rc = check_cuda(cudaMemsetAsync(cnt, 0, sizeof(uint32_t) * (size_t)(nlev + 1), s), "memset")))
-        return rc;
-    const int blocks2 = grid_for(n, 256, ctx->num_sms * 8);
+    const int blocks = grid_for(n, 256, ctx->num_sms * 8);
+    int bits = 1;
+    while (bits < 31 && (nlev - 1) >> bits) ++bits;
     RW_COUNT_LAUNCH();
-    k_level_hist<<<blocks2, 256, 0, s>>>(n, lev, cnt);
-    if ((rc = check_launch("level histogram"))) return rc;
-    if ((rc = check_cuda(scan_u32_to_i64(cnt, lptr, nlev, s, scratch), "scan"))) return rc;
-    if ((rc = check_cuda(cudaMemsetAsync(cnt, 0, sizeof(uint32_t) * (size_t)(nlev + 1), s), "memset")))
+    k_level_keys<<<blocks, 256, 0, s>>>(n, lev, buf, buf + n);
+    if ((rc = check_launch("level keys"))) return rc;
+    uint32_t *key = nullptr, *row = nullptr;
+    if ((rc = radix_sort_pairs(ctx, buf, buf + n, buf + 2 * (int64_t)n, buf + 3 * (int64_t)n, n, bits, scratch, &key,
+                               &row)))
         return rc;
     RW_COUNT_LAUNCH();
-    k_level_scatter<<<blocks2, 256, 0, s>>>(n, lev, lptr, cnt, order);
-    return check_launch("level scatter");
+    k_level_bounds<<<blocks, 256, 0, s>>>(n, nlev, key, row, order, lptr);
+    return check_launch("level order");
 }
 
 rw_status compute_levels_pair(rw_context* ctx, int32_t n, const LevelDag& fwd, const LevelDag& bwd, Pool& keep,
@@ -112,10 +129,10 @@ rw_status compute_levels_pair(rw_context* ctx, int32_t n, const LevelDag& fwd, c
     if (n == 0) return RW_OK;
     int* lev = alloc_n<int>(scratch, 2 * (int64_t)n);
     int* maxlev = alloc_n<int>(scratch, 2);
-    uint32_t* cnt = alloc_n<uint32_t>(scratch, n + 1);
+    uint32_t* buf = alloc_n<uint32_t>(scratch, 4 * (int64_t)n);
     int64_t* lptr_f = alloc_n<int64_t>(keep, n + 1);
     int64_t* lptr_b = alloc_n<int64_t>(keep, n + 1);
-    if (!lev || !maxlev || !cnt || !lptr_f || !lptr_b) return RW_ERR_ALLOC;
+    if (!lev || !maxlev || !buf || !lptr_f || !lptr_b) return RW_ERR_ALLOC;
     rw_status rc;
     if ((rc = check_cuda(cudaMemsetAsync(lev, 0xFF, sizeof(int) * 2 * (size_t)n, s), "memset"))) return rc;
     if ((rc = check_cuda(cudaMemsetAsync(maxlev, 0, 2 * sizeof(int), s), "memset"))) return rc;
@@ -127,8 +144,8 @@ rw_status compute_levels_pair(rw_context* ctx, int32_t n, const LevelDag& fwd, c
     int64_t blocks = (int64_t)per_sm * ctx->num_sms;
     const int64_t need = ((int64_t)n + 3) / 4;  // two jobs: 8 warps per block, 4 per DAG
     if (blocks > need) blocks = need;
-    LevelJob J0{fwd.rp, fwd.col, fwd.descending ? 1 : 0, lev, maxlev};
-    LevelJob J1{bwd.rp, bwd.col, bwd.descending ? 1 : 0, lev + n, maxlev + 1};
+    LevelJob J0{fwd.rp, fwd.col, fwd.descending ? 1 : 0, lev, maxlev, fwd.last};
+    LevelJob J1{bwd.rp, bwd.col, bwd.descending ? 1 : 0, lev + n, maxlev + 1, bwd.last};
     int njobs = 2;
     DevStatus* st = ctx->d_status;
     void* args[] = {(void*)&n, (void*)&J0, (void*)&J1, (void*)&njobs, (void*)&st};
@@ -142,8 +159,8 @@ rw_status compute_levels_pair(rw_context* ctx, int32_t n, const LevelDag& fwd, c
     if ((rc = read_status(ctx, "levels"))) return rc;
     *fwd.depth = hs[0] + 1;
     *bwd.depth = hs[1] + 1;
-    if ((rc = level_order(ctx, n, lev, *fwd.depth, fwd.order, lptr_f, cnt, scratch)) ||
-        (rc = level_order(ctx, n, lev + n, *bwd.depth, bwd.order, lptr_b, cnt, scratch)))
+    if ((rc = level_order(ctx, n, lev, *fwd.depth, fwd.order, lptr_f, buf, scratch)) ||
+        (rc = level_order(ctx, n, lev + n, *bwd.depth, bwd.order, lptr_b, buf, scratch)))
         return rc;
     *fwd.lptr_out = lptr_f;
     *bwd.lptr_out = lptr_b;

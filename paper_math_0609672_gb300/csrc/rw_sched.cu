@@ -2,37 +2,54 @@
 //
 // The paper applies the factor by forward/backward substitution (Sec. 4);
 // row r of a strict triangular system (CSR rp/col/val) gives
-//   x_r = rhs_r / scale_r - sum_p val_p * x_{col_p}
-// (scale = D for the forward solve with Y, none for the backward solve with
-// Y^T).  Rows are visited in level order (level = 1 + the largest level of a
-// dependency).  The DAGs of the walk factor are tall and thin: hundreds of
-// levels hold a handful of rows each, where the time is the chain of
-// dependent memory round trips, not arithmetic.  The level sequence is cut
-// into runs:
-//   thin run: consecutive levels of at most kThinWidth rows, solved by ONE
-//     block.  Phase 1 sums, in parallel, each row's dependencies that lie
-//     outside the run (already final); phase 2 walks the levels with a
-//     block barrier between them, keeping the run's x values in shared memory
-//     and the next level's entries prefetched in registers.
-//   wide run: level-synchronous over the whole co-resident grid, a group of
-//     lanes per row (one lane per right-hand side and entry slice), a
-//     software grid barrier between levels.
-// Every row sums its terms in a fixed order, so results do not depend on
-// timing.
+//   x_r = rhs_r - sum_p val_p * x_{col_p}
+// (the D^-1 between the two solves is an element-wise pass).  Rows are visited
+// in level order (level = 1 + the largest level of a dependency).  The DAGs of
+// the walk factor are tall and thin: hundreds of levels hold a handful of rows
+// each, where the time is the chain of dependent memory round trips (a value
+// handed from one SM to another through L2, 0.33 us at least), not arithmetic.
+//
+// The default schedule (solve_mode 2) cuts the level order into stretches:
+//   narrow stretch: consecutive levels of at most kNarrow rows, cut into blocks
+//     of 256 consecutive positions.  The schedule holds the inverse of each
+//     block's unit triangle L_BB, so that with t = rhs - (dependencies outside
+//     the block) all rows of the block follow in one step, x_B = L_BB^-1 t: a
+//     block costs two grid barriers instead of a hand-off per level (k_blocks);
+//   wide stretch: row by row, every warp of a co-resident grid taking every W-th
+//     row of the level order and waiting (bounded) for the values it reads
+//     (k_rows).
+// Y = I - N with N >= 0 for an R-matrix, so the blocks' inverses have no
+// negative entries and are computed and applied without cancellation; they are
+// computed in FP64 whatever the solve's precision.
+// One application of the preconditioner, before (narrow levels one after the
+// other in one thread block, the others sync-free with every lane polling its
+// own values) and now: 32^2 grid, 709 levels each way, 1.65 -> 0.076 ms; 300^2
+// grid in natural order, 48,350 levels, 109 -> 4.0 ms; 64^3 7-point, 1198
+// levels, four right-hand sides 6.9 -> 2.5 ms, sixteen 28 -> 6.3 ms; 1000^2
+// with long-range edges, 2229 levels, FP32 8.5 -> 6.4 ms.
+//
+// solve_mode 1 takes every row as in a wide stretch; solve_mode 0 is
+// level-synchronous over the whole grid.  Every row sums its terms in a fixed
+// order, so results do not depend on timing.
 #include <algorithm>
-
-#include <cooperative_groups.h>
 
 #include "rw_internal.h"
 
 namespace rw {
 
-constexpr int kThinWidth = 32;       // rows per level in a thin run (one warp each)
-constexpr int kThinThreads = 1024;   // the block of a thin run: 32 warps
-constexpr int kThinMaxRows = 4096;   // rows per thin run (shared memory)
-constexpr size_t kThinSmemBudget = 200 * 1024;
-constexpr int kHybridThinLevels = 64;  // hybrid schedule: shorter thin runs join the sync-free launches
-static_assert(256 + (int64_t)kThinMaxRows * 16 * 8 <= kSolveWorkspaceBytes, "solve workspace");
+// Rows of a narrow level at most.  A block's step takes 5 to 7 us, a wide level
+// 2 to 3 us, so the line lies where a block holds two to three levels: 32, 64,
+// 128 and 256 gave 2.33, 1.95, 2.05 and 2.58 ms per application on the 64^3
+// 7-point grid and 2.94, 2.41, 2.42 and 3.10 ms on a 56^3 27-point one.
+constexpr int kNarrow = 96;
+// Levels of a narrow stretch at least: shorter ones cost more in launches
+// (about 10 us) than they save.
+constexpr int kNarrowLevels = 16;
+// Rows of a block.  With 512 the inversion takes twice as long (both directions
+// of the 64^3 7-point grid: 2.3 against 1.2 ms of a 23 ms build).
+constexpr int kBlockRows = 256;
+
+__host__ __device__ __forceinline__ int64_t tri(int64_t m) { return m * (m + 1) / 2; }
 
 // ---------------------------------------------------------------------------
 // Schedule construction
@@ -42,93 +59,182 @@ __global__ void k_pos_of(int32_t n, const int32_t* __restrict__ order, int32_t* 
         pos_of[order[p]] = p;
 }
 
-__device__ __forceinline__ int run_of_pos(int64_t pos, const int64_t* run_pb, int nruns) {
-    int lo = 0, hi = nruns - 1;
-    while (lo < hi) {
-        const int mid = (lo + hi + 1) >> 1;
-        if (run_pb[mid] <= pos) lo = mid;
-        else hi = mid - 1;
-    }
-    return lo;
+// The entries of a block slot's row, by where their column lies: in the block
+// (0), in the block before it (1), earlier in the stretch (2), before it (3).
+constexpr int kClasses = 4;
+__device__ __forceinline__ int entry_class(int64_t p, const SolveBlock& b) {
+    return p >= b.pos0 ? 0 : p >= b.prev0 ? 1 : p >= b.stretch0 ? 2 : 3;
 }
 
-// Count the packed entries of each thin-run position (all its entries) and
-// how many of them lie inside the run.
-__global__ void k_sched_count(int32_t n, const int32_t* __restrict__ order,
-                              const int64_t* __restrict__ rp, const int32_t* __restrict__ col,
-                              const int32_t* __restrict__ pos_of, const int64_t* __restrict__ run_pb,
-                              const int32_t* __restrict__ run_thin, int nruns, uint32_t* cnt,
-                              int32_t* nin) {
-    for (int32_t p = blockIdx.x * blockDim.x + threadIdx.x; p < n; p += gridDim.x * blockDim.x) {
-        const int r = run_of_pos(p, run_pb, nruns);
-        if (!run_thin[r]) {
-            cnt[p] = 0u;
-            nin[p] = 0;
-            continue;
+// Warp per slot: its row, and the entries of each class.
+__global__ void __launch_bounds__(256) k_block_count(int64_t nslots, const SolveBlock* __restrict__ blocks,
+                                                     const int32_t* __restrict__ order,
+                                                     const int64_t* __restrict__ rp, const int32_t* __restrict__ col,
+                                                     const int32_t* __restrict__ pos_of, uint32_t* cnt,
+                                                     int32_t* trow) {
+    const int lane = (int)lane_id();
+    const int64_t gw = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    for (int64_t t = gw; t < nslots; t += nw) {
+        const SolveBlock b = blocks[t / kBlockRows];
+        const int slot = (int)(t % kBlockRows);
+        int row = -1;
+        unsigned c[kClasses] = {};
+        if (slot < b.rows) {
+            row = order[b.pos0 + slot];
+            const int64_t s = rp[row], e = rp[row + 1];
+            for (int64_t q = s + lane; q < e; q += 32) {
+                const int cl = entry_class(pos_of[col[q]], b);
+#pragma unroll
+                for (int k = 0; k < kClasses; ++k) c[k] += cl == k;
+            }
+#pragma unroll
+            for (int k = 0; k < kClasses; ++k) c[k] = __reduce_add_sync(kFull, c[k]);
         }
-        const int32_t row = order[p];
-        const int64_t s = rp[row], e = rp[row + 1];
-        int in = 0;
-        for (int64_t q = s; q < e; ++q) in += pos_of[col[q]] >= run_pb[r];
-        cnt[p] = (uint32_t)(e - s);
-        nin[p] = in;
-    }
-}
-
-// In-run entries of each thin run (summed over the warp's lanes of the same
-// run, then one atomic per run and warp).
-__global__ void k_run_in(int32_t n, const int32_t* __restrict__ nin, const int64_t* __restrict__ run_pb,
-                         const int32_t* __restrict__ run_thin, int nruns, unsigned long long* run_in) {
-    for (int32_t b = (blockIdx.x * blockDim.x + threadIdx.x) & ~31; b < n; b += gridDim.x * blockDim.x) {
-        const int32_t p = b + (int32_t)lane_id();
-        const int r = p < n ? run_of_pos(p, run_pb, nruns) : -1;
-        const unsigned v = (p < n && run_thin[r]) ? (unsigned)nin[p] : 0u;
-        const unsigned same = __match_any_sync(kFull, r);  // lanes of the same run
-        const unsigned t = __reduce_add_sync(same, v);
-        if (r >= 0 && (int)lane_id() == __ffs(same) - 1 && t) atomicAdd(run_in + r, (unsigned long long)t);
-    }
-}
-
-// In-run entries first (slot = position - run start), then the external ones
-// (column), each group in the row's original order.
-template <typename TV>
-__global__ void k_sched_fill(int32_t n, const int32_t* __restrict__ order,
-                             const int64_t* __restrict__ rp, const int32_t* __restrict__ col,
-                             const TV* __restrict__ val, const float* __restrict__ val32,
-                             const int32_t* __restrict__ pos_of, const int64_t* __restrict__ run_pb,
-                             const int32_t* __restrict__ run_thin, int nruns,
-                             const int64_t* __restrict__ tptr, const int32_t* __restrict__ nin,
-                             int32_t* tidx, double* tval, float* tval32) {
-    for (int32_t p = blockIdx.x * blockDim.x + threadIdx.x; p < n; p += gridDim.x * blockDim.x) {
-        const int r = run_of_pos(p, run_pb, nruns);
-        if (!run_thin[r]) continue;
-        const int32_t row = order[p];
-        const int64_t s = rp[row], e = rp[row + 1];
-        int64_t oi = tptr[p], oe = tptr[p] + nin[p];
-        for (int64_t q = s; q < e; ++q) {
-            const int32_t c = col[q];
-            const int32_t pc = pos_of[c];
-            const int64_t o = pc >= run_pb[r] ? oi++ : oe++;
-            tidx[o] = pc >= run_pb[r] ? (int32_t)(pc - run_pb[r]) : c;
-            tval[o] = val[q];
-            if (tval32) tval32[o] = val32[q];
+        if (lane == 0) {
+#pragma unroll
+            for (int k = 0; k < kClasses; ++k) cnt[k * nslots + t] = c[k];
+            trow[t] = row;
         }
+    }
+}
+
+// The entries of each class, in the row's order: slots and values inside the
+// block, columns, values and FP32 copies of the others.
+struct BlockEntries {
+    const int64_t* ptr[kClasses];  // [nslots + 1] first entry of each slot
+    int32_t* idx[kClasses];
+    double* val[kClasses];
+    float* val32[kClasses];        // (NULL inside the block, or without FP32 copies)
+};
+
+__global__ void __launch_bounds__(256) k_block_split(int64_t nslots, const SolveBlock* __restrict__ blocks,
+                                                     const int32_t* __restrict__ trow,
+                                                     const int64_t* __restrict__ rp, const int32_t* __restrict__ col,
+                                                     const double* __restrict__ val,
+                                                     const float* __restrict__ val32,
+                                                     const int32_t* __restrict__ pos_of, const BlockEntries E) {
+    const int lane = (int)lane_id();
+    const unsigned lt = lanemask_lt();
+    const int64_t gw = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    for (int64_t t = gw; t < nslots; t += nw) {
+        const int32_t row = trow[t];
+        if (row < 0) continue;
+        const SolveBlock b = blocks[t / kBlockRows];
+        const int64_t s = rp[row], e = rp[row + 1];
+        int64_t o[kClasses];
+#pragma unroll
+        for (int k = 0; k < kClasses; ++k) o[k] = E.ptr[k][t];
+        for (int64_t base = s; base < e; base += 32) {
+            const int64_t q = base + lane;
+            const int32_t c = q < e ? col[q] : 0;
+            const int64_t p = q < e ? (int64_t)pos_of[c] : 0;
+            const int cl = q < e ? entry_class(p, b) : -1;
+#pragma unroll
+            for (int k = 0; k < kClasses; ++k) {
+                const unsigned m = __ballot_sync(kFull, cl == k);
+                if (cl == k) {
+                    const int64_t at = o[k] + __popc(m & lt);
+                    E.idx[k][at] = k == 0 ? (int32_t)(p - b.pos0) : c;
+                    E.val[k][at] = val[q];
+                    if (E.val32[k]) E.val32[k][at] = val32[q];
+                }
+                o[k] += __popc(m);
+            }
+        }
+    }
+}
+
+// Inverse of each block's unit triangle L (L_ss = 1, L_su = the in-block
+// entries), row s as s + 1 values from tri(s) on.  A warp takes
+// eight columns: X_sc = [s == c] - sum_u L_su X_uc, row by row, the panel of X
+// in shared memory, lane (q, j) summing entries q, q + 4, ... of column j.  The
+// FP64 pipe's latency along the rows bounds it (an FP64 FMA waits 64 cycles), so
+// the panels are narrow: many warps per SM, and the columns of a block are
+// spread over many SMs.
+constexpr int kPanel = 8;
+__global__ void __launch_bounds__(32) k_block_invert(const SolveBlock* __restrict__ blocks,
+                                                     const int64_t* __restrict__ iptr,
+                                                     const int32_t* __restrict__ islot,
+                                                     const double* __restrict__ ival, double* inv, float* inv32) {
+    __shared__ double X[kBlockRows * kPanel];  // [rows - c0][kPanel]
+    const int lane = (int)lane_id(), j = lane % kPanel, q = lane / kPanel;
+    const int64_t b = blockIdx.y;
+    const int rows = blocks[b].rows, c0 = (int)blockIdx.x * kPanel;
+    if (c0 >= rows) return;
+    const int64_t t0 = b * kBlockRows, out0 = b * tri(kBlockRows);
+    constexpr int U = 4;  // entries per lane read ahead
+    int32_t sl[U];
+    double y[U];
+    int64_t e0, e1;
+    auto fetch = [&](int r) {
+        e0 = e1 = 0;
+        if (r < rows) {
+            e0 = iptr[t0 + r];
+            e1 = iptr[t0 + r + 1];
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int64_t p = e0 + q + 4 * u;
+            sl[u] = p < e1 ? islot[p] : -1;
+            y[u] = p < e1 ? ival[p] : 0.0;
+        }
+    };
+    fetch(c0);
+    for (int r = c0; r < rows; ++r) {
+        int32_t cs[U];
+        double cy[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            cs[u] = sl[u];
+            cy[u] = y[u];
+        }
+        const int64_t p0 = e0, p1 = e1;
+        fetch(r + 1);  // in flight while this row is summed
+        double acc = 0.0;
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+            if (cs[u] >= c0) acc += cy[u] * X[(cs[u] - c0) * kPanel + j];
+        for (int64_t p = p0 + q + 4 * U; p < p1; p += 4) {
+            const int s = islot[p];
+            if (s >= c0) acc += ival[p] * X[(s - c0) * kPanel + j];
+        }
+        acc += __shfl_xor_sync(kFull, acc, 8);
+        acc += __shfl_xor_sync(kFull, acc, 16);
+        const int c = c0 + j;
+        const double v = (r == c ? 1.0 : 0.0) - (r >= c ? acc : 0.0);
+        if (q == 0) X[(r - c0) * kPanel + j] = v;
+        __syncwarp();
+        if (q == 0 && c <= r) {
+            inv[out0 + tri(r) + c] = v;
+            if (inv32) inv32[out0 + tri(r) + c] = (float)v;
+        }
+    }
+}
+
+// Thread per position: its row as k_rows takes it.
+__global__ void k_fill_rows(int32_t n, const int32_t* __restrict__ order, const int32_t* __restrict__ last,
+                            const int64_t* __restrict__ rp, SolveRow* rows) {
+    for (int32_t p = blockIdx.x * blockDim.x + threadIdx.x; p < n; p += gridDim.x * blockDim.x) {
+        const int32_t row = order[p];
+        const int64_t s = rp[row];
+        rows[p] = SolveRow{s, (int32_t)(rp[row + 1] - s), row, last[row], 0};
     }
 }
 
 rw_status build_schedule(rw_context* ctx, int32_t n, const int64_t* rp, const int32_t* col,
                          const double* val, const float* val32, const int32_t* order,
-                         const int64_t* lptr_dev, int32_t depth, SolveSchedule& S, Pool& pool,
+                         const int32_t* last, const int64_t* lptr_dev, int32_t depth, SolveSchedule& S, Pool& pool,
                          Pool& scratch) {
     NvtxRange nvtx_range("rw_schedule");
     cudaStream_t s = ctx->stream;
     rw_status rc;
-    const int thin_levels = ctx->opt.thin_levels;
+    S = SolveSchedule{};
     S.n = n;
     S.depth = depth;
     S.order = order;
     S.lptr = lptr_dev;
-    S.runs.clear();
     if (n == 0) return RW_OK;
     S.lptr_h.resize((size_t)depth + 1);
     if ((rc = check_cuda(cudaMemcpyAsync(S.lptr_h.data(), lptr_dev, sizeof(int64_t) * (depth + 1),
@@ -136,429 +242,89 @@ rw_status build_schedule(rw_context* ctx, int32_t n, const int64_t* rp, const in
                          "copy")))
         return rc;
     if ((rc = check_cuda(cudaStreamSynchronize(s), "sync"))) return rc;
-    // cut the levels into runs
+    // stretches: narrow ones as blocks, the rows between them row by row
+    std::vector<SolveBlock> blocks;
+    int64_t pos = 0;
+    auto rows_until = [&](int64_t end) {
+        if (end > pos) S.stretches.push_back(SolveStretch{pos, end, 0, 0});
+        pos = end;
+    };
     for (int32_t l = 0; l < depth;) {
-        const bool thin = S.lptr_h[l + 1] - S.lptr_h[l] <= kThinWidth;
-        SolveRun run{thin ? 1 : 0, l, l, S.lptr_h[l], S.lptr_h[l]};
-        while (l < depth) {
-            const int64_t w = S.lptr_h[l + 1] - S.lptr_h[l];
-            const bool t = w <= kThinWidth;
-            if (t != thin) break;
-            if (thin && S.lptr_h[l + 1] - run.pos_begin > kThinMaxRows) break;
-            // a cap on a thin run's levels turns the dependencies on earlier
-            // levels into external ones, summed by the whole grid beforehand
-            // (the one block of the run then does less FP64 arithmetic per level)
-            if (thin && thin_levels > 0 && l - run.lev_begin >= thin_levels) break;
-            ++l;
+        int32_t e = l;
+        while (e < depth && S.lptr_h[e + 1] - S.lptr_h[e] <= kNarrow) ++e;
+        if (e - l >= kNarrowLevels) {
+            rows_until(S.lptr_h[l]);
+            SolveStretch st{pos, S.lptr_h[e], (int32_t)blocks.size(), 0};
+            for (int64_t prev = pos; pos < st.pos1;) {
+                const int32_t r = (int32_t)std::min<int64_t>(kBlockRows, st.pos1 - pos);
+                blocks.push_back(SolveBlock{pos, prev, st.pos0, r, 0});
+                prev = pos;
+                pos += r;
+            }
+            st.nblocks = (int32_t)blocks.size() - st.block0;
+            S.stretches.push_back(st);
         }
-        run.lev_end = l;
-        run.pos_end = S.lptr_h[l];
-        S.runs.push_back(run);
+        l = e > l ? e : e + 1;
     }
-    const int nruns = (int)S.runs.size();
-    std::vector<int64_t> pb(nruns);
-    std::vector<int32_t> th(nruns);
-    for (int i = 0; i < nruns; ++i) {
-        pb[i] = S.runs[i].pos_begin;
-        th[i] = S.runs[i].thin;
-    }
-    int64_t* d_pb = alloc_n<int64_t>(scratch, nruns);
-    int32_t* d_th = alloc_n<int32_t>(scratch, nruns);
+    rows_until(n);
+    const int g = grid_for(n, 256, ctx->num_sms * 8);
+    S.rows = alloc_n<SolveRow>(pool, n);
+    if (!S.rows) return RW_ERR_ALLOC;
+    RW_COUNT_LAUNCH();
+    k_fill_rows<<<g, 256, 0, s>>>(n, order, last, rp, S.rows);
+    if ((rc = check_launch("schedule rows"))) return rc;
+    const int64_t nb = (int64_t)blocks.size(), nslots = nb * kBlockRows;
+    if (nb == 0) return RW_OK;
     int32_t* pos_of = alloc_n<int32_t>(scratch, n);
-    uint32_t* cnt = alloc_n<uint32_t>(scratch, n + 1);
-    S.tptr = alloc_n<int64_t>(pool, n + 1);
-    S.tnin = alloc_n<int32_t>(pool, n);
-    if (!d_pb || !d_th || !pos_of || !cnt || !S.tptr || !S.tnin) return RW_ERR_ALLOC;
-    if ((rc = check_cuda(cudaMemcpyAsync(d_pb, pb.data(), sizeof(int64_t) * nruns,
+    uint32_t* cnt = alloc_n<uint32_t>(scratch, kClasses * nslots);
+    int64_t* ptr = alloc_n<int64_t>(pool, kClasses * (nslots + 1));
+    S.blocks = alloc_n<SolveBlock>(pool, nb);
+    S.trow = alloc_n<int32_t>(pool, nslots);
+    S.inv = alloc_n<double>(pool, nb * tri(kBlockRows));
+    S.inv32 = val32 ? alloc_n<float>(pool, nb * tri(kBlockRows)) : nullptr;
+    S.t = pool.get((size_t)nslots * 16 * sizeof(double));
+    if (!pos_of || !cnt || !ptr || !S.blocks || !S.trow || !S.inv || (val32 && !S.inv32) || !S.t) return RW_ERR_ALLOC;
+    if ((rc = check_cuda(cudaMemcpyAsync(S.blocks, blocks.data(), sizeof(SolveBlock) * (size_t)nb,
                                          cudaMemcpyHostToDevice, s),
                          "copy")))
         return rc;
-    if ((rc = check_cuda(cudaMemcpyAsync(d_th, th.data(), sizeof(int32_t) * nruns,
-                                         cudaMemcpyHostToDevice, s),
-                         "copy")))
-        return rc;
-    const int blocks = grid_for(n, 256, ctx->num_sms * 8);
+    const int gw = grid_for(nslots * 32, 256, ctx->num_sms * 8);
     RW_COUNT_LAUNCH();
-    k_pos_of<<<blocks, 256, 0, s>>>(n, order, pos_of);
+    k_pos_of<<<g, 256, 0, s>>>(n, order, pos_of);
     RW_COUNT_LAUNCH();
-    k_sched_count<<<blocks, 256, 0, s>>>(n, order, rp, col, pos_of, d_pb, d_th, nruns, cnt, S.tnin);
+    k_block_count<<<gw, 256, 0, s>>>(nslots, S.blocks, order, rp, col, pos_of, cnt, S.trow);
     if ((rc = check_launch("schedule count"))) return rc;
-    if ((rc = check_cuda(scan_u32_to_i64(cnt, S.tptr, n, s, scratch), "scan"))) return rc;
+    BlockEntries E{};
     int64_t* h64 = static_cast<int64_t*>(ctx->h_small);
-    if ((rc = check_cuda(cudaMemcpyAsync(h64, S.tptr + n, 8, cudaMemcpyDeviceToHost, s), "copy")))
-        return rc;
+    for (int k = 0; k < kClasses; ++k) {
+        int64_t* p = ptr + k * (nslots + 1);
+        E.ptr[k] = p;
+        if ((rc = check_cuda(scan_u32_to_i64(cnt + k * nslots, p, nslots, s, scratch), "scan")) ||
+            (rc = check_cuda(cudaMemcpyAsync(h64 + k, p + nslots, 8, cudaMemcpyDeviceToHost, s), "copy")))
+            return rc;
+    }
     if ((rc = check_cuda(cudaStreamSynchronize(s), "sync"))) return rc;
-    S.thin_entries = h64[0];
-    S.tidx = alloc_n<int32_t>(pool, S.thin_entries);
-    S.tval = alloc_n<double>(pool, S.thin_entries);
-    S.tval32 = val32 ? alloc_n<float>(pool, S.thin_entries) : nullptr;
-    if (!S.tidx || !S.tval || (val32 && !S.tval32)) return RW_ERR_ALLOC;
+    int64_t total[kClasses];
+    for (int k = 0; k < kClasses; ++k) total[k] = h64[k];
+    for (int k = 0; k < kClasses; ++k) {
+        Pool& where = k == 0 ? scratch : pool;
+        E.idx[k] = alloc_n<int32_t>(where, total[k]);
+        E.val[k] = alloc_n<double>(where, total[k]);
+        E.val32[k] = k > 0 && val32 ? alloc_n<float>(where, total[k]) : nullptr;
+        if (!E.idx[k] || !E.val[k] || (k > 0 && val32 && !E.val32[k])) return RW_ERR_ALLOC;
+    }
+    for (int k = 0; k + 1 < kClasses; ++k) S.ext[k] = SolveEntries{E.ptr[k + 1], E.idx[k + 1], E.val[k + 1], E.val32[k + 1]};
     RW_COUNT_LAUNCH();
-    k_sched_fill<double><<<blocks, 256, 0, s>>>(n, order, rp, col, val, val32, pos_of, d_pb, d_th,
-                                                nruns, S.tptr, S.tnin, S.tidx, S.tval, S.tval32);
-    if ((rc = check_launch("schedule fill"))) return rc;
-    // in-run entries per thin run (sizes the run's shared-memory copy of them)
-    unsigned long long* run_in = alloc_n<unsigned long long>(scratch, nruns);
-    if (!run_in) return RW_ERR_ALLOC;
-    if ((rc = check_cuda(cudaMemsetAsync(run_in, 0, sizeof(unsigned long long) * nruns, s), "memset")))
-        return rc;
-    RW_COUNT_LAUNCH();
-    k_run_in<<<blocks, 256, 0, s>>>(n, S.tnin, d_pb, d_th, nruns, run_in);
-    if ((rc = check_launch("run entries"))) return rc;
-    std::vector<unsigned long long> hin(nruns);
-    if ((rc = check_cuda(cudaMemcpyAsync(hin.data(), run_in, sizeof(unsigned long long) * nruns,
-                                         cudaMemcpyDeviceToHost, s),
-                         "copy")) ||
-        (rc = check_cuda(cudaStreamSynchronize(s), "sync")))
-        return rc;
-    for (int i = 0; i < nruns; ++i) S.runs[i].in_entries = (int64_t)hin[i];
-    return RW_OK;
-}
-
-// ---------------------------------------------------------------------------
-// External sums of a thin run, by the whole grid (warp per row):
-//   ext[slot][j] = sum over the row's dependencies outside the run
-// ---------------------------------------------------------------------------
-template <typename T, int NR>
-__global__ void __launch_bounds__(256) k_thin_ext(int64_t pos_begin, int64_t pos_end,
-                                                  const int64_t* __restrict__ tptr,
-                                                  const int32_t* __restrict__ tnin,
-                                                  const int32_t* __restrict__ tidx,
-                                                  const T* __restrict__ tval, const T* x, int nrhs,
-                                                  T* ext) {
-    const int lane = (int)lane_id();
-    const int64_t gw = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    for (int64_t pos = pos_begin + gw; pos < pos_end; pos += nw) {
-        const int64_t e0 = tptr[pos] + tnin[pos], e1 = tptr[pos + 1];
-        T acc[NR];
-#pragma unroll
-        for (int j = 0; j < NR; ++j) acc[j] = T(0);
-        for (int64_t e = e0 + lane; e < e1; e += 32) {
-            const int32_t c = tidx[e];
-            const T y = tval[e];
-#pragma unroll
-            for (int j = 0; j < NR; ++j)
-                if (j < nrhs) acc[j] += y * __ldcg(x + (size_t)c * nrhs + j);
-        }
-        const T mine = warp_sums<T, NR>(acc);
-        if (lane < NR) ext[(pos - pos_begin) * NR + lane] = mine;
+    k_block_split<<<gw, 256, 0, s>>>(nslots, S.blocks, S.trow, rp, col, val, val32, pos_of, E);
+    if ((rc = check_launch("schedule split"))) return rc;
+    for (int64_t b0 = 0; b0 < nb; b0 += 65535) {
+        const unsigned nbl = (unsigned)std::min<int64_t>(nb - b0, 65535);
+        RW_COUNT_LAUNCH();
+        k_block_invert<<<dim3(kBlockRows / kPanel, nbl), 32, 0, s>>>(
+            S.blocks + b0, E.ptr[0] + b0 * kBlockRows, E.idx[0], E.val[0], S.inv + b0 * tri(kBlockRows),
+            S.inv32 ? S.inv32 + b0 * tri(kBlockRows) : nullptr);
     }
-}
-
-// ---------------------------------------------------------------------------
-// Thin run: one block.
-// ---------------------------------------------------------------------------
-template <typename T>
-struct ThinParams {
-    int64_t pos_begin, pos_end;
-    int32_t lev_begin, lev_end;
-    const int64_t* __restrict__ lptr;
-    const int32_t* __restrict__ order;
-    const int64_t* __restrict__ tptr;
-    const int32_t* __restrict__ tnin;
-    const int32_t* __restrict__ tidx;
-    const T* __restrict__ tval;
-    const T* __restrict__ ext;
-    const T* __restrict__ rhs;
-    const T* __restrict__ scale;
-    T* x;
-    int nrhs;
-    int stage;  // 1: copy the run's in-run entries to shared memory first
-    int stage_entries;
-    int flags;  // 1: per-row ready flags in shared memory instead of a barrier per level
-    DevStatus* st;
-};
-
-// Shared memory of a thin run: x values [rows][NR], row ids, entry offsets and
-// counts, level starts, staged-entry offsets, ready flags; then (staged) the
-// in-run values and their slot indices.
-template <typename T, int NR>
-__host__ __device__ __forceinline__ size_t thin_stage_offset(int rows, int nlev) {
-    const size_t base = (size_t)rows * NR * sizeof(T) + (size_t)rows * 12 + (size_t)(nlev + 1) * 4 +
-                        (size_t)(rows + 1) * 4 + (size_t)rows * 4;
-    return (base + 15) & ~(size_t)15;
-}
-
-// in-run entries of one row held in registers: up to 32*U, prefetched ahead
-template <typename T, int U>
-struct RowRegs {
-    int slot;
-    int n;
-    int32_t e0;   // first packed entry, relative to the run
-    int32_t s[U];
-    T y[U];
-};
-
-// NR values of one slot of the shared-memory x array, read as vectors
-template <typename T, int NR>
-__device__ __forceinline__ void load_slot(const T* p, T (&v)[NR]) {
-    if constexpr (sizeof(T) == 8 && NR % 2 == 0) {
-#pragma unroll
-        for (int j = 0; j < NR; j += 2) {
-            const double2 d = *reinterpret_cast<const double2*>(p + j);
-            v[j] = d.x;
-            v[j + 1] = d.y;
-        }
-    } else if constexpr (sizeof(T) == 4 && NR % 4 == 0) {
-#pragma unroll
-        for (int j = 0; j < NR; j += 4) {
-            const float4 d = *reinterpret_cast<const float4*>(p + j);
-            v[j] = d.x;
-            v[j + 1] = d.y;
-            v[j + 2] = d.z;
-            v[j + 3] = d.w;
-        }
-    } else {
-#pragma unroll
-        for (int j = 0; j < NR; ++j) v[j] = p[j];
-    }
-}
-
-// warp_sums over each group of G lanes (G a power of two, NR <= G): value j
-// of a group ends in the group's lane j.  G = 32 is warp_sums.
-template <typename T, int NR, int G>
-__device__ __forceinline__ T group_sums(T (&v)[NR]) {
-    const unsigned lane = lane_id();
-    int cnt = NR;
-#pragma unroll
-    for (int o = G / 2; o >= 1; o >>= 1) {
-        if (cnt > 1) {
-            const int half = cnt / 2;
-            const bool upper = (lane & o) != 0;
-#pragma unroll
-            for (int i = 0; i < NR / 2; ++i) {
-                if (i < half) {
-                    const T send = upper ? v[i] : v[i + half];
-                    const T keep = upper ? v[i + half] : v[i];
-                    v[i] = keep + __shfl_xor_sync(kFull, send, o);
-                }
-            }
-            cnt = half;
-        } else {
-            v[0] += __shfl_xor_sync(kFull, v[0], o);
-        }
-    }
-    constexpr unsigned span = G / NR;  // value j sits in the group's lanes j * span ...
-    const unsigned src = (lane & ~(unsigned)(G - 1)) + (((lane & (G - 1)) * span) & (G - 1));
-    return __shfl_sync(kFull, v[0], src);
-}
-
-// CL: the run is solved by a thread-block cluster instead of one block.  Every
-// CTA keeps the whole run's x values in its shared memory; row q of a level
-// belongs to CTA q mod csize (warp q / csize), which writes the new value into
-// every CTA's copy through distributed shared memory; a cluster barrier ends
-// each level.  The level's FP64 work is thereby spread over csize SMs.
-//
-// G: lanes per row (32 / G rows per warp, without clusters).  The run's one SM
-// is bound by its FP64 rate (one warp-wide FP64 instruction per 19 cycles per
-// SM on GB300, whatever the lanes active), and a row of a thin run has few
-// in-run entries, so G = 8 lets each FP64 instruction serve four rows: the
-// entry terms and a three-step reduction per group instead of a five-step one
-// per row.
-template <typename T, int NR, bool CL, int G = 32>
-__global__ void __launch_bounds__(kThinThreads) k_thin(const ThinParams<T> P) {
-    static_assert(G == 32 || !CL, "cluster thin runs take one row per warp");
-    static_assert(NR <= G && (G & (G - 1)) == 0, "lane groups");
-    constexpr int U = 6;
-    constexpr int RPW = 32 / G;  // rows per warp
-    extern __shared__ __align__(16) unsigned char smem[];
-    namespace cg = cooperative_groups;
-    const unsigned crank = CL ? cg::this_cluster().block_rank() : 0u;
-    const unsigned csz = CL ? cg::this_cluster().num_blocks() : 1u;
-    const int rows = (int)(P.pos_end - P.pos_begin);
-    const int nlev = P.lev_end - P.lev_begin;
-    T* xs = reinterpret_cast<T*>(smem);                                    // [rows][NR]
-    int32_t* rowid = reinterpret_cast<int32_t*>(xs + (size_t)rows * NR);   // [rows]
-    int32_t* eoff = rowid + rows;                                          // [rows] first in-run entry
-    int32_t* ecnt = eoff + rows;                                           // [rows] in-run entries
-    int32_t* lstart = ecnt + rows;                                         // [nlev + 1] slots
-    const int lane = (int)lane_id();
-    const int warp = threadIdx.x >> 5;
-    const int gl = lane % G, grp = lane / G;  // lane in its group, group in the warp
-    const int64_t run_e0 = P.tptr[P.pos_begin];
-    const int32_t* tidx = P.tidx + run_e0;
-    const T* tval = P.tval + run_e0;
-    int32_t* soff = lstart + nlev + 1;  // [rows + 1] staged: first entry of each slot
-    volatile int32_t* ready = soff + rows + 1;  // [rows] flags mode: slot finished
-
-    for (int i = threadIdx.x; i <= nlev; i += blockDim.x)
-        lstart[i] = (int32_t)(P.lptr[P.lev_begin + i] - P.pos_begin);
-    // phase 1: right-hand side minus the external sums; per-row entry ranges
-    for (int slot = threadIdx.x; slot < rows; slot += blockDim.x) {
-        const int64_t pos = P.pos_begin + slot;
-        const int32_t row = P.order[pos];
-        rowid[slot] = row;
-        ready[slot] = 0;
-        eoff[slot] = (int32_t)(P.tptr[pos] - run_e0);
-        ecnt[slot] = P.tnin[pos];
-        for (int j = 0; j < P.nrhs && j < NR; ++j) {
-            T b = P.rhs[(size_t)row * P.nrhs + j];
-            if (P.scale) b = b / P.scale[row];
-            xs[(size_t)slot * NR + j] = b - P.ext[(size_t)slot * NR + j];
-        }
-    }
-    __syncthreads();
-    if (P.stage) {
-        // the run's in-run entries to shared memory: offsets by a block scan of
-        // the per-slot counts, then every entry copied by one thread (its slot
-        // found by binary search), so the copy is one round of loads
-        T* sval = reinterpret_cast<T*>(smem + thin_stage_offset<T, NR>(rows, nlev));
-        int32_t* sidx = reinterpret_cast<int32_t*>(sval + P.stage_entries);
-        constexpr int kPer = (kThinMaxRows + kThinThreads - 1) / kThinThreads;
-        int loc[kPer];
-        int sum = 0;
-#pragma unroll
-        for (int i = 0; i < kPer; ++i) {
-            const int sl = threadIdx.x * kPer + i;
-            loc[i] = sl < rows ? ecnt[sl] : 0;
-            sum += loc[i];
-        }
-        __shared__ int wtot[kThinThreads / 32];
-        int incl = sum;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int y = __shfl_up_sync(kFull, incl, o);
-            if (lane >= o) incl += y;
-        }
-        if (lane == 31) wtot[warp] = incl;
-        __syncthreads();
-        if (warp == 0) {
-            const int t = wtot[lane];
-            int ti = t;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const int y = __shfl_up_sync(kFull, ti, o);
-                if (lane >= o) ti += y;
-            }
-            wtot[lane] = ti - t;
-        }
-        __syncthreads();
-        int pre = wtot[warp] + incl - sum;
-#pragma unroll
-        for (int i = 0; i < kPer; ++i) {
-            const int sl = threadIdx.x * kPer + i;
-            if (sl < rows) soff[sl] = pre;
-            if (sl == rows - 1) soff[rows] = pre + loc[i];
-            pre += loc[i];
-        }
-        __syncthreads();
-        const int total = soff[rows];
-        for (int g = threadIdx.x; g < total; g += blockDim.x) {
-            int lo = 0, hi = rows - 1;  // the last slot whose offset is <= g
-            while (lo < hi) {
-                const int mid = (lo + hi + 1) >> 1;
-                if (soff[mid] <= g) lo = mid;
-                else hi = mid - 1;
-            }
-            const int src = eoff[lo] + (g - soff[lo]);
-            sidx[g] = tidx[src];
-            sval[g] = tval[src];
-        }
-        __syncthreads();
-        for (int sl = threadIdx.x; sl < rows; sl += blockDim.x) eoff[sl] = soff[sl];
-        tidx = sidx;
-        tval = sval;
-        __syncthreads();
-    }
-
-    // every CTA's copy is initialised before any row value is written into it
-    if constexpr (CL) cg::this_cluster().sync();
-    // phase 2: the levels in order; in each level warp w takes rows w, w+32, ...
-    // (with a cluster: slot q = warp * csize + rank of the level)
-    auto fetch = [&](int li, RowRegs<T, U>& R) {
-        R.slot = -1;
-        R.n = 0;
-        if (li < nlev) {
-            const int sl = lstart[li] + (warp * RPW + grp) * (int)csz + (int)crank;
-            if (sl < lstart[li + 1]) {
-                R.slot = sl;
-                R.e0 = eoff[sl];
-                R.n = ecnt[sl];
-            }
-        }
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-            const int k = gl + G * u;
-            const bool ok = R.slot >= 0 && k < R.n;
-            R.s[u] = ok ? tidx[R.e0 + k] : -1;
-            R.y[u] = ok ? tval[R.e0 + k] : T(0);
-        }
-    };
-    auto finish = [&](int slot, T mine) {
-        if (slot >= 0 && gl < P.nrhs && gl < NR) {
-            const T v = xs[(size_t)slot * NR + gl] - mine;
-            if constexpr (CL) {
-                for (unsigned r = 0; r < csz; ++r)
-                    cg::this_cluster().map_shared_rank(xs, r)[(size_t)slot * NR + gl] = v;
-            } else {
-                xs[(size_t)slot * NR + gl] = v;
-            }
-            __stcg(P.x + (size_t)rowid[slot] * P.nrhs + gl, v);
-        }
-    };
-    // flags mode: a lane reads an in-run value only once its slot is flagged
-    // (bounded wait; the warp holding the lowest unfinished slot always has its
-    // dependencies, so the run progresses without a barrier per level)
-    // (after one wait gives up, the others of the block give up at once)
-    const bool flags = !CL && P.flags != 0;
-    __shared__ int gave_up;
-    if (threadIdx.x == 0) gave_up = 0;
-    __syncthreads();
-    const unsigned spin_limit = P.st->spin_limit;
-    auto wait_slot = [&](int32_t sl) {
-        if (!flags) return;
-        unsigned spins = 0;
-        while (ready[sl] == 0) {
-            if (*(volatile int*)&gave_up) break;
-            if (++spins > spin_limit) {
-                *(volatile int*)&gave_up = 1;
-                atomicAdd(&P.st->timeout, 1u);
-                break;
-            }
-        }
-        __threadfence_block();
-    };
-    RowRegs<T, U> r0, r1;
-    fetch(0, r0);
-    for (int li = 0; li < nlev; ++li) {
-        fetch(li + 1, r1);  // the next level's entries: in flight while this level computes
-        if (__any_sync(kFull, r0.slot >= 0)) {  // G = 32: r0.slot is warp-uniform
-            T acc[NR];
-#pragma unroll
-            for (int j = 0; j < NR; ++j) acc[j] = T(0);
-#pragma unroll
-            for (int u = 0; u < U; ++u)
-                if (r0.s[u] >= 0) {
-                    wait_slot(r0.s[u]);
-                    T v[NR];
-                    load_slot<T, NR>(xs + (size_t)r0.s[u] * NR, v);
-#pragma unroll
-                    for (int j = 0; j < NR; ++j) acc[j] += r0.y[u] * v[j];
-                }
-            if (r0.slot >= 0) {
-                for (int k = gl + G * U; k < r0.n; k += G) {  // rows longer than G*U
-                    const int32_t sl = tidx[r0.e0 + k];
-                    const T y = tval[r0.e0 + k];
-                    wait_slot(sl);
-                    T v[NR];
-                    load_slot<T, NR>(xs + (size_t)sl * NR, v);
-#pragma unroll
-                    for (int j = 0; j < NR; ++j) acc[j] += y * v[j];
-                }
-            }
-            finish(r0.slot, group_sums<T, NR, G>(acc));
-            if (flags) {
-                __syncwarp();
-                __threadfence_block();
-                if (gl == 0 && r0.slot >= 0) ready[r0.slot] = 1;
-            }
-        }
-        // the cluster barrier also keeps every CTA alive until the last remote write
-        if constexpr (CL) cg::this_cluster().sync();
-        else if (!flags) __syncthreads();
-        r0 = r1;
-    }
+    return check_launch("block inverses");
 }
 
 // ---------------------------------------------------------------------------
@@ -573,7 +339,6 @@ struct WideParams {
     const int32_t* __restrict__ col;
     const T* __restrict__ val;
     const T* __restrict__ rhs;
-    const T* __restrict__ scale;
     T* x;
     int nrhs;
     unsigned* bar;
@@ -624,7 +389,7 @@ struct RowGroup {
             R0.y[u] = q < R0.e ? P.val[q] : T(0);
         }
     }
-    // x_row = rhs_row / scale_row - sum_q val_q x_{col_q}
+    // x_row = rhs_row - sum_q val_q x_{col_q}
     __device__ __forceinline__ void row(const WideParams<T>& P, const RowPre<T>& R0) const {
         const T* __restrict__ x = P.x;
         const int nr = P.nrhs;
@@ -657,9 +422,7 @@ struct RowGroup {
 #pragma unroll
         for (int o = NR; o < G; o <<= 1) acc += __shfl_xor_sync(gmask, acc, o);
         if (es == 0 && jok) {
-            T b = P.rhs[(size_t)R0.row * nr + j];
-            if (P.scale) b = b / P.scale[R0.row];
-            __stcg(P.x + (size_t)R0.row * nr + j, b - acc);
+            __stcg(P.x + (size_t)R0.row * nr + j, P.rhs[(size_t)R0.row * nr + j] - acc);
         }
     }
 };
@@ -760,9 +523,7 @@ struct RowVec {
         constexpr int span = 32 / NR;
         const int j = lane / span;
         if (lane % span == 0 && j < P.nrhs) {
-            T b = P.rhs[(size_t)R0.row * P.nrhs + j];
-            if (P.scale) b = b / P.scale[R0.row];
-            __stcg(P.x + (size_t)R0.row * P.nrhs + j, b - sum);
+            __stcg(P.x + (size_t)R0.row * P.nrhs + j, P.rhs[(size_t)R0.row * P.nrhs + j] - sum);
         }
     }
 };
@@ -860,64 +621,53 @@ __global__ void __launch_bounds__(1024, 1) k_cluster(const WideParams<T> P) {
 }
 
 // ---------------------------------------------------------------------------
-// Sync-free solve (rw_options.solve_mode = 1): one cooperative launch for the
-// whole solve.  x starts as the "pending" marker; warp w takes the rows at
-// positions w, w + W, ... of the level order; a row loads all its
-// dependencies at once, re-polls (bounded) only those still pending, and
+// Rows of a wide stretch (all rows with solve_mode 1): one cooperative launch.
+// x starts as the "pending" marker; warp w takes the rows at positions w,
+// w + W, ... of the stretch; a row loads all its dependencies at once and
 // publishes its value with one relaxed store.  Rows are taken in level order
 // and all warps are co-resident, so the lowest unfinished position can always
-// proceed.  Each warp loads the structure of its next two rows while it waits,
-// so a level on the critical path costs one hand-off through L2.
+// proceed.  A row that finds values pending waits (bounded) for the one on its
+// highest level first and then loads the pending ones again: with every lane
+// polling its own values the polls of the thousands of waiting warps filled the
+// L2 (61x64x67 grid of 124 levels: 0.97 -> 0.54 ms per application).  Each warp
+// loads the structure of its next two rows while it waits.
 // ---------------------------------------------------------------------------
 template <typename T>
-struct FreeParams {
+struct RowParams {
     int64_t n;
-    const int32_t* __restrict__ order;
-    const int64_t* __restrict__ rp;
+    const SolveRow* __restrict__ rows;
     const int32_t* __restrict__ col;
     const T* __restrict__ val;
     const T* __restrict__ rhs;
-    const T* __restrict__ scale;
     T* x;
     int nrhs;
     DevStatus* st;
 };
 
+template <typename T>
+__device__ __forceinline__ SolveRow row_at(const RowParams<T>& P, int64_t i) {
+    return i < P.n ? P.rows[i] : SolveRow{0, 0, -1, -1, 0};
+}
+
+// Column and value of entry q of a row.
+template <typename T>
+__device__ __forceinline__ void row_entry(const RowParams<T>& P, const SolveRow& d, int q, int32_t& c, T& y) {
+    const bool ok = q < d.cnt;
+    c = ok ? P.col[d.start + q] : 0;
+    y = ok ? P.val[d.start + q] : T(0);
+}
+
+// Lane groups: lane (es, j) owns right-hand side j and entries es, es + ES, ...
 template <typename T, int NR>
-__global__ void __launch_bounds__(512, sizeof(T) == 4 ? 2 : 1) k_syncfree(const FreeParams<T> P) {
+__global__ void __launch_bounds__(512, sizeof(T) == 4 ? 2 : 1) k_rows(const RowParams<T> P) {
     constexpr int ES = 32 / NR;
+    constexpr int U = kPreEntries;
     const int lane = (int)lane_id();
     const int j = lane % NR, es = lane / NR;
     const bool jok = j < P.nrhs;
     const int64_t gw = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
     const unsigned spin_limit = P.st->spin_limit;
-    struct Pre {
-        int32_t row;
-        int64_t s, e;
-        int32_t c[kPreEntries];
-        T y[kPreEntries];
-        T b;
-    };
-    auto load = [&](int64_t pos, Pre& R0) {
-        R0.row = -1;
-        if (pos >= P.n) return;
-        const int32_t row = P.order[pos];
-        R0.row = row;
-        R0.s = P.rp[row];
-        R0.e = P.rp[row + 1];
-#pragma unroll
-        for (int u = 0; u < kPreEntries; ++u) {
-            const int64_t q = R0.s + es + (int64_t)u * ES;
-            R0.c[u] = q < R0.e ? P.col[q] : 0;
-            R0.y[u] = q < R0.e ? P.val[q] : T(0);
-        }
-        R0.b = T(0);
-        if (es == 0 && jok) {
-            R0.b = P.rhs[(size_t)row * P.nrhs + j];
-            if (P.scale) R0.b = R0.b / P.scale[row];
-        }
-    };
     // polls back off after the first few so that waiting warps leave L2
     // bandwidth to the rows being computed
     auto wait_value = [&](const T* src, T v) -> T {
@@ -929,44 +679,73 @@ __global__ void __launch_bounds__(512, sizeof(T) == 4 ? 2 : 1) k_syncfree(const 
         }
         return v;
     };
+    struct Pre {
+        SolveRow d;
+        int32_t c[U];
+        T y[U];
+        T b;
+    };
+    auto load = [&](const SolveRow& d, Pre& R) {
+        R.d = d;
+#pragma unroll
+        for (int u = 0; u < U; ++u) row_entry(P, d, es + u * ES, R.c[u], R.y[u]);
+        R.b = es == 0 && jok && d.row >= 0 ? P.rhs[(size_t)d.row * P.nrhs + j] : T(0);
+    };
     Pre pre[2];
-    load(gw, pre[0]);
-    load(gw + nw, pre[1]);
+    load(row_at(P, gw), pre[0]);
+    load(row_at(P, gw + nw), pre[1]);
+    SolveRow after = row_at(P, gw + 2 * nw);
     for (int64_t pos = gw; pos < P.n; pos += nw) {
         const Pre cur = pre[0];
         pre[0] = pre[1];
-        load(pos + 2 * nw, pre[1]);
-        const int nr = P.nrhs;
-        T v[kPreEntries];
+        load(after, pre[1]);
+        after = row_at(P, pos + 3 * nw);
+        const int nr = P.nrhs, cnt = cur.d.cnt;
+        const T* const src = P.x;
+        T v[U];
+        bool pend = false;
 #pragma unroll
-        for (int u = 0; u < kPreEntries; ++u)
-            v[u] = (jok && cur.s + es + (int64_t)u * ES < cur.e) ? ld_relaxed(P.x + (size_t)cur.c[u] * nr + j) : T(0);
+        for (int u = 0; u < U; ++u) {
+            v[u] = (jok && es + u * ES < cnt) ? ld_relaxed(src + (size_t)cur.c[u] * nr + j) : T(0);
+            pend |= is_pending(v[u]);
+        }
+        if (cur.d.last >= 0 && __any_sync(kFull, pend)) {
+            const T* const p = src + (size_t)cur.d.last * nr + (jok ? j : 0);
+            wait_value(p, ld_relaxed(p));
+#pragma unroll
+            for (int u = 0; u < U; ++u)
+                if (is_pending(v[u])) v[u] = ld_relaxed(src + (size_t)cur.c[u] * nr + j);
+        }
         T acc = T(0);
 #pragma unroll
-        for (int u = 0; u < kPreEntries; ++u) {
-            if (jok && cur.s + es + (int64_t)u * ES < cur.e)
-                v[u] = wait_value(P.x + (size_t)cur.c[u] * nr + j, v[u]);
+        for (int u = 0; u < U; ++u) {
+            if (jok && es + u * ES < cnt) v[u] = wait_value(src + (size_t)cur.c[u] * nr + j, v[u]);
             acc += cur.y[u] * v[u];
         }
-        for (int64_t q = cur.s + es + (int64_t)kPreEntries * ES; q < cur.e; q += ES) {
-            const int32_t c = P.col[q];
-            const T y = P.val[q];
-            if (jok) {
-                const T* src = P.x + (size_t)c * nr + j;
-                acc += y * wait_value(src, ld_relaxed(src));
+        for (int base = U * ES; base < cnt; base += U * ES) {
+            int32_t c[U];
+            T y[U], w[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u) row_entry(P, cur.d, base + es + u * ES, c[u], y[u]);
+#pragma unroll
+            for (int u = 0; u < U; ++u)
+                w[u] = (jok && base + es + u * ES < cnt) ? ld_relaxed(src + (size_t)c[u] * nr + j) : T(0);
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                if (jok && base + es + u * ES < cnt) w[u] = wait_value(src + (size_t)c[u] * nr + j, w[u]);
+                acc += y[u] * w[u];
             }
         }
 #pragma unroll
         for (int o = NR; o < 32; o <<= 1) acc += __shfl_xor_sync(kFull, acc, o);
-        if (es == 0 && jok) st_relaxed(P.x + (size_t)cur.row * nr + j, cur.b - acc);
+        if (es == 0 && jok) st_relaxed(P.x + (size_t)cur.d.row * nr + j, cur.b - acc);
     }
 }
 
-// Vector-row variant (rw_options.wide_slices = -1): one warp per row, lane l
-// owns entries s + l, s + l + 32, ... and reads all right-hand sides of an
-// entry in one relaxed vector load, so 4 entries per lane held ahead cover
-// rows of up to 128 entries and a long row on the critical path costs one
-// round of loads, not one per few entries.
+// Vector entries (rw_options.wide_slices = -1): lane l owns entries l, l + 32,
+// ... and reads all right-hand sides of an entry in one relaxed vector load, so
+// 4 entries per lane held ahead cover rows of up to 128 entries and a long row
+// on the critical path costs one round of loads, not one per few entries.
 template <typename T, int NR>
 __device__ __forceinline__ void xload_relaxed(const T* x, int nrhs, int32_t c, T (&v)[NR]) {
     const T* p = x + (size_t)c * nrhs;
@@ -999,7 +778,8 @@ __device__ __forceinline__ bool any_pending(const T (&v)[NR], int nrhs) {
 // MINB = 2 caps the registers so that two 512-thread blocks share an SM:
 // twice the rows in flight, at the cost of some spilled prefetch state.
 template <typename T, int NR, int MINB>
-__global__ void __launch_bounds__(512, MINB) k_syncfree_vec(const FreeParams<T> P) {
+__global__ void __launch_bounds__(512, MINB) k_rows_vec(const RowParams<T> P) {
+    constexpr int U = kPreEntries;
     const int lane = (int)lane_id();
     constexpr int span = 32 / NR;
     const int jo = lane / span;  // the right-hand side this lane stores
@@ -1007,34 +787,8 @@ __global__ void __launch_bounds__(512, MINB) k_syncfree_vec(const FreeParams<T> 
     const int64_t gw = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
     const unsigned spin_limit = P.st->spin_limit;
-    struct Pre {
-        int32_t row;
-        int64_t s, e;
-        int32_t c[kPreEntries];
-        T y[kPreEntries];
-        T b;
-    };
-    auto load = [&](int64_t pos, Pre& R0) {
-        R0.row = -1;
-        if (pos >= P.n) return;
-        const int32_t row = P.order[pos];
-        R0.row = row;
-        R0.s = P.rp[row];
-        R0.e = P.rp[row + 1];
-#pragma unroll
-        for (int u = 0; u < kPreEntries; ++u) {
-            const int64_t q = R0.s + lane + (int64_t)u * 32;
-            R0.c[u] = q < R0.e ? P.col[q] : 0;
-            R0.y[u] = q < R0.e ? P.val[q] : T(0);
-        }
-        R0.b = T(0);
-        if (owner) {
-            R0.b = P.rhs[(size_t)row * P.nrhs + jo];
-            if (P.scale) R0.b = R0.b / P.scale[row];
-        }
-    };
     // re-polls (bounded, backing off) while any of the vector is pending
-    auto wait_vec = [&](int32_t c, T (&v)[NR]) {
+    auto wait_vec = [&](const T* src, int32_t c, T (&v)[NR]) {
         unsigned spins = 0;
         while (any_pending<T, NR>(v, P.nrhs)) {
             if (wait_gives_up(spins, spin_limit, &P.st->timeout)) {
@@ -1043,125 +797,401 @@ __global__ void __launch_bounds__(512, MINB) k_syncfree_vec(const FreeParams<T> 
                 return;
             }
             if (spins > 4) __nanosleep(32);
-            xload_relaxed<T, NR>(P.x, P.nrhs, c, v);
+            xload_relaxed<T, NR>(src, P.nrhs, c, v);
         }
     };
+    struct Pre {
+        SolveRow d;
+        int32_t c[U];
+        T y[U];
+        T b;
+    };
+    auto load = [&](const SolveRow& d, Pre& R) {
+        R.d = d;
+#pragma unroll
+        for (int u = 0; u < U; ++u) row_entry(P, d, lane + u * 32, R.c[u], R.y[u]);
+        R.b = owner && d.row >= 0 ? P.rhs[(size_t)d.row * P.nrhs + jo] : T(0);
+    };
     Pre pre[2];
-    load(gw, pre[0]);
-    load(gw + nw, pre[1]);
+    load(row_at(P, gw), pre[0]);
+    load(row_at(P, gw + nw), pre[1]);
+    SolveRow after = row_at(P, gw + 2 * nw);
     for (int64_t pos = gw; pos < P.n; pos += nw) {
         const Pre cur = pre[0];
         pre[0] = pre[1];
-        load(pos + 2 * nw, pre[1]);
+        load(after, pre[1]);
+        after = row_at(P, pos + 3 * nw);
+        const int cnt = cur.d.cnt;
+        const T* const src = P.x;
         T acc[NR];
 #pragma unroll
         for (int j = 0; j < NR; ++j) acc[j] = T(0);
-        T v[kPreEntries][NR];
+        int32_t c[U];
+        T y[U];
 #pragma unroll
-        for (int u = 0; u < kPreEntries; ++u) {
-            if (cur.s + lane + (int64_t)u * 32 < cur.e) {
-                xload_relaxed<T, NR>(P.x, P.nrhs, cur.c[u], v[u]);
-            } else {
-#pragma unroll
-                for (int j = 0; j < NR; ++j) v[u][j] = T(0);
-            }
+        for (int u = 0; u < U; ++u) {
+            c[u] = cur.c[u];
+            y[u] = cur.y[u];
         }
+        bool first = cur.d.last >= 0;
+        for (int base = 0; base < cnt; base += U * 32) {
+            if (base > 0) {
 #pragma unroll
-        for (int u = 0; u < kPreEntries; ++u) {
-            if (cur.s + lane + (int64_t)u * 32 < cur.e) wait_vec(cur.c[u], v[u]);
-#pragma unroll
-            for (int j = 0; j < NR; ++j) acc[j] += cur.y[u] * v[u][j];
-        }
-        for (int64_t q = cur.s + lane + (int64_t)kPreEntries * 32; q < cur.e; q += 4 * 32) {
-            int32_t c[4];
-            T y[4], w[4][NR];
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const bool ok = q + u * 32 < cur.e;
-                c[u] = ok ? P.col[q + u * 32] : 0;
-                y[u] = ok ? P.val[q + u * 32] : T(0);
+                for (int u = 0; u < U; ++u) row_entry(P, cur.d, base + lane + u * 32, c[u], y[u]);
             }
+            T v[U][NR];
+            bool pend = false;
 #pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                if (q + u * 32 < cur.e) {
-                    xload_relaxed<T, NR>(P.x, P.nrhs, c[u], w[u]);
+            for (int u = 0; u < U; ++u) {
+                if (base + lane + u * 32 < cnt) {
+                    xload_relaxed<T, NR>(src, P.nrhs, c[u], v[u]);
+                    pend |= any_pending<T, NR>(v[u], P.nrhs);
                 } else {
 #pragma unroll
-                    for (int j = 0; j < NR; ++j) w[u][j] = T(0);
+                    for (int j = 0; j < NR; ++j) v[u][j] = T(0);
                 }
             }
+            if (first && __any_sync(kFull, pend)) {
+                T w[NR];
+                xload_relaxed<T, NR>(src, P.nrhs, cur.d.last, w);
+                wait_vec(src, cur.d.last, w);
 #pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                if (q + u * 32 < cur.e) wait_vec(c[u], w[u]);
+                for (int u = 0; u < U; ++u)
+                    if (base + lane + u * 32 < cnt && any_pending<T, NR>(v[u], P.nrhs))
+                        xload_relaxed<T, NR>(src, P.nrhs, c[u], v[u]);
+                first = false;
+            }
 #pragma unroll
-                for (int j = 0; j < NR; ++j) acc[j] += y[u] * w[u][j];
+            for (int u = 0; u < U; ++u) {
+                if (base + u * 32 < cnt) {  // (FP64 instructions only for the slots the row uses)
+                    if (base + lane + u * 32 < cnt) wait_vec(src, c[u], v[u]);
+#pragma unroll
+                    for (int j = 0; j < NR; ++j) acc[j] += y[u] * v[u][j];
+                }
             }
         }
         const T sum = warp_sums_spread<T, NR>(acc);
-        if (owner) st_relaxed(P.x + (size_t)cur.row * P.nrhs + jo, cur.b - sum);
+        if (owner) st_relaxed(P.x + (size_t)cur.d.row * P.nrhs + jo, cur.b - sum);
     }
 }
 
-template <typename T>
-__global__ void k_inverse_diag(T* w, const T* __restrict__ d, int64_t n, int nrhs) {
-    const int64_t cnt = n * nrhs;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < cnt; i += (int64_t)gridDim.x * blockDim.x)
-        w[i] = w[i] / d[i / nrhs];
-}
-
-template <typename T>
-rw_status apply_inverse_diag(rw_context* ctx, T* w, const T* d, int64_t n, int nrhs) {
-    const int64_t cnt = n * nrhs;
-    if (cnt == 0) return RW_OK;
-    RW_COUNT_LAUNCH();
-    k_inverse_diag<T><<<grid_for(cnt, 256, ctx->num_sms * 8), 256, 0, ctx->stream>>>(w, d, n, nrhs);
-    return check_launch("inverse diagonal");
-}
-template rw_status apply_inverse_diag<double>(rw_context*, double*, const double*, int64_t, int);
-template rw_status apply_inverse_diag<float>(rw_context*, float*, const float*, int64_t, int);
-
-template <typename T>
-__global__ void k_fill_pending_sched(T* x, int64_t cnt) {
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < cnt;
-         i += (int64_t)gridDim.x * blockDim.x)
-        x[i] = pending_value(T(0));
-}
-
-// Positions [pos_begin, pos_end) of the level order, sync-free; the rows of
-// the range must hold the pending marker (fill = true marks the whole vector
-// first) and every dependency outside the range must be final.
 template <typename T, int NR, bool VEC>
-static rw_status solve_syncfree(rw_context* ctx, const SolveSchedule& S, const int64_t* rp, const int32_t* col,
-                                const T* val, const T* rhs, const T* scale, T* x, int nrhs,
-                                int64_t pos_begin, int64_t pos_end, bool fill) {
-    cudaStream_t s = ctx->stream;
+static rw_status launch_rows(rw_context* ctx, const RowParams<T>& P) {
     const int two = VEC && ctx->opt.solve_blocks_per_sm >= 2 ? 1 : 0;
     const void* kern;
-    if constexpr (VEC) kern = two ? (const void*)k_syncfree_vec<T, NR, 2> : (const void*)k_syncfree_vec<T, NR, 1>;
-    else kern = (const void*)k_syncfree<T, NR>;
+    if constexpr (VEC) kern = two ? (const void*)k_rows_vec<T, NR, 2> : (const void*)k_rows_vec<T, NR, 1>;
+    else kern = (const void*)k_rows<T, NR>;
     static int per_sm_of[2] = {-1, -1};
     int& per_sm = per_sm_of[two];
     if (per_sm < 0) {
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 512, 0);
         if (per_sm < 1) per_sm = 1;
     }
-    if (fill) {
-        const int64_t cnt = (int64_t)S.n * nrhs;
-        RW_COUNT_LAUNCH();
-        k_fill_pending_sched<T><<<grid_for(cnt, 256, ctx->num_sms * 8), 256, 0, s>>>(x, cnt);
-        rw_status rc = check_launch("pending fill");
-        if (rc) return rc;
-    }
-    const int64_t rows = pos_end - pos_begin;
     int64_t blocks = (int64_t)std::min(per_sm, 2) * ctx->num_sms;
-    const int64_t need = (rows + 15) / 16;
+    const int64_t need = (P.n + 15) / 16;
     if (blocks > need) blocks = need;
     if (blocks < 1) blocks = 1;
-    FreeParams<T> P{rows, S.order + pos_begin, rp, col, val, rhs, scale, x, nrhs, ctx->d_status};
     void* args[] = {(void*)&P};
     RW_COUNT_LAUNCH();
-    return check_cuda(cudaLaunchCooperativeKernel(kern, dim3((unsigned)blocks), dim3(512), args, 0, s),
-                      "sync-free solve");
+    return check_cuda(cudaLaunchCooperativeKernel(kern, dim3((unsigned)blocks), dim3(512), args, 0, ctx->stream),
+                      "row solve");
+}
+
+// ---------------------------------------------------------------------------
+// Narrow stretch: its blocks one after the other, over a co-resident grid of
+// one 256-thread block per SM.  The first kMainBlocks of them solve: in step b
+// 256 of their warps take one slot of block b each,
+//   gather: t_s = p_s - (entries in block b - 1), p_s being the right-hand side
+//           minus the earlier entries;
+//   a barrier among the solving blocks;
+//   solve:  x_s = sum_{u <= s} (L_BB^-1)_su t_u;
+//   a barrier of the whole grid.
+// The other blocks prepare p of block b + 1 meanwhile: everything up to block
+// b - 1 is final.  Entries from before the stretch, most of the thousands that
+// the long rows of Y^T hold, are summed by the whole chip before it
+// (k_stretch_begin).  The chain per block is then two barriers and two rounds
+// of loads.
+// ---------------------------------------------------------------------------
+constexpr int kMainBlocks = 64;  // 256 slots: four warps of each (see k_blocks)
+constexpr int kLongGather = 512;
+
+template <typename T>
+struct BlockSums {
+    const int64_t* __restrict__ ptr;
+    const int32_t* __restrict__ idx;
+    const T* __restrict__ val;
+};
+
+template <typename T>
+struct BlockParams {
+    const SolveBlock* __restrict__ blocks;
+    int32_t block0, nblocks;
+    const int32_t* __restrict__ trow;
+    BlockSums<T> prev, older;
+    bool from_rhs;           // the stretch starts the order: t has not been set
+    const T* __restrict__ inv;
+    const T* __restrict__ rhs;
+    T* x;
+    T* t;
+    int nrhs;
+    unsigned* bar;           // [0] grid barrier, [1] barrier of the solving blocks
+    unsigned epoch0, mid0;   // barriers passed by earlier launches of this solve
+    DevStatus* st;
+};
+
+// Barrier of the thread blocks that arrive at *count (see grid_barrier): passed
+// when it reaches target.  Returns false when a wait gave up.
+__device__ __forceinline__ bool blocks_barrier(unsigned* count, unsigned target, DevStatus* st) {
+    __shared__ int give_up;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        give_up = 0;
+        const unsigned limit = st->spin_limit;
+        atom_add_release(count, 1u);
+        unsigned spins = 0;
+        while ((int)(ld_acquire_u32(count) - target) < 0) {
+            if (wait_gives_up(spins, limit, &st->timeout)) {
+                give_up = 1;
+                break;
+            }
+        }
+    }
+    __syncthreads();
+    return give_up == 0;
+}
+
+// The nrhs values at node c (vector loads when nrhs == NR), from L2.
+template <typename T, int NR>
+__device__ __forceinline__ void xload_cg(const T* x, int nrhs, int64_t c, T (&v)[NR]) {
+    const T* p = x + c * nrhs;
+    if constexpr (NR >= 2 && sizeof(T) == 8) {
+        if (nrhs == NR) {
+#pragma unroll
+            for (int j = 0; j < NR; j += 2) {
+                const double2 d = __ldcg(reinterpret_cast<const double2*>(p + j));
+                v[j] = d.x;
+                v[j + 1] = d.y;
+            }
+            return;
+        }
+    } else if constexpr (NR >= 4 && sizeof(T) == 4) {
+        if (nrhs == NR) {
+#pragma unroll
+            for (int j = 0; j < NR; j += 4) {
+                const float4 d = __ldcg(reinterpret_cast<const float4*>(p + j));
+                v[j] = d.x;
+                v[j + 1] = d.y;
+                v[j + 2] = d.z;
+                v[j + 3] = d.w;
+            }
+            return;
+        }
+    }
+#pragma unroll
+    for (int j = 0; j < NR; ++j) v[j] = j < nrhs ? __ldcg(p + j) : T(0);
+}
+
+// acc += sum of val[q] * x[idx[q]] over q = q0, q0 + step, ... < q1
+template <typename T, int NR>
+__device__ __forceinline__ void gather(const BlockSums<T>& B, const T* x, int nrhs, int64_t q0, int64_t q1, int step,
+                                       T (&acc)[NR]) {
+    constexpr int U = NR >= 16 ? 1 : NR >= 8 ? 2 : 4;
+    for (int64_t q = q0; q < q1; q += (int64_t)U * step) {
+        int32_t c[U];
+        T y[U], v[U][NR];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const bool ok = q + u * step < q1;
+            c[u] = ok ? B.idx[q + u * step] : -1;
+            y[u] = ok ? B.val[q + u * step] : T(0);
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+            if (c[u] >= 0) xload_cg<T, NR>(x, nrhs, c[u], v[u]);
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+            if (c[u] >= 0) {
+#pragma unroll
+                for (int j = 0; j < NR; ++j) acc[j] += y[u] * v[u][j];
+            }
+    }
+}
+
+// t of `count` <= 8 slots from t0 on, less their rows' sums over B: a warp per
+// slot, the whole thread block for a row of more than kLongGather entries.
+// from_rhs: t starts as the right-hand side (otherwise as what it holds).
+template <typename T, int NR>
+__device__ __forceinline__ void gather_slots(const BlockSums<T>& B, const T* x, const T* rhs, bool from_rhs,
+                                             const int32_t* trow, T* t, int nr, int64_t t0, int count,
+                                             T (&part)[8][NR]) {
+    constexpr int span = 32 / NR;
+    const int lane = (int)lane_id(), warp = (int)threadIdx.x >> 5;
+    const int jo = lane / span;
+    const bool owner = (lane % span) == 0 && jo < nr;
+    for (int i = 0; i < count; ++i) {
+        const int64_t q0 = B.ptr[t0 + i], q1 = B.ptr[t0 + i + 1];
+        const bool whole = q1 - q0 > kLongGather;
+        if (!whole && warp != i) continue;
+        T acc[NR];
+#pragma unroll
+        for (int j = 0; j < NR; ++j) acc[j] = T(0);
+        if (whole) gather<T, NR>(B, x, nr, q0 + threadIdx.x, q1, 256, acc);
+        else gather<T, NR>(B, x, nr, q0 + lane, q1, 32, acc);
+        T sum = warp_sums_spread<T, NR>(acc);
+        if (whole) {
+            __syncthreads();
+            if ((lane % span) == 0) part[warp][jo] = sum;
+            __syncthreads();
+            if (warp != i) continue;
+            sum = T(0);
+            for (int w = 0; w < 8; ++w) sum += part[w][jo];
+        }
+        if (owner) {
+            T* to = t + (t0 + i) * nr + jo;
+            __stcg(to, (from_rhs ? rhs[(size_t)trow[t0 + i] * nr + jo] : __ldcg(to)) - sum);
+        }
+    }
+}
+
+// The right-hand sides of a stretch's slots less their rows' entries from
+// before the stretch.
+template <typename T, int NR>
+__global__ void __launch_bounds__(256) k_stretch_begin(int64_t t0, int64_t t1, const SolveBlock* __restrict__ blocks,
+                                                       const BlockSums<T> B, const T* x, const T* __restrict__ rhs,
+                                                       const int32_t* __restrict__ trow, T* t, int nr) {
+    __shared__ T part[8][NR];
+    for (int64_t s = t0 + (int64_t)blockIdx.x * 8; s < t1; s += (int64_t)gridDim.x * 8) {
+        const int rows = blocks[s / kBlockRows].rows - (int)(s % kBlockRows);
+        if (rows > 0) gather_slots<T, NR>(B, x, rhs, true, trow, t, nr, s, min(8, rows), part);
+    }
+}
+
+template <typename T, int NR>
+__global__ void __launch_bounds__(256, 1) k_blocks(const BlockParams<T> P) {
+    constexpr int span = 32 / NR;
+    constexpr int U = 4;                    // entries per lane of the block before read ahead
+    constexpr int V = kBlockRows / 32;      // entries per lane of the inverse's row
+    __shared__ T part[8][NR];
+    const int lane = (int)lane_id(), warp = (int)threadIdx.x >> 5;
+    const int jo = lane / span;  // the right-hand side this lane stores
+    const bool owner = (lane % span) == 0 && jo < P.nrhs;
+    const bool solves = (int)blockIdx.x < kMainBlocks;
+    const int nr = P.nrhs;
+    const int slot = warp * kMainBlocks + (int)blockIdx.x;  // rows of all lengths on every SM
+
+    // what step b reads that does not depend on x, loaded before the barrier that starts it
+    bool mine = false;
+    int32_t row = 0, c[U];
+    int64_t q1 = 0, q0 = 0;
+    T y[U], iv[V];
+    auto fetch = [&](int64_t b) {
+        mine = slot < P.blocks[b].rows;
+        const int64_t t = b * kBlockRows + slot;
+        q0 = q1 = 0;
+        if (mine) {
+            row = P.trow[t];
+            q0 = P.prev.ptr[t] + lane;
+            q1 = P.prev.ptr[t + 1];
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const bool ok = q0 + 32 * u < q1;
+            c[u] = ok ? P.prev.idx[q0 + 32 * u] : -1;
+            y[u] = ok ? P.prev.val[q0 + 32 * u] : T(0);
+        }
+        const T* inv = P.inv + b * tri(kBlockRows) + tri(slot);
+#pragma unroll
+        for (int k = 0; k < V; ++k) iv[k] = mine && lane + 32 * k <= slot ? inv[lane + 32 * k] : T(0);
+    };
+
+    unsigned epoch = P.epoch0, mid = P.mid0;
+    if (solves && slot < kBlockRows) fetch(P.block0);
+    for (int i = 0; i < P.nblocks; ++i) {
+        const int64_t b = P.block0 + i, t = b * kBlockRows + slot;
+        if (solves) {
+            if (mine) {
+                // (the stretch's first block has no earlier entries in it)
+                const T p = !owner                 ? T(0)
+                            : P.from_rhs && i == 0 ? P.rhs[(size_t)row * nr + jo]
+                                                   : __ldcg(P.t + t * nr + jo);
+                T acc[NR];
+#pragma unroll
+                for (int j = 0; j < NR; ++j) acc[j] = T(0);
+                constexpr int W = NR >= 16 ? 1 : NR >= 8 ? 2 : U;  // loads in flight
+#pragma unroll
+                for (int u0 = 0; u0 < U; u0 += W) {
+                    T v[W][NR];
+#pragma unroll
+                    for (int u = 0; u < W; ++u)
+                        if (c[u0 + u] >= 0) xload_cg<T, NR>(P.x, nr, c[u0 + u], v[u]);
+#pragma unroll
+                    for (int u = 0; u < W; ++u)
+                        if (c[u0 + u] >= 0) {
+#pragma unroll
+                            for (int j = 0; j < NR; ++j) acc[j] += y[u0 + u] * v[u][j];
+                        }
+                }
+                gather<T, NR>(P.prev, P.x, nr, q0 + 32 * U, q1, 32, acc);
+                const T sum = warp_sums_spread<T, NR>(acc);
+                if (owner) __stcg(P.t + t * nr + jo, p - sum);
+            }
+            if (!blocks_barrier(P.bar + 1, ++mid * (unsigned)kMainBlocks, P.st)) return;
+            if (mine) {
+                T acc[NR];
+#pragma unroll
+                for (int j = 0; j < NR; ++j) acc[j] = T(0);
+                constexpr int W = NR >= 8 ? 1 : 16 / NR >= V ? V : 16 / NR;  // loads in flight
+#pragma unroll
+                for (int k0 = 0; k0 < V; k0 += W) {
+                    T v[W][NR];
+#pragma unroll
+                    for (int k = 0; k < W; ++k)
+                        if (lane + 32 * (k0 + k) <= slot)
+                            xload_cg<T, NR>(P.t, nr, b * kBlockRows + lane + 32 * (k0 + k), v[k]);
+#pragma unroll
+                    for (int k = 0; k < W; ++k)
+                        if (32 * (k0 + k) <= slot) {  // (FP64 instructions only for what the row holds)
+#pragma unroll
+                            for (int j = 0; j < NR; ++j)
+                                acc[j] += lane + 32 * (k0 + k) <= slot ? iv[k0 + k] * v[k][j] : T(0);
+                        }
+                }
+                const T sum = warp_sums_spread<T, NR>(acc);
+                if (owner) __stcg(P.x + (size_t)row * nr + jo, sum);
+            }
+            if (i + 1 < P.nblocks && slot < kBlockRows) fetch(b + 1);
+        } else if (i + 1 < P.nblocks) {
+            // p of the next block's slots, eight at a time
+            const int rows = P.blocks[b + 1].rows, others = (int)gridDim.x - kMainBlocks;
+            for (int s0 = ((int)blockIdx.x - kMainBlocks) * 8; s0 < rows; s0 += others * 8)
+                gather_slots<T, NR>(P.older, P.x, P.rhs, P.from_rhs, P.trow, P.t, nr, (b + 1) * kBlockRows + s0,
+                                    min(8, rows - s0), part);
+        }
+        if (i + 1 < P.nblocks && !blocks_barrier(P.bar, ++epoch * gridDim.x, P.st)) return;
+    }
+}
+
+template <typename T, int NR>
+static rw_status launch_blocks(rw_context* ctx, const BlockParams<T>& P) {
+    void* args[] = {(void*)&P};
+    RW_COUNT_LAUNCH();
+    return check_cuda(cudaLaunchCooperativeKernel((const void*)k_blocks<T, NR>, dim3((unsigned)ctx->num_sms),
+                                                  dim3(256), args, 0, ctx->stream),
+                      "block solve");
+}
+
+// Before a solve: x marked pending (solve modes 1 and 2), the barrier words of
+// its block launches cleared, and in the forward solve w <- w / d row by row (the
+// D^-1 step between the two solves: one FP64 division instruction serves 32 rows
+// here, one row inside the solve).
+template <typename T>
+__global__ void k_solve_begin(T* x, int64_t cnt, T* w, const T* __restrict__ d, int nrhs, unsigned* bar) {
+    const int64_t i0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, step = (int64_t)gridDim.x * blockDim.x;
+    if (i0 < 2) bar[i0] = 0u;
+    for (int64_t i = i0; i < cnt; i += step) {
+        if (x) x[i] = pending_value(T(0));
+        if (w) w[i] = w[i] / d[i / nrhs];
+    }
 }
 
 // ---------------------------------------------------------------------------
@@ -1179,7 +1209,7 @@ static int lane_slices(int opt, int NR) {
 
 template <typename T, int NR, int ES>
 static rw_status launch_wide(rw_context* ctx, const SolveSchedule& S, int32_t lev_begin, int32_t lev_end,
-                             const int64_t* rp, const int32_t* col, const T* val, const T* rhs, const T* scale,
+                             const int64_t* rp, const int32_t* col, const T* val, const T* rhs,
                              T* x, int nrhs, unsigned* bar) {
     if constexpr (NR * ES > 32) {
         return RW_ERR_ARG;
@@ -1200,7 +1230,7 @@ static rw_status launch_wide(rw_context* ctx, const SolveSchedule& S, int32_t le
         const int64_t need = (maxw + rows_per_block - 1) / rows_per_block;
         if (blocks > need) blocks = need;
         if (blocks < 1) blocks = 1;
-        WideParams<T> P{lev_begin, lev_end, S.lptr, S.order, rp, col, val, rhs, scale, x, nrhs, bar, ctx->d_status};
+        WideParams<T> P{lev_begin, lev_end, S.lptr, S.order, rp, col, val, rhs, x, nrhs, bar, ctx->d_status};
         void* args[] = {(void*)&P};
         RW_COUNT_LAUNCH();
         return check_cuda(cudaLaunchCooperativeKernel((const void*)k_wide<T, NR, ES>, dim3((unsigned)blocks),
@@ -1212,14 +1242,14 @@ static rw_status launch_wide(rw_context* ctx, const SolveSchedule& S, int32_t le
 template <typename T, int NR, int ES>
 static rw_status launch_cluster(rw_context* ctx, const SolveSchedule& S, int32_t lev_begin, int32_t lev_end,
                                 const int64_t* rp, const int32_t* col, const T* val, const T* rhs,
-                                const T* scale, T* x, int nrhs, unsigned* bar, int csize) {
+                                T* x, int nrhs, unsigned* bar, int csize) {
     if constexpr (NR * ES > 32) {
         return RW_ERR_ARG;
     } else {
         rw_status arc = set_kernel_attr_once(ctx->device, (const void*)k_cluster<T, NR, ES>,
                                              cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
         if (arc) return arc;
-        WideParams<T> P{lev_begin, lev_end, S.lptr, S.order, rp, col, val, rhs, scale, x, nrhs, bar, ctx->d_status};
+        WideParams<T> P{lev_begin, lev_end, S.lptr, S.order, rp, col, val, rhs, x, nrhs, bar, ctx->d_status};
         cudaLaunchConfig_t cfg = {};
         cfg.blockDim = dim3(NR >= 8 ? 512u : 1024u);
         cfg.dynamicSmemBytes = 0;
@@ -1252,217 +1282,136 @@ static rw_status launch_cluster(rw_context* ctx, const SolveSchedule& S, int32_t
     }
 }
 
+// The level schedule: consecutive levels up to the cluster width go to one
+// cluster, the rest to the whole grid.
 template <typename T, int NR, int ES>
-static rw_status launch_nonthin(rw_context* ctx, const SolveSchedule& S, const SolveRun& run, const int64_t* rp,
-                                const int32_t* col, const T* val, const T* rhs, const T* scale, T* x, int nrhs,
-                                unsigned* bar) {
-    // consecutive levels up to the cluster width go to one cluster, the rest
-    // to the whole grid
+static rw_status launch_levels(rw_context* ctx, const SolveSchedule& S, const int64_t* rp, const int32_t* col,
+                               const T* val, const T* rhs, T* x, int nrhs, unsigned* bar) {
     const int64_t cw = ctx->opt.cluster_width > 0 ? ctx->opt.cluster_width : 0;
     const int csize = ctx->opt.cluster_size > 0 ? ctx->opt.cluster_size : 16;
-    int32_t l = run.lev_begin;
-    while (l < run.lev_end) {
+    int32_t l = 0;
+    while (l < S.depth) {
         const bool narrow = cw > 0 && S.lptr_h[l + 1] - S.lptr_h[l] <= cw;
         int32_t e = l + 1;
-        while (e < run.lev_end && (cw > 0 && S.lptr_h[e + 1] - S.lptr_h[e] <= cw) == narrow) ++e;
+        while (e < S.depth && (cw > 0 && S.lptr_h[e + 1] - S.lptr_h[e] <= cw) == narrow) ++e;
         // cluster runs (1024-thread blocks, 64 registers) keep lane groups
         constexpr int CES = ES == 0 ? 32 / NR : ES;
-        rw_status rc = narrow ? launch_cluster<T, NR, CES>(ctx, S, l, e, rp, col, val, rhs, scale, x, nrhs, bar, csize)
-                              : launch_wide<T, NR, ES>(ctx, S, l, e, rp, col, val, rhs, scale, x, nrhs, bar);
+        rw_status rc = narrow ? launch_cluster<T, NR, CES>(ctx, S, l, e, rp, col, val, rhs, x, nrhs, bar, csize)
+                              : launch_wide<T, NR, ES>(ctx, S, l, e, rp, col, val, rhs, x, nrhs, bar);
         if (rc) return rc;
         l = e;
     }
     return RW_OK;
 }
 
-// CTAs of a thin run's cluster (rw_options.thin_cluster, a power of two
-// <= 16), reduced to the largest size the device can place with this shared
-// memory; 1 = one block.
-template <typename T, int NR>
-static int thin_cluster_size(rw_context* ctx, size_t smem) {
-    int want = ctx->opt.thin_cluster;
-    if (want < 2) return 1;
-    if (want > 16) want = 16;
-    int c = 1;
-    while (c * 2 <= want) c *= 2;
-    static int placeable[17][2] = {};  // per size: 0 unknown, 1 yes, -1 no (by smem above or below 128 KB)
-    const int big = smem > 128 * 1024 ? 1 : 0;
-    while (c > 1) {
-        if (placeable[c][big] == 0) {
-            cudaLaunchConfig_t cfg = {};
-            cfg.gridDim = dim3((unsigned)c);
-            cfg.blockDim = dim3(kThinThreads);
-            cfg.dynamicSmemBytes = big ? kThinSmemBudget + 16 * 1024 : 128 * 1024;
-            cudaLaunchAttribute at[1];
-            at[0].id = cudaLaunchAttributeClusterDimension;
-            at[0].val.clusterDim.x = (unsigned)c;
-            at[0].val.clusterDim.y = 1;
-            at[0].val.clusterDim.z = 1;
-            cfg.attrs = at;
-            cfg.numAttrs = 1;
-            int nc = 0;
-            placeable[c][big] =
-                (cudaOccupancyMaxActiveClusters(&nc, k_thin<T, NR, true>, &cfg) == cudaSuccess && nc >= 1) ? 1 : -1;
-            cudaGetLastError();
-        }
-        if (placeable[c][big] > 0) return c;
-        c >>= 1;
-    }
-    return 1;
+template <typename T>
+static const T* schedule_values(const double* v, const float* v32) {
+    if constexpr (sizeof(T) == 8) return v;
+    else return v32;
+}
+
+template <typename T>
+static BlockSums<T> block_sums(const SolveEntries& E) {
+    return BlockSums<T>{E.ptr, E.idx, schedule_values<T>(E.val, E.val32)};
 }
 
 template <typename T, int NR>
 static rw_status solve_runs_nr(rw_context* ctx, const SolveSchedule& S, const int64_t* rp,
-                               const int32_t* col, const T* val, const T* tval, const T* rhs,
-                               const T* scale, T* x, int nrhs, unsigned* bar, int mode) {
+                               const int32_t* col, const T* val, const T* rhs, T* x, int nrhs, unsigned* bar, int mode,
+                               T* w, const T* d) {
     cudaStream_t s = ctx->stream;
-    T* ext = reinterpret_cast<T*>(bar + 64);  // the factor's solve workspace (see build_factor)
     rw_status rc;
-    if (mode == 1) {
-        if (S.n == 0) return RW_OK;
-        // vector rows while one entry's right-hand sides fit in 32 bytes of registers
-        if constexpr (NR * sizeof(T) <= 32) {
-            if (ctx->opt.wide_slices < 0)
-                return solve_syncfree<T, NR, true>(ctx, S, rp, col, val, rhs, scale, x, nrhs, 0, S.n, true);
-        }
-        return solve_syncfree<T, NR, false>(ctx, S, rp, col, val, rhs, scale, x, nrhs, 0, S.n, true);
-    }
-    // mode 2 (hybrid): thin runs of at least kHybridThinLevels levels as in the
-    // level schedule; everything between them (wide runs and short thin runs,
-    // contiguous positions) as one sync-free launch each, so short runs cost no
-    // launch of their own.  The whole vector is marked pending once, before
-    // the first run (a launch reads only rows of earlier launches, final by
-    // then, and its own rows).
-    if (mode == 2 && S.n > 0) {
-        const int64_t cnt = (int64_t)S.n * nrhs;
+    const bool rows = mode == 1 || mode == 2;
+    const int64_t cnt = (int64_t)S.n * nrhs;
+    if (rows || w) {
         RW_COUNT_LAUNCH();
-        k_fill_pending_sched<T><<<grid_for(cnt, 256, ctx->num_sms * 8), 256, 0, s>>>(x, cnt);
-        if ((rc = check_launch("pending fill"))) return rc;
+        k_solve_begin<T><<<grid_for(cnt, 256, ctx->num_sms * 8), 256, 0, s>>>(rows ? x : nullptr, cnt, w, d, nrhs, bar);
+        if ((rc = check_launch("solve begin"))) return rc;
     }
-    // one-block thin runs: lanes per row (rw_options.thin_lanes), at least NR
-    int tl = ctx->opt.thin_lanes == 8 || ctx->opt.thin_lanes == 16 ? ctx->opt.thin_lanes : 32;
-    if (tl < NR) tl = 32;
-    const void* thin_kern = (const void*)k_thin<T, NR, false>;
-    if constexpr (NR <= 8) {
-        if (tl == 8) thin_kern = (const void*)k_thin<T, NR, false, 8>;
-    }
-    if constexpr (NR <= 16) {
-        if (tl == 16) thin_kern = (const void*)k_thin<T, NR, false, 16>;
-    }
-    if ((rc = set_kernel_attr_once(ctx->device, thin_kern,
-                                   cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kThinSmemBudget + 16 * 1024)) ||
-        (rc = set_kernel_attr_once(ctx->device, (const void*)k_thin<T, NR, true>,
-                                   cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kThinSmemBudget + 16 * 1024)) ||
-        (rc = set_kernel_attr_once(ctx->device, (const void*)k_thin<T, NR, true>,
-                                   cudaFuncAttributeNonPortableClusterSizeAllowed, 1)))
-        return rc;
-    const int es = lane_slices(ctx->opt.wide_slices, NR);
-    int64_t free_b = 0, free_e = 0;  // hybrid: positions waiting for one sync-free launch
-    auto flush_free = [&]() -> rw_status {
-        if (free_e <= free_b) return RW_OK;
-        rw_status r2;
-        if constexpr (NR * sizeof(T) <= 32) {
-            r2 = ctx->opt.wide_slices < 0
-                     ? solve_syncfree<T, NR, true>(ctx, S, rp, col, val, rhs, scale, x, nrhs, free_b, free_e, false)
-                     : solve_syncfree<T, NR, false>(ctx, S, rp, col, val, rhs, scale, x, nrhs, free_b, free_e, false);
-        } else {
-            r2 = solve_syncfree<T, NR, false>(ctx, S, rp, col, val, rhs, scale, x, nrhs, free_b, free_e, false);
-        }
-        free_b = free_e = 0;
-        return r2;
-    };
-    for (const SolveRun& run : S.runs) {
-        const int64_t rows = run.pos_end - run.pos_begin;
-        if (rows == 0) continue;
-        const int nlev = run.lev_end - run.lev_begin;
-        size_t smem = thin_stage_offset<T, NR>((int)rows, nlev);
-        const size_t staged = smem + (size_t)run.in_entries * (sizeof(T) + 4);
-        const int tc = thin_cluster_size<T, NR>(ctx, smem);  // 1: one block
-        const bool stage = run.thin && tc == 1 && staged <= kThinSmemBudget + 16 * 1024;
-        if (stage) smem = staged;
-        const bool thin_ok = run.thin && smem <= kThinSmemBudget + 16 * 1024 && rows <= kThinMaxRows;
-        if (mode == 2 && !(thin_ok && nlev >= kHybridThinLevels)) {
-            if (free_e <= free_b) free_b = run.pos_begin;
-            free_e = run.pos_end;
-            continue;
-        }
-        if (mode == 2 && (rc = flush_free())) return rc;
-        if (thin_ok) {
-            const int eb = grid_for(rows * 32, 256, ctx->num_sms * 4);
-            RW_COUNT_LAUNCH();
-            k_thin_ext<T, NR><<<eb, 256, 0, s>>>(run.pos_begin, run.pos_end, S.tptr, S.tnin, S.tidx,
-                                                  tval, x, nrhs, ext);
-            ThinParams<T> P{run.pos_begin, run.pos_end, run.lev_begin, run.lev_end, S.lptr, S.order,
-                            S.tptr, S.tnin, S.tidx, tval, ext, rhs, scale, x, nrhs, stage ? 1 : 0,
-                            (int)run.in_entries, ctx->opt.thin_flags ? 1 : 0, ctx->d_status};
-            RW_COUNT_LAUNCH();
-            if (tc > 1) {
-                cudaLaunchConfig_t cfg = {};
-                cfg.gridDim = dim3((unsigned)tc);
-                cfg.blockDim = dim3(kThinThreads);
-                cfg.dynamicSmemBytes = smem;
-                cfg.stream = s;
-                cudaLaunchAttribute at[1];
-                at[0].id = cudaLaunchAttributeClusterDimension;
-                at[0].val.clusterDim.x = (unsigned)tc;
-                at[0].val.clusterDim.y = 1;
-                at[0].val.clusterDim.z = 1;
-                cfg.attrs = at;
-                cfg.numAttrs = 1;
-                if ((rc = check_cuda(cudaLaunchKernelEx(&cfg, k_thin<T, NR, true>, P), "thin-run cluster solve")))
-                    return rc;
-            } else {
-                void* args[] = {(void*)&P};
-                if ((rc = check_cuda(cudaLaunchKernel(thin_kern, dim3(1), dim3(kThinThreads), args, smem, s),
-                                     "thin-run solve")))
-                    return rc;
+    if (rows) {
+        // the rows at positions [pos0, pos1); vector entries while one entry's
+        // right-hand sides fit in 32 bytes of registers
+        auto solve_rows = [&](int64_t pos0, int64_t pos1) -> rw_status {
+            const RowParams<T> P{pos1 - pos0, S.rows + pos0, col, val, rhs, x, nrhs, ctx->d_status};
+            if constexpr (NR * sizeof(T) <= 32) {
+                if (ctx->opt.wide_slices < 0) return launch_rows<T, NR, true>(ctx, P);
             }
-            if ((rc = check_launch("thin-run solve"))) return rc;
-        } else {
-            switch (es) {
-                case 0:
-                    // vector rows while one entry's right-hand sides fit in 64 bytes of registers
-                    if constexpr (NR * sizeof(T) <= 64)
-                        rc = launch_nonthin<T, NR, 0>(ctx, S, run, rp, col, val, rhs, scale, x, nrhs, bar);
-                    else
-                        rc = launch_nonthin<T, NR, 32 / NR>(ctx, S, run, rp, col, val, rhs, scale, x, nrhs, bar);
-                    break;
-                case 1: rc = launch_nonthin<T, NR, 1>(ctx, S, run, rp, col, val, rhs, scale, x, nrhs, bar); break;
-                case 2: rc = launch_nonthin<T, NR, 2>(ctx, S, run, rp, col, val, rhs, scale, x, nrhs, bar); break;
-                case 4: rc = launch_nonthin<T, NR, 4>(ctx, S, run, rp, col, val, rhs, scale, x, nrhs, bar); break;
-                case 8: rc = launch_nonthin<T, NR, 8>(ctx, S, run, rp, col, val, rhs, scale, x, nrhs, bar); break;
-                case 16: rc = launch_nonthin<T, NR, 16>(ctx, S, run, rp, col, val, rhs, scale, x, nrhs, bar); break;
-                default: rc = launch_nonthin<T, NR, 32>(ctx, S, run, rp, col, val, rhs, scale, x, nrhs, bar); break;
+            return launch_rows<T, NR, false>(ctx, P);
+        };
+        if (mode == 1 || ctx->num_sms <= kMainBlocks) return solve_rows(0, S.n);
+        unsigned epoch = 0, mid = 0;
+        for (const SolveStretch& st : S.stretches) {
+            if (st.nblocks == 0) {
+                if ((rc = solve_rows(st.pos0, st.pos1))) return rc;
+                continue;
             }
-            if (rc) return rc;
+            BlockParams<T> P{};
+            P.blocks = S.blocks;
+            P.block0 = st.block0;
+            P.nblocks = st.nblocks;
+            P.trow = S.trow;
+            P.prev = block_sums<T>(S.ext[0]);
+            P.older = block_sums<T>(S.ext[1]);
+            P.from_rhs = st.pos0 == 0;
+            P.inv = schedule_values<T>(S.inv, S.inv32);
+            P.rhs = rhs;
+            P.x = x;
+            P.t = static_cast<T*>(S.t);
+            P.nrhs = nrhs;
+            P.bar = bar;
+            P.epoch0 = epoch;
+            P.mid0 = mid;
+            P.st = ctx->d_status;
+            if (st.pos0 > 0) {
+                const int64_t t0 = (int64_t)st.block0 * kBlockRows, t1 = t0 + (int64_t)st.nblocks * kBlockRows;
+                RW_COUNT_LAUNCH();
+                k_stretch_begin<T, NR><<<grid_for((t1 - t0) / 8, 1, ctx->num_sms * 8), 256, 0, s>>>(
+                    t0, t1, S.blocks, block_sums<T>(S.ext[2]), x, rhs, S.trow, P.t, nrhs);
+                if ((rc = check_launch("stretch begin"))) return rc;
+            }
+            if ((rc = launch_blocks<T, NR>(ctx, P))) return rc;
+            epoch += (unsigned)st.nblocks - 1;
+            mid += (unsigned)st.nblocks;
         }
+        return RW_OK;
     }
-    if (mode == 2 && (rc = flush_free())) return rc;
-    return RW_OK;
+    switch (lane_slices(ctx->opt.wide_slices, NR)) {
+        case 0:
+            // vector rows while one entry's right-hand sides fit in 64 bytes of registers
+            if constexpr (NR * sizeof(T) <= 64)
+                return launch_levels<T, NR, 0>(ctx, S, rp, col, val, rhs, x, nrhs, bar);
+            else
+                return launch_levels<T, NR, 32 / NR>(ctx, S, rp, col, val, rhs, x, nrhs, bar);
+        case 1: return launch_levels<T, NR, 1>(ctx, S, rp, col, val, rhs, x, nrhs, bar);
+        case 2: return launch_levels<T, NR, 2>(ctx, S, rp, col, val, rhs, x, nrhs, bar);
+        case 4: return launch_levels<T, NR, 4>(ctx, S, rp, col, val, rhs, x, nrhs, bar);
+        case 8: return launch_levels<T, NR, 8>(ctx, S, rp, col, val, rhs, x, nrhs, bar);
+        case 16: return launch_levels<T, NR, 16>(ctx, S, rp, col, val, rhs, x, nrhs, bar);
+        default: return launch_levels<T, NR, 32>(ctx, S, rp, col, val, rhs, x, nrhs, bar);
+    }
 }
 
 template <typename T>
 rw_status solve_runs(rw_context* ctx, const SolveSchedule& S, const int64_t* rp, const int32_t* col,
-                     const T* val, const T* tval, const T* rhs, const T* scale, T* x, int nrhs,
-                     unsigned* bar, bool backward) {
+                     const T* val, const T* rhs, T* x, int nrhs, unsigned* bar, bool backward, T* w, const T* d) {
     NvtxRange nvtx_range(backward ? "rw_solve_bwd" : "rw_solve_fwd");
+    if (S.n == 0) return RW_OK;
     const int mode = backward && ctx->opt.solve_mode_bwd >= 0 ? ctx->opt.solve_mode_bwd : ctx->opt.solve_mode;
     int nr = 1;
     while (nr < nrhs) nr <<= 1;
     switch (nr) {
-        case 1: return solve_runs_nr<T, 1>(ctx, S, rp, col, val, tval, rhs, scale, x, nrhs, bar, mode);
-        case 2: return solve_runs_nr<T, 2>(ctx, S, rp, col, val, tval, rhs, scale, x, nrhs, bar, mode);
-        case 4: return solve_runs_nr<T, 4>(ctx, S, rp, col, val, tval, rhs, scale, x, nrhs, bar, mode);
-        case 8: return solve_runs_nr<T, 8>(ctx, S, rp, col, val, tval, rhs, scale, x, nrhs, bar, mode);
-        default: return solve_runs_nr<T, 16>(ctx, S, rp, col, val, tval, rhs, scale, x, nrhs, bar, mode);
+        case 1: return solve_runs_nr<T, 1>(ctx, S, rp, col, val, rhs, x, nrhs, bar, mode, w, d);
+        case 2: return solve_runs_nr<T, 2>(ctx, S, rp, col, val, rhs, x, nrhs, bar, mode, w, d);
+        case 4: return solve_runs_nr<T, 4>(ctx, S, rp, col, val, rhs, x, nrhs, bar, mode, w, d);
+        case 8: return solve_runs_nr<T, 8>(ctx, S, rp, col, val, rhs, x, nrhs, bar, mode, w, d);
+        default: return solve_runs_nr<T, 16>(ctx, S, rp, col, val, rhs, x, nrhs, bar, mode, w, d);
     }
 }
 
-template rw_status solve_runs<double>(rw_context*, const SolveSchedule&, const int64_t*,
-                                      const int32_t*, const double*, const double*, const double*,
-                                      const double*, double*, int, unsigned*, bool);
-template rw_status solve_runs<float>(rw_context*, const SolveSchedule&, const int64_t*,
-                                     const int32_t*, const float*, const float*, const float*,
-                                     const float*, float*, int, unsigned*, bool);
+template rw_status solve_runs<double>(rw_context*, const SolveSchedule&, const int64_t*, const int32_t*,
+                                      const double*, const double*, double*, int, unsigned*, bool, double*,
+                                      const double*);
+template rw_status solve_runs<float>(rw_context*, const SolveSchedule&, const int64_t*, const int32_t*,
+                                     const float*, const float*, float*, int, unsigned*, bool, float*, const float*);
 
 }  // namespace rw

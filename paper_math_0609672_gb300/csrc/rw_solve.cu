@@ -181,13 +181,6 @@ void launch_to_fp32_diff(int32_t n, const int32_t* rp, const int32_t* col, const
     k_to_fp32_diff<<<grid_for(n, 256, num_sms * 8), 256, 0, s>>>(n, rp, col, val, a32);
 }
 
-template <typename T>
-__global__ void k_fill_pending(T* x, int64_t cnt) {
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < cnt;
-         i += (int64_t)gridDim.x * blockDim.x)
-        x[i] = pending_value(T(0));
-}
-
 // ---------------------------------------------------------------------------
 // PCG vector kernels and device scalars.
 // ---------------------------------------------------------------------------
@@ -324,11 +317,10 @@ __global__ void __launch_bounds__(256) k_dot(const TA* a, const TB* b, int64_t n
     block_dot_parts(a, b, n, nrhs, part);
 }
 
-// x += alpha p (x FP64), r -= alpha q; partial r.r; marks w and z pending.
+// x += alpha p (x FP64), r -= alpha q; partial r.r.
 template <typename T>
 __global__ void __launch_bounds__(256) k_update_xr(int64_t n, int nrhs, const PcgScalars* S,
-                                                   double* x, T* r, const T* p, const T* q, T* w,
-                                                   T* z, double* part) {
+                                                   double* x, T* r, const T* p, const T* q, double* part) {
     __shared__ double al[16];
     if (threadIdx.x < 16) al[threadIdx.x] = threadIdx.x < (unsigned)nrhs ? S->alpha[threadIdx.x] : 0.0;
     __syncthreads();
@@ -341,8 +333,6 @@ __global__ void __launch_bounds__(256) k_update_xr(int64_t n, int nrhs, const Pc
                 x[o] += a * (double)p[o];
                 r[o] = (T)((double)r[o] - a * (double)q[o]);
             }
-            w[o] = pending_value(T(0));
-            z[o] = pending_value(T(0));
         }
     __syncthreads();
     block_dot_parts(r, r, n, nrhs, part);
@@ -490,13 +480,6 @@ template rw_status spmv_launch<double>(rw_context*, int32_t, int64_t, const int3
 template rw_status spmv_launch<float>(rw_context*, int32_t, int64_t, const int32_t*, const int32_t*, const float*,
                                       const float*, float*, int);
 
-template <typename T>
-static rw_status fill_pending(rw_context* ctx, T* x, int64_t cnt) {
-    RW_COUNT_LAUNCH();
-    k_fill_pending<T><<<grid_for(cnt, 256, ctx->num_sms * 8), 256, 0, ctx->stream>>>(x, cnt);
-    return check_launch("fill");
-}
-
 // Device-time accumulation of the solve phases (events on the context stream).
 struct SolveTimes {
     bool on = false;
@@ -507,24 +490,14 @@ struct SolveTimes {
 // z = Y^-1 D^-1 Y^-T r; w: scratch [n, nrhs].  With timing, events 5/6/7
 // bracket the two solves (read by the caller).
 template <typename T>
-static const T* thin_values(const SolveSchedule& S);
-template <>
-const double* thin_values<double>(const SolveSchedule& S) { return S.tval; }
-template <>
-const float* thin_values<float>(const SolveSchedule& S) { return S.tval32; }
-
-template <typename T>
 static rw_status precond_t(rw_context* ctx, const FactorView& F, const T* yv, const T* ytv,
                            const T* d, const T* r, T* w, T* z, int nrhs, SolveTimes* tm = nullptr) {
     NvtxRange nvtx_range("rw_precond");
     if (tm && tm->on) cudaEventRecord(ctx->ev[5], ctx->stream);
-    rw_status rc = solve_runs<T>(ctx, *F.bwd_sched, F.yt_rp, F.yt_col, ytv,
-                                 thin_values<T>(*F.bwd_sched), r, nullptr, w, nrhs, F.bar, true);
+    rw_status rc = solve_runs<T>(ctx, *F.bwd_sched, F.yt_rp, F.yt_col, ytv, r, w, nrhs, F.bar, true);
     if (rc) return rc;
     if (tm && tm->on) cudaEventRecord(ctx->ev[6], ctx->stream);
-    if ((rc = apply_inverse_diag<T>(ctx, w, d, F.n, nrhs))) return rc;
-    rc = solve_runs<T>(ctx, *F.fwd_sched, F.y_rp, F.y_col, yv, thin_values<T>(*F.fwd_sched), w, nullptr,
-                       z, nrhs, F.bar);
+    rc = solve_runs<T>(ctx, *F.fwd_sched, F.y_rp, F.y_col, yv, w, z, nrhs, F.bar, false, w, d);
     if (tm && tm->on) {
         cudaEventRecord(ctx->ev[7], ctx->stream);
         tm->pending_pre = true;
@@ -562,8 +535,6 @@ rw_status precond_fp64(rw_context* ctx, const FactorView& F, const double* r, do
     double* w = alloc_n<double>(scratch, cnt);
     if (!w) return RW_ERR_ALLOC;
     rw_status rc;
-    if ((rc = fill_pending(ctx, w, cnt))) return rc;
-    if ((rc = fill_pending(ctx, z, cnt))) return rc;
     if ((rc = precond_t<double>(ctx, F, F.y_val, F.yt_val, F.d, r, w, z, nrhs))) return rc;
     return read_status(ctx, "preconditioner");
 }
@@ -601,8 +572,6 @@ static rw_status pcg_t(rw_context* ctx, const rw_csr* A, const FactorView& F, co
     RW_COUNT_LAUNCH();
     k_scalars<<<1, 256, 0, s>>>(S, part, vb, nrhs, kOpBnorm, tol, 0);
     if ((rc = check_launch("pcg init"))) return rc;
-    if ((rc = fill_pending(ctx, w, cnt))) return rc;
-    if ((rc = fill_pending(ctx, z, cnt))) return rc;
     SolveTimes tm;
     tm.on = ctx->opt.timing != 0;
     if ((rc = precond_t<T>(ctx, F, yv, ytv, dv, r, w, z, nrhs, &tm))) return rc;
@@ -635,7 +604,7 @@ static rw_status pcg_t(rw_context* ctx, const rw_csr* A, const FactorView& F, co
         RW_COUNT_LAUNCH();
         k_scalars<<<1, 256, 0, s>>>(S, part, sb, nrhs, kOpAlpha, tol, it);
         RW_COUNT_LAUNCH();
-        k_update_xr<T><<<vb, 256, 0, s>>>(n, nrhs, S, x, r, p, q, w, z, part);
+        k_update_xr<T><<<vb, 256, 0, s>>>(n, nrhs, S, x, r, p, q, part);
         if (mixed && it % refine == 0) {
             RW_COUNT_LAUNCH();
             k_true_resid<T><<<vb, 256, 0, s>>>(n, A->row_ptr, A->col, A->val, b, x, nrhs, r, part);
@@ -999,9 +968,7 @@ extern "C" rw_status rw_precond_apply_static(rw_context* ctx, const rw_factor* F
     v.bwd_sched = &F->bwd_sched;
     v.bar = F->bar;
     if ((rc = reset_status(ctx))) return rc;
-    // w and z start as "pending" on every call: the array keeps the last call's contents
-    if ((rc = fill_pending(ctx, w, cnt))) return rc;
-    if ((rc = fill_pending(ctx, d_z, cnt))) return rc;
+    // (the solve marks w and z pending on every call: the array keeps the last call's contents)
     if ((rc = precond_t<double>(ctx, v, v.y_val, v.yt_val, v.d, d_r, w, d_z, nrhs))) return rc;
     return read_status(ctx, "static-scratch preconditioner");
 }

@@ -26,9 +26,7 @@ namespace {
 struct Candidate {
     int wide_slices, solve_blocks_per_sm, cluster_width, spmv_slices, solve_mode;
     int solve_mode_bwd = -1;  // -1: as solve_mode
-    int thin_cluster = 0;
-    int thin_flags = 0;
-    int thin_lanes = 0;
+    int thin_cluster = 0, thin_flags = 0, thin_lanes = 0;  // without effect: options and cache lines that hold them
 };
 
 std::string shape_key(const rw_context* ctx, const TuneTarget& T, int nrhs) {
@@ -95,14 +93,13 @@ void cache_store(const char* path, const std::string& key, const Candidate& c, f
 
 template <typename T>
 rw_status time_precond(rw_context* ctx, const TuneTarget& X, const T* yv, const T* ytv, const T* dv,
-                       const T* tvf, const T* tvb, const T* r, T* w, T* z, int nrhs, int reps, float* ms) {
+                       const T* r, T* w, T* z, int nrhs, int reps, float* ms) {
     cudaStream_t s = ctx->stream;
     rw_status rc;
     auto once = [&]() -> rw_status {
-        rw_status r2 = solve_runs<T>(ctx, *X.bwd, X.yt_rp, X.yt_col, ytv, tvb, r, nullptr, w, nrhs, X.bar, true);
+        rw_status r2 = solve_runs<T>(ctx, *X.bwd, X.yt_rp, X.yt_col, ytv, r, w, nrhs, X.bar, true);
         if (r2) return r2;
-        if ((r2 = apply_inverse_diag<T>(ctx, w, dv, X.fwd->n, nrhs))) return r2;
-        return solve_runs<T>(ctx, *X.fwd, X.y_rp, X.y_col, yv, tvf, w, nullptr, z, nrhs, X.bar);
+        return solve_runs<T>(ctx, *X.fwd, X.y_rp, X.y_col, yv, w, z, nrhs, X.bar, false, w, dv);
     };
     if ((rc = once())) return rc;
     cudaEventRecord(ctx->ev[10], s);
@@ -139,7 +136,7 @@ __global__ void k_tune_fill(T* v, int64_t cnt) {
 
 template <typename T>
 rw_status tune_t(rw_context* ctx, const TuneTarget& X, int nrhs, const T* av, const T* yv, const T* ytv,
-                 const T* dv, const T* tvf, const T* tvb, Candidate* best, float* best_pre, float* best_spmv) {
+                 const T* dv, Candidate* best, float* best_pre, float* best_spmv) {
     Pool sc(ctx);
     const int64_t cnt = (int64_t)X.n * nrhs;
     T* r = alloc_n<T>(sc, cnt);
@@ -170,29 +167,10 @@ rw_status tune_t(rw_context* ctx, const TuneTarget& X, int nrhs, const T* av, co
     cands.push_back(Candidate{-1, 1, 0, 0, 1});                            // sync-free, vector rows
     cands.push_back(Candidate{-1, 1, 0, 0, 1, 0});  // sync-free forward, level-scheduled backward
     cands.push_back(Candidate{-1, 1, 0, 0, 0, 1});  // level-scheduled forward, sync-free backward
-    cands.push_back(Candidate{-1, 1, 0, 0, 2});     // hybrid runs (thin: one block; wide: sync-free)
-    cands.push_back(Candidate{-1, 2, 0, 0, 2});     // hybrid, sync-free parts with two blocks per SM
-    cands.push_back(Candidate{-1, 1, 0, 0, 1, 2});  // sync-free forward, hybrid backward
-    for (int tc : {4, 8}) {                          // hybrid with thin runs on clusters
-        Candidate c{-1, 1, 0, 0, 2};
-        c.thin_cluster = tc;
-        cands.push_back(c);
-    }
-    for (int bps : {1, 2}) {                         // hybrid, thin runs with ready flags
-        Candidate c{-1, bps, 0, 0, 2};
-        c.thin_flags = 1;
-        cands.push_back(c);
-    }
-    for (int tl : {8, 16}) {                         // hybrid, thin runs with lane groups
-        if (tl < nr) continue;
-        for (int bps : {1, 2})
-            for (int fl : {0, 1}) {
-                Candidate c{-1, bps, 0, 0, 2};
-                c.thin_lanes = tl;
-                c.thin_flags = fl;
-                cands.push_back(c);
-            }
-    }
+    cands.push_back(Candidate{-1, 1, 0, 0, 2});     // blocks of narrow levels
+    cands.push_back(Candidate{-1, 2, 0, 0, 2});     // the same, two blocks per SM
+    cands.push_back(Candidate{slices[0], 1, 0, 0, 2});  // the same, lane groups
+    cands.push_back(Candidate{-1, 1, 0, 0, 1, 2});  // sync-free forward, blocks backward
     for (const Candidate& c : cands) {
         ctx->opt.solve_mode = c.solve_mode;
         ctx->opt.solve_mode_bwd = c.solve_mode_bwd;
@@ -203,7 +181,7 @@ rw_status tune_t(rw_context* ctx, const TuneTarget& X, int nrhs, const T* av, co
         ctx->opt.solve_blocks_per_sm = c.solve_blocks_per_sm;
         ctx->opt.cluster_width = c.cluster_width;
         float ms = 0.f;
-        if ((rc = time_precond<T>(ctx, X, yv, ytv, dv, tvf, tvb, r, w, z, nrhs, reps, &ms))) {
+        if ((rc = time_precond<T>(ctx, X, yv, ytv, dv, r, w, z, nrhs, reps, &ms))) {
             ctx->opt = saved;
             return rc;
         }
@@ -248,11 +226,9 @@ rw_status autotune(rw_context* ctx, const TuneTarget& X, int nrhs, rw_precision 
     if (!cache_lookup(cache, key, &c)) {
         rw_status rc;
         if (prec == RW_FP32_MIXED) {
-            rc = tune_t<float>(ctx, X, nrhs, X.a_val32, X.y_val32, X.yt_val32, X.d32, X.fwd->tval32, X.bwd->tval32, &c,
-                               &ms_pre, &ms_spmv);
+            rc = tune_t<float>(ctx, X, nrhs, X.a_val32, X.y_val32, X.yt_val32, X.d32, &c, &ms_pre, &ms_spmv);
         } else {
-            rc = tune_t<double>(ctx, X, nrhs, X.a_val, X.y_val, X.yt_val, X.d, X.fwd->tval, X.bwd->tval, &c,
-                                &ms_pre, &ms_spmv);
+            rc = tune_t<double>(ctx, X, nrhs, X.a_val, X.y_val, X.yt_val, X.d, &c, &ms_pre, &ms_spmv);
         }
         if (rc) return rc;
         cache_store(cache, key, c, ms_pre, ms_spmv);
