@@ -49,11 +49,14 @@ constexpr int kSpmvEntries = 2048;  // entries of a pass (24 KB of columns and F
 constexpr int kSpmvRows = 512;      // rows of a pass
 constexpr int kLongRow = 64;
 
-template <typename TA, typename TV, int NR, int ES, bool DIFF>
+// RES: the true residual b - A x of PCG instead of A x: stored as FP32
+// (out32) or FP64 where y is given, its squares in place of the dot products.
+template <typename TA, typename TV, int NR, int ES, bool DIFF, bool RES>
 __global__ void __launch_bounds__(256) k_spmv(int32_t n, const int32_t* __restrict__ rp,
                                               const int32_t* __restrict__ col,
                                               const TA* __restrict__ val, const TV* __restrict__ x,
-                                              TV* __restrict__ y, int nrhs, int rows_per_pass, double* part) {
+                                              TV* __restrict__ y, int nrhs, int rows_per_pass, double* part,
+                                              const double* __restrict__ b, int out32) {
     constexpr int G = NR * ES;
     static_assert(G <= 32 && 32 % G == 0, "lane group");
     __shared__ __align__(16) TA sval[kSpmvEntries];
@@ -67,6 +70,18 @@ __global__ void __launch_bounds__(256) k_spmv(int32_t n, const int32_t* __restri
         const TV xc = x[(size_t)c * nrhs + j];
         if (DIFF) return c == row ? a * xi : a * (xc - xi);
         return a * xc;
+    };
+    // the row's sum is complete: stores it, adds its part of the dot product
+    auto finish = [&](size_t at, TV acc, double& dot) {
+        if constexpr (RES) {
+            const double t = b[at] - (double)acc;
+            if (y && out32) reinterpret_cast<float*>(y)[at] = (float)t;
+            else if (y) y[at] = (TV)t;
+            dot += t * t;
+        } else {
+            y[at] = acc;
+            if (part) dot += (double)x[at] * (double)acc;
+        }
     };
     const int64_t npass = ((int64_t)n + rows_per_pass - 1) / rows_per_pass;
     for (int64_t ps = blockIdx.x; ps < npass; ps += gridDim.x) {
@@ -117,11 +132,7 @@ __global__ void __launch_bounds__(256) k_spmv(int32_t n, const int32_t* __restri
 #pragma unroll
                     for (int o = NR; o < G; o <<= 1) acc += __shfl_xor_sync(kFull, acc, o);
                 }
-                if (r < nr && jok && es == 0) {
-                    const size_t at = (size_t)(base + r) * nrhs + j;
-                    y[at] = acc;
-                    if (part) mydot += (double)x[at] * (double)acc;
-                }
+                if (r < nr && jok && es == 0) finish((size_t)(base + r) * nrhs + j, acc, mydot);
             }
         } else {
             constexpr int EW = 32 / NR;
@@ -135,11 +146,7 @@ __global__ void __launch_bounds__(256) k_spmv(int32_t n, const int32_t* __restri
                     for (int32_t p = srp[r] + es; p < srp[r + 1]; p += EW) acc += term(col[p], val[p], row, j, xi);
 #pragma unroll
                 for (int o = NR; o < 32; o <<= 1) acc += __shfl_xor_sync(kFull, acc, o);
-                if (es == 0 && jok) {
-                    const size_t at = (size_t)row * nrhs + j;
-                    y[at] = acc;
-                    if (part) wdot += (double)x[at] * (double)acc;
-                }
+                if (es == 0 && jok) finish((size_t)row * nrhs + j, acc, wdot);
             }
         }
         __syncthreads();
@@ -201,30 +208,50 @@ struct PcgScalars {
     int pad;
 };
 
-// Deterministic reduction of per-block partials: part[b * NR + j].
-__device__ double reduce_parts(const double* part, int nparts, int j) {
+// Threads of a block that work on an [n][nrhs] array element by element, each
+// on one right-hand side (tid % nrhs): whole groups of nrhs threads.
+__device__ __forceinline__ int rhs_threads(int nrhs) { return 256 / nrhs * nrhs; }
+
+// Sum of v over the block's rhs_threads, per right-hand side, in a fixed order;
+// threads j < nrhs hold the sums.
+__device__ __forceinline__ double block_rhs_sum(double v, int nrhs) {
     __shared__ double red[256];
-    double s = 0.0;
-    for (int b = threadIdx.x; b < nparts; b += blockDim.x) s += part[(size_t)b * 16 + j];
-    red[threadIdx.x] = s;
+    const int tid = (int)threadIdx.x, groups = 256 / nrhs, g = tid / nrhs;
+    red[tid] = v;
     __syncthreads();
-    for (int w = blockDim.x / 2; w > 0; w >>= 1) {
-        if ((int)threadIdx.x < w) red[threadIdx.x] += red[threadIdx.x + w];
+    int w = 1;
+    while (w < groups) w <<= 1;
+    for (w >>= 1; w > 0; w >>= 1) {
+        if (g < w && g + w < groups) red[tid] += red[tid + w * nrhs];
         __syncthreads();
     }
-    const double r = red[0];
+    const double r = red[tid];
     __syncthreads();
     return r;
 }
 
 enum ScalarOp { kOpBnorm = 0, kOpRho0, kOpAlpha, kOpResid, kOpTrue, kOpBeta, kOpReport };
 
-// One block of 256 threads.  part: [kDotParts][16].
-__global__ void __launch_bounds__(256) k_scalars(PcgScalars* S, const double* part, int nparts,
-                                                 int nrhs, int op, double tol, int it) {
-    for (int j = 0; j < nrhs; ++j) {
-        const double v = reduce_parts(part, nparts, j);
-        if (threadIdx.x != 0) continue;
+// One block of 1024 threads: the partials part[nparts][16] of all right-hand
+// sides in one round of loads (a thread takes partials b, b + 64, ... of one),
+// then a fixed tree, then the step of Algorithm 1 by one thread each.  (Summed
+// one right-hand side after the other the kernel took 10 us of every step.)
+__global__ void __launch_bounds__(1024) k_scalars(PcgScalars* S, const double* part, int nparts,
+                                                  int nrhs, int op, double tol, int it) {
+    __shared__ double red[1024];
+    const int tid = (int)threadIdx.x;
+    double sum = 0.0;
+    if (tid % 16 < nrhs)
+        for (int b = tid / 16; b < nparts; b += 64) sum += part[(size_t)b * 16 + tid % 16];
+    red[tid] = sum;
+    __syncthreads();
+    for (int w = 32; w > 0; w >>= 1) {
+        if (tid < w * 16) red[tid] += red[tid + w * 16];
+        __syncthreads();
+    }
+    if (tid < nrhs) {
+        const int j = tid;
+        const double v = red[j];
         switch (op) {
             case kOpBnorm:
                 S->bnorm2[j] = v;
@@ -268,7 +295,8 @@ __global__ void __launch_bounds__(256) k_scalars(PcgScalars* S, const double* pa
                 break;
         }
     }
-    if (threadIdx.x == 0) {
+    __syncthreads();
+    if (tid == 0) {
         int a = 0, c = 0;
         for (int j = 0; j < nrhs; ++j) {
             a |= S->active[j];
@@ -281,101 +309,64 @@ __global__ void __launch_bounds__(256) k_scalars(PcgScalars* S, const double* pa
     }
 }
 
-// Fixed-order block sum of one value per (thread, right-hand side j < 16):
-// warp sums, then the warps' sums in warp order, into part[blockIdx][j].
-__device__ __forceinline__ void block_parts16(double (&acc)[16], double* part) {
-    __shared__ double ws[8][16];
-#pragma unroll
-    for (int j = 0; j < 16; ++j) acc[j] = warp_sum(acc[j]);
-    if (lane_id() == 0)
-#pragma unroll
-        for (int j = 0; j < 16; ++j) ws[threadIdx.x >> 5][j] = acc[j];
-    __syncthreads();
-    if (threadIdx.x < 16) {
-        double t = 0.0;
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += ws[w][threadIdx.x];
-        part[(size_t)blockIdx.x * 16 + threadIdx.x] = t;
+// The vector kernels of PCG work element by element over the node-major arrays
+// (coalesced; a thread keeps one right-hand side, so its scalar and its one
+// accumulator stay in registers) and are bound by memory: with a thread per node
+// and accumulators for sixteen right-hand sides, reduced one after the other on
+// the FP64 pipe, a dot product of 261,568 entries took 49 us and now takes 5.
+template <typename F>
+__device__ __forceinline__ void for_elements(int64_t n, int nrhs, F f) {
+    const int t = rhs_threads(nrhs);
+    if ((int)threadIdx.x >= t) return;
+    const int64_t cnt = n * nrhs, step = (int64_t)gridDim.x * t;
+    for (int64_t i = (int64_t)blockIdx.x * t + threadIdx.x; i < cnt; i += step) f(i);
+}
+
+// Per-block partial sums of a.b (and with a2 given a2.b2) per right-hand side
+// into part[blockIdx][j] (and part2).
+template <typename TA, typename TB>
+__global__ void __launch_bounds__(256) k_dot(const TA* __restrict__ a, const TB* __restrict__ b, int64_t n, int nrhs,
+                                             double* part, const TA* __restrict__ a2, const TB* __restrict__ b2,
+                                             double* part2) {
+    double acc = 0.0, acc2 = 0.0;
+    for_elements(n, nrhs, [&](int64_t i) {
+        acc += (double)a[i] * (double)b[i];
+        if (a2) acc2 += (double)a2[i] * (double)b2[i];
+    });
+    const double s = block_rhs_sum(acc, nrhs);
+    if ((int)threadIdx.x < nrhs) part[(size_t)blockIdx.x * 16 + threadIdx.x] = s;
+    if (a2) {
+        const double s2 = block_rhs_sum(acc2, nrhs);
+        if ((int)threadIdx.x < nrhs) part2[(size_t)blockIdx.x * 16 + threadIdx.x] = s2;
     }
-}
-
-// Block-level partial sums of a.b per right-hand side into part[blockIdx][j].
-template <typename TA, typename TB>
-__device__ void block_dot_parts(const TA* a, const TB* b, int64_t n, int nrhs, double* part) {
-    double acc[16];
-    for (int j = 0; j < 16; ++j) acc[j] = 0.0;
-    // thread handles whole nodes so that each accumulator belongs to one rhs
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-         i += (int64_t)gridDim.x * blockDim.x)
-        for (int j = 0; j < nrhs; ++j)
-            acc[j] += (double)a[i * nrhs + j] * (double)b[i * nrhs + j];
-    block_parts16(acc, part);
-}
-
-template <typename TA, typename TB>
-__global__ void __launch_bounds__(256) k_dot(const TA* a, const TB* b, int64_t n, int nrhs,
-                                             double* part) {
-    block_dot_parts(a, b, n, nrhs, part);
 }
 
 // x += alpha p (x FP64), r -= alpha q; partial r.r.
 template <typename T>
-__global__ void __launch_bounds__(256) k_update_xr(int64_t n, int nrhs, const PcgScalars* S,
-                                                   double* x, T* r, const T* p, const T* q, double* part) {
-    __shared__ double al[16];
-    if (threadIdx.x < 16) al[threadIdx.x] = threadIdx.x < (unsigned)nrhs ? S->alpha[threadIdx.x] : 0.0;
-    __syncthreads();
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-         i += (int64_t)gridDim.x * blockDim.x)
-        for (int j = 0; j < nrhs; ++j) {
-            const size_t o = (size_t)i * nrhs + j;
-            const double a = al[j];
-            if (a != 0.0) {
-                x[o] += a * (double)p[o];
-                r[o] = (T)((double)r[o] - a * (double)q[o]);
-            }
+__global__ void __launch_bounds__(256) k_update_xr(int64_t n, int nrhs, const PcgScalars* S, double* __restrict__ x,
+                                                   T* __restrict__ r, const T* __restrict__ p,
+                                                   const T* __restrict__ q, double* part) {
+    const double a = S->alpha[threadIdx.x % nrhs];
+    double acc = 0.0;
+    for_elements(n, nrhs, [&](int64_t i) {
+        T ri = r[i];
+        if (a != 0.0) {
+            x[i] += a * (double)p[i];
+            ri = (T)((double)ri - a * (double)q[i]);
+            r[i] = ri;
         }
-    __syncthreads();
-    block_dot_parts(r, r, n, nrhs, part);
+        acc += (double)ri * (double)ri;
+    });
+    const double s = block_rhs_sum(acc, nrhs);
+    if ((int)threadIdx.x < nrhs) part[(size_t)blockIdx.x * 16 + threadIdx.x] = s;
 }
 
 // p = z + beta p
 template <typename T>
-__global__ void __launch_bounds__(256) k_update_p(int64_t n, int nrhs, const PcgScalars* S,
-                                                  const T* z, T* p) {
-    __shared__ double be[16];
-    if (threadIdx.x < 16) be[threadIdx.x] = threadIdx.x < (unsigned)nrhs ? S->beta[threadIdx.x] : 0.0;
-    __syncthreads();
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-         i += (int64_t)gridDim.x * blockDim.x)
-        for (int j = 0; j < nrhs; ++j) {
-            const size_t o = (size_t)i * nrhs + j;
-            p[o] = (T)((double)z[o] + be[j] * (double)p[o]);
-        }
-}
-
-// t = b - A x in FP64 (true residual), optionally stored to r (residual
-// replacement) in T; partial t.t.
-template <typename T>
-__global__ void __launch_bounds__(256) k_true_resid(int32_t n, const int32_t* __restrict__ rp,
-                                                    const int32_t* __restrict__ col,
-                                                    const double* __restrict__ val,
-                                                    const double* __restrict__ b,
-                                                    const double* __restrict__ x, int nrhs,
-                                                    T* r_out, double* part) {
-    double acc2[16];
-    for (int j = 0; j < 16; ++j) acc2[j] = 0.0;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        const int32_t s = rp[i], e = rp[i + 1];
-        for (int j = 0; j < nrhs; ++j) {
-            double ax = 0.0;
-            for (int32_t p = s; p < e; ++p) ax += val[p] * x[(size_t)col[p] * nrhs + j];
-            const double t = b[(size_t)i * nrhs + j] - ax;
-            if (r_out) r_out[(size_t)i * nrhs + j] = (T)t;
-            acc2[j] += t * t;
-        }
-    }
-    block_parts16(acc2, part);
+__global__ void __launch_bounds__(256) k_update_p(int64_t n, int nrhs, const PcgScalars* S, const T* __restrict__ z,
+                                                  T* __restrict__ p) {
+    const double be = S->beta[threadIdx.x % nrhs];
+    for_elements(n, nrhs, [&](int64_t i) { p[i] = (T)((double)z[i] + be * (double)p[i]); });
 }
 
 template <typename Tin, typename Tout>
@@ -400,9 +391,10 @@ static int pow2_at_least(int v) {
     return p;
 }
 
-template <typename TA, typename TV, int NR, int ES>
+template <typename TA, typename TV, int NR, int ES, bool RES>
 static void launch_spmv_es(const rw_context* ctx, int32_t n, int64_t nnz, const int32_t* rp, const int32_t* col,
-                           const TA* val, const TV* x, TV* y, int nrhs, double* part, int* blocks_out, cudaStream_t s) {
+                           const TA* val, const TV* x, TV* y, int nrhs, double* part, int* blocks_out, cudaStream_t s,
+                           const double* b, int out32) {
     if constexpr (NR * ES <= 32) {
         // rows of a pass: as many as the copy holds with a tenth to spare, in whole sets of row groups
         const int set = 256 / (ES == 1 ? nrhs : NR * ES);
@@ -414,7 +406,7 @@ static void launch_spmv_es(const rw_context* ctx, int32_t n, int64_t nnz, const 
         const int64_t passes = ((int64_t)n + rows - 1) / rows;
         static int per_sm = 0;
         if (per_sm < 1) {
-            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_spmv<TA, TV, NR, ES, sizeof(TA) == 4>, 256, 0);
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_spmv<TA, TV, NR, ES, sizeof(TA) == 4, RES>, 256, 0);
             if (per_sm < 1) per_sm = 1;
         }
         int blocks = grid_for(passes, 1, ctx->num_sms * per_sm);
@@ -422,7 +414,8 @@ static void launch_spmv_es(const rw_context* ctx, int32_t n, int64_t nnz, const 
         if (blocks_out) *blocks_out = blocks;
         RW_COUNT_LAUNCH();
         // FP32 values are always the excess + difference form of the mixed mode
-        k_spmv<TA, TV, NR, ES, sizeof(TA) == 4><<<blocks, 256, 0, s>>>(n, rp, col, val, x, y, nrhs, rows, part);
+        k_spmv<TA, TV, NR, ES, sizeof(TA) == 4, RES>
+            <<<blocks, 256, 0, s>>>(n, rp, col, val, x, y, nrhs, rows, part, b, out32);
     }
 }
 
@@ -430,9 +423,10 @@ static void launch_spmv_es(const rw_context* ctx, int32_t n, int64_t nnz, const 
 // block's threads hold at once fit the copy (27 entries a row and one
 // right-hand side: four slices; nine: one), and while the rows' lanes do not
 // fill the chip.
-template <typename TA, typename TV, int NR>
+template <typename TA, typename TV, int NR, bool RES>
 static void launch_spmv_nr(const rw_context* ctx, int32_t n, int64_t nnz, const int32_t* rp, const int32_t* col,
-                           const TA* val, const TV* x, TV* y, int nrhs, double* part, int* blocks, cudaStream_t s) {
+                           const TA* val, const TV* x, TV* y, int nrhs, double* part, int* blocks, cudaStream_t s,
+                           const double* b, int out32) {
     int p = 1;
     if (ctx->opt.spmv_slices > 0) {
         while (p * 2 <= ctx->opt.spmv_slices && p * 2 * NR <= 32) p *= 2;
@@ -443,28 +437,29 @@ static void launch_spmv_nr(const rw_context* ctx, int32_t n, int64_t nnz, const 
             p *= 2;
     }
     switch (p) {
-        case 1: launch_spmv_es<TA, TV, NR, 1>(ctx, n, nnz, rp, col, val, x, y, nrhs, part, blocks, s); break;
-        case 2: launch_spmv_es<TA, TV, NR, 2>(ctx, n, nnz, rp, col, val, x, y, nrhs, part, blocks, s); break;
-        case 4: launch_spmv_es<TA, TV, NR, 4>(ctx, n, nnz, rp, col, val, x, y, nrhs, part, blocks, s); break;
-        case 8: launch_spmv_es<TA, TV, NR, 8>(ctx, n, nnz, rp, col, val, x, y, nrhs, part, blocks, s); break;
-        case 16: launch_spmv_es<TA, TV, NR, 16>(ctx, n, nnz, rp, col, val, x, y, nrhs, part, blocks, s); break;
-        default: launch_spmv_es<TA, TV, NR, 32>(ctx, n, nnz, rp, col, val, x, y, nrhs, part, blocks, s); break;
+        case 1: launch_spmv_es<TA, TV, NR, 1, RES>(ctx, n, nnz, rp, col, val, x, y, nrhs, part, blocks, s, b, out32); break;
+        case 2: launch_spmv_es<TA, TV, NR, 2, RES>(ctx, n, nnz, rp, col, val, x, y, nrhs, part, blocks, s, b, out32); break;
+        case 4: launch_spmv_es<TA, TV, NR, 4, RES>(ctx, n, nnz, rp, col, val, x, y, nrhs, part, blocks, s, b, out32); break;
+        case 8: launch_spmv_es<TA, TV, NR, 8, RES>(ctx, n, nnz, rp, col, val, x, y, nrhs, part, blocks, s, b, out32); break;
+        case 16: launch_spmv_es<TA, TV, NR, 16, RES>(ctx, n, nnz, rp, col, val, x, y, nrhs, part, blocks, s, b, out32); break;
+        default: launch_spmv_es<TA, TV, NR, 32, RES>(ctx, n, nnz, rp, col, val, x, y, nrhs, part, blocks, s, b, out32); break;
     }
 }
 
 // part: per-block dot products x.y of the right-hand sides ([blocks][16], at
 // most kDotParts blocks; *blocks receives their number).
-template <typename TA, typename TV>
+template <typename TA, typename TV, bool RES = false>
 static rw_status launch_spmv(rw_context* ctx, int32_t n, int64_t nnz, const int32_t* rp, const int32_t* col,
-                             const TA* val, const TV* x, TV* y, int nrhs, double* part, int* blocks = nullptr) {
+                             const TA* val, const TV* x, TV* y, int nrhs, double* part, int* blocks = nullptr,
+                             const double* b = nullptr, int out32 = 0) {
     cudaStream_t s = ctx->stream;
     const int nr = pow2_at_least(nrhs);
     switch (nr) {
-        case 1: launch_spmv_nr<TA, TV, 1>(ctx, n, nnz, rp, col, val, x, y, nrhs, part, blocks, s); break;
-        case 2: launch_spmv_nr<TA, TV, 2>(ctx, n, nnz, rp, col, val, x, y, nrhs, part, blocks, s); break;
-        case 4: launch_spmv_nr<TA, TV, 4>(ctx, n, nnz, rp, col, val, x, y, nrhs, part, blocks, s); break;
-        case 8: launch_spmv_nr<TA, TV, 8>(ctx, n, nnz, rp, col, val, x, y, nrhs, part, blocks, s); break;
-        default: launch_spmv_nr<TA, TV, 16>(ctx, n, nnz, rp, col, val, x, y, nrhs, part, blocks, s); break;
+        case 1: launch_spmv_nr<TA, TV, 1, RES>(ctx, n, nnz, rp, col, val, x, y, nrhs, part, blocks, s, b, out32); break;
+        case 2: launch_spmv_nr<TA, TV, 2, RES>(ctx, n, nnz, rp, col, val, x, y, nrhs, part, blocks, s, b, out32); break;
+        case 4: launch_spmv_nr<TA, TV, 4, RES>(ctx, n, nnz, rp, col, val, x, y, nrhs, part, blocks, s, b, out32); break;
+        case 8: launch_spmv_nr<TA, TV, 8, RES>(ctx, n, nnz, rp, col, val, x, y, nrhs, part, blocks, s, b, out32); break;
+        default: launch_spmv_nr<TA, TV, 16, RES>(ctx, n, nnz, rp, col, val, x, y, nrhs, part, blocks, s, b, out32); break;
     }
     return check_launch("spmv");
 }
@@ -557,28 +552,26 @@ static rw_status pcg_t(rw_context* ctx, const rw_csr* A, const FactorView& F, co
     PcgScalars* S = alloc_n<PcgScalars>(sc, 1);
     if (!r || !z || !p || !q || !w || !part || !S) return RW_ERR_ALLOC;
     PcgScalars* hS = static_cast<PcgScalars*>(ctx->h_small);
-    const int vb = grid_for(n, 256, kDotParts);
+    const int vb = grid_for(cnt, 1024, ctx->num_sms * 4);  // partial sums: four elements a thread and more
     rw_status rc;
     if ((rc = check_cuda(cudaMemsetAsync(S, 0, sizeof(PcgScalars), s), "memset"))) return rc;
     if ((rc = check_cuda(cudaMemsetAsync(x, 0, sizeof(double) * (size_t)cnt, s), "memset"))) return rc;
-    if ((rc = check_cuda(cudaMemsetAsync(part, 0, sizeof(double) * kDotParts * 16, s), "memset")))
-        return rc;
     RW_COUNT_LAUNCH();
     k_check_finite<<<vb, 256, 0, s>>>(b, cnt, ctx->d_status);
     RW_COUNT_LAUNCH();
     k_convert<double, T><<<vb, 256, 0, s>>>(b, r, cnt);
     RW_COUNT_LAUNCH();
-    k_dot<double, double><<<vb, 256, 0, s>>>(b, b, n, nrhs, part);
+    k_dot<double, double><<<vb, 256, 0, s>>>(b, b, n, nrhs, part, nullptr, nullptr, nullptr);
     RW_COUNT_LAUNCH();
-    k_scalars<<<1, 256, 0, s>>>(S, part, vb, nrhs, kOpBnorm, tol, 0);
+    k_scalars<<<1, 1024, 0, s>>>(S, part, vb, nrhs, kOpBnorm, tol, 0);
     if ((rc = check_launch("pcg init"))) return rc;
     SolveTimes tm;
     tm.on = ctx->opt.timing != 0;
     if ((rc = precond_t<T>(ctx, F, yv, ytv, dv, r, w, z, nrhs, &tm))) return rc;
     RW_COUNT_LAUNCH();
-    k_dot<T, T><<<vb, 256, 0, s>>>(r, z, n, nrhs, part);
+    k_dot<T, T><<<vb, 256, 0, s>>>(r, z, n, nrhs, part, nullptr, nullptr, nullptr);
     RW_COUNT_LAUNCH();
-    k_scalars<<<1, 256, 0, s>>>(S, part, vb, nrhs, kOpRho0, tol, 0);
+    k_scalars<<<1, 1024, 0, s>>>(S, part, vb, nrhs, kOpRho0, tol, 0);
     RW_COUNT_LAUNCH();
     k_convert<T, T><<<vb, 256, 0, s>>>(z, p, cnt);
     if ((rc = check_launch("pcg start"))) return rc;
@@ -589,6 +582,12 @@ static rw_status pcg_t(rw_context* ctx, const rw_csr* A, const FactorView& F, co
         set_error("pcg: right-hand side holds a non-finite value");
         return RW_ERR_ARG;
     }
+    // t = b - A x in FP64 (true residual), stored to out in T where given; partial t.t in *blocks blocks
+    auto true_resid = [&](T* out, int* blocks) -> rw_status {
+        return launch_spmv<double, double, true>(ctx, n, A->nnz, A->row_ptr, A->col, A->val, x,
+                                                 reinterpret_cast<double*>(out), nrhs, part, blocks, b,
+                                                 sizeof(T) == 4 ? 1 : 0);
+    };
     int done_iters = 0;
     const int refine = ctx->opt.refine_every > 0 ? ctx->opt.refine_every : 50;
     bool any_active = hS->any_active != 0;
@@ -602,15 +601,13 @@ static rw_status pcg_t(rw_context* ctx, const rw_csr* A, const FactorView& F, co
             tm.pending_spmv = true;
         }
         RW_COUNT_LAUNCH();
-        k_scalars<<<1, 256, 0, s>>>(S, part, sb, nrhs, kOpAlpha, tol, it);
+        k_scalars<<<1, 1024, 0, s>>>(S, part, sb, nrhs, kOpAlpha, tol, it);
         RW_COUNT_LAUNCH();
         k_update_xr<T><<<vb, 256, 0, s>>>(n, nrhs, S, x, r, p, q, part);
-        if (mixed && it % refine == 0) {
-            RW_COUNT_LAUNCH();
-            k_true_resid<T><<<vb, 256, 0, s>>>(n, A->row_ptr, A->col, A->val, b, x, nrhs, r, part);
-        }
+        int rb = vb;
+        if (mixed && it % refine == 0 && (rc = true_resid(r, &rb))) return rc;
         RW_COUNT_LAUNCH();
-        k_scalars<<<1, 256, 0, s>>>(S, part, vb, nrhs, kOpResid, tol, it);
+        k_scalars<<<1, 1024, 0, s>>>(S, part, rb, nrhs, kOpResid, tol, it);
         if ((rc = check_launch("pcg step"))) return rc;
         if ((rc = check_cuda(cudaMemcpyAsync(hS, S, sizeof(PcgScalars), cudaMemcpyDeviceToHost, s),
                              "copy")))
@@ -618,11 +615,10 @@ static rw_status pcg_t(rw_context* ctx, const rw_csr* A, const FactorView& F, co
         if ((rc = check_cuda(cudaStreamSynchronize(s), "sync"))) return rc;
         if (tm.on) collect_times(ctx, tm);
         if (hS->any_check) {
+            int tb = 0;
+            if ((rc = true_resid(nullptr, &tb))) return rc;
             RW_COUNT_LAUNCH();
-            k_true_resid<T><<<vb, 256, 0, s>>>(n, A->row_ptr, A->col, A->val, b, x, nrhs, nullptr,
-                                               part);
-            RW_COUNT_LAUNCH();
-            k_scalars<<<1, 256, 0, s>>>(S, part, vb, nrhs, kOpTrue, tol, it);
+            k_scalars<<<1, 1024, 0, s>>>(S, part, tb, nrhs, kOpTrue, tol, it);
             if ((rc = check_launch("pcg true residual"))) return rc;
             if ((rc = check_cuda(cudaMemcpyAsync(hS, S, sizeof(PcgScalars), cudaMemcpyDeviceToHost,
                                                  s),
@@ -634,18 +630,18 @@ static rw_status pcg_t(rw_context* ctx, const rw_csr* A, const FactorView& F, co
         if (hS->broke) break;
         if ((rc = precond_t<T>(ctx, F, yv, ytv, dv, r, w, z, nrhs, &tm))) return rc;
         RW_COUNT_LAUNCH();
-        k_dot<T, T><<<vb, 256, 0, s>>>(r, z, n, nrhs, part);
+        k_dot<T, T><<<vb, 256, 0, s>>>(r, z, n, nrhs, part, nullptr, nullptr, nullptr);
         RW_COUNT_LAUNCH();
-        k_scalars<<<1, 256, 0, s>>>(S, part, vb, nrhs, kOpBeta, tol, it);
+        k_scalars<<<1, 1024, 0, s>>>(S, part, vb, nrhs, kOpBeta, tol, it);
         RW_COUNT_LAUNCH();
         k_update_p<T><<<vb, 256, 0, s>>>(n, nrhs, S, z, p);
         if ((rc = check_launch("pcg direction"))) return rc;
     }
     // final true residuals for the report
+    int fb = 0;
+    if ((rc = true_resid(nullptr, &fb))) return rc;
     RW_COUNT_LAUNCH();
-    k_true_resid<T><<<vb, 256, 0, s>>>(n, A->row_ptr, A->col, A->val, b, x, nrhs, nullptr, part);
-    RW_COUNT_LAUNCH();
-    k_scalars<<<1, 256, 0, s>>>(S, part, vb, nrhs, kOpReport, tol, done_iters);
+    k_scalars<<<1, 1024, 0, s>>>(S, part, fb, nrhs, kOpReport, tol, done_iters);
     if ((rc = check_launch("pcg report"))) return rc;
     if ((rc = check_cuda(cudaMemcpyAsync(hS, S, sizeof(PcgScalars), cudaMemcpyDeviceToHost, s), "copy")))
         return rc;
@@ -733,12 +729,14 @@ __global__ void k_lin3(int64_t n, double* out, const double* a, double ca, const
     }
 }
 
-// One warp adds the block sums of right-hand side 0 in a fixed order.
-__global__ void k_sum_parts(const double* __restrict__ part, int nblocks, double* out) {
+// A warp per dot product adds its block sums of right-hand side 0 in a fixed order.
+__global__ void k_sum_parts(const double* __restrict__ part, const double* __restrict__ part2, int nblocks,
+                            double* out) {
+    const double* p = threadIdx.x < 32 ? part : part2;
     double t = 0.0;
-    for (int b = (int)lane_id(); b < nblocks; b += 32) t += part[(size_t)b * 16];
+    for (int b = (int)lane_id(); b < nblocks; b += 32) t += p[(size_t)b * 16];
     t = warp_sum(t);
-    if (lane_id() == 0) *out = t;
+    if (lane_id() == 0) out[threadIdx.x >> 5] = t;
 }
 
 rw_status bicgstab_run(rw_context* ctx, const rw_csr* A, const FactorView& F, const double* b, double* x, double tol,
@@ -756,25 +754,32 @@ rw_status bicgstab_run(rw_context* ctx, const rw_csr* A, const FactorView& F, co
     double* sh = alloc_n<double>(sc, n);
     double* t = alloc_n<double>(sc, n);
     double* w = alloc_n<double>(sc, n);
-    double* part = alloc_n<double>(sc, (int64_t)kDotParts * 16);
-    double* dres = alloc_n<double>(sc, 1);
+    double* part = alloc_n<double>(sc, (int64_t)kDotParts * 32);
+    double* const part2 = part + (int64_t)kDotParts * 16;
+    double* dres = alloc_n<double>(sc, 2);
     if (!r || !rh || !pv || !ph || !v || !sv || !sh || !t || !w || !part || !dres) return RW_ERR_ALLOC;
     double* hd = static_cast<double*>(ctx->h_small);
-    const int vb = grid_for(n, 256, kDotParts);
+    const int vb = grid_for(n, 1024, ctx->num_sms * 2);
     const int gb = grid_for(n, 256, ctx->num_sms * 8);
     rw_status rc;
-    auto dot = [&](const double* a, const double* c, double* out) -> rw_status {
+    // one or two dot products in one launch and one read back
+    auto dots = [&](const double* a, const double* c, double* out, const double* a2, const double* c2,
+                    double* out2) -> rw_status {
         RW_COUNT_LAUNCH();
-        k_dot<double, double><<<vb, 256, 0, s>>>(a, c, n, 1, part);
+        k_dot<double, double><<<vb, 256, 0, s>>>(a, c, n, 1, part, a2, c2, part2);
         RW_COUNT_LAUNCH();
-        k_sum_parts<<<1, 32, 0, s>>>(part, vb, dres);
+        k_sum_parts<<<1, a2 ? 64 : 32, 0, s>>>(part, part2, vb, dres);
         rw_status r2;
         if ((r2 = check_launch("bicgstab dot")) ||
-            (r2 = check_cuda(cudaMemcpyAsync(hd, dres, sizeof(double), cudaMemcpyDeviceToHost, s), "copy")) ||
+            (r2 = check_cuda(cudaMemcpyAsync(hd, dres, 2 * sizeof(double), cudaMemcpyDeviceToHost, s), "copy")) ||
             (r2 = check_cuda(cudaStreamSynchronize(s), "sync")))
             return r2;
         *out = hd[0];
+        if (a2) *out2 = hd[1];
         return RW_OK;
+    };
+    auto dot = [&](const double* a, const double* c, double* out) -> rw_status {
+        return dots(a, c, out, nullptr, nullptr, nullptr);
     };
     auto lin3 = [&](double* out, const double* a, double ca, const double* bb, double cb, const double* c,
                     double cc) -> rw_status {
@@ -805,6 +810,8 @@ rw_status bicgstab_run(rw_context* ctx, const rw_csr* A, const FactorView& F, co
     double rho_old = 1.0, alpha = 1.0, omega = 1.0, relres = bnorm > 0.0 ? 1.0 : 0.0;
     int it = 0;
     bool done = bnorm == 0.0, broke = false;
+    double rho_next = bb;  // rh . r for the next iteration (r = rh = b), if have_rho
+    bool have_rho = true;
     // the true residual b - A x into r; returns its relative norm
     auto true_residual = [&](double* rel) -> rw_status {
         rw_status r2;
@@ -815,8 +822,9 @@ rw_status bicgstab_run(rw_context* ctx, const rw_csr* A, const FactorView& F, co
     };
     while (!done && it < max_iter) {
         ++it;
-        double rho = 0.0, rv = 0.0;
-        if ((rc = dot(rh, r, &rho))) return rc;
+        double rho = rho_next, rv = 0.0;
+        if (!have_rho && (rc = dot(rh, r, &rho))) return rc;
+        have_rho = false;
         if (rho == 0.0 || !std::isfinite(rho)) {
             broke = true;
             break;
@@ -843,7 +851,8 @@ rw_status bicgstab_run(rw_context* ctx, const rw_csr* A, const FactorView& F, co
             continue;
         }
         double ts = 0.0, tt = 0.0;
-        if ((rc = apply_m(sv, sh)) || (rc = spmv(sh, t)) || (rc = dot(t, sv, &ts)) || (rc = dot(t, t, &tt))) return rc;
+        if ((rc = apply_m(sv, sh)) || (rc = spmv(sh, t)) || (rc = dots(t, sv, &ts, t, t, &tt)))
+            return rc;
         if (tt == 0.0 || !std::isfinite(tt)) {
             broke = true;
             break;
@@ -851,10 +860,12 @@ rw_status bicgstab_run(rw_context* ctx, const rw_csr* A, const FactorView& F, co
         omega = ts / tt;
         double rr = 0.0;
         if ((rc = lin3(x, x, 1.0, ph, alpha, sh, omega)) || (rc = lin3(r, sv, 1.0, t, -omega, nullptr, 0.0)) ||
-            (rc = dot(r, r, &rr)))
+            (rc = dots(r, r, &rr, rh, r, &rho_next)))
             return rc;
+        have_rho = true;
         relres = std::sqrt(rr) / bnorm;
         if (relres < tol) {
+            have_rho = false;  // (replaces r)
             if ((rc = true_residual(&relres))) return rc;
             if (relres < tol) done = true;
         }
