@@ -271,10 +271,13 @@ struct SolveRow {
     int32_t pad;
 };
 
-// Positions [pos0, pos1) solved together: as blocks, or (nblocks 0) row by row.
+// Positions [pos0, pos1) solved together: as blocks, or (nblocks 0) row by row
+// from slots [slot0, slot1) of the rows array; pack: levels padded to whole
+// groups of rows.
 struct SolveStretch {
-    int64_t pos0, pos1;
+    int64_t pos0, pos1, slot0, slot1;
     int32_t block0, nblocks;
+    bool pack;
 };
 
 // Block of a narrow stretch: positions [pos0, pos0 + rows); prev0: the first
@@ -299,7 +302,8 @@ struct SolveSchedule {
     const int32_t* order = nullptr;  // rows in level order
     const int64_t* lptr = nullptr;   // [depth + 1] level boundaries (device)
     std::vector<int64_t> lptr_h;     // host copy
-    SolveRow* rows = nullptr;        // [n] by position
+    int64_t nrows = 0;
+    SolveRow* rows = nullptr;        // [nrows] by position, packed stretches padded
     std::vector<SolveStretch> stretches;
     // blocks of the narrow stretches
     SolveBlock* blocks = nullptr;

@@ -49,6 +49,15 @@ constexpr int kNarrowLevels = 16;
 // of the 64^3 7-point grid: 2.3 against 1.2 ms of a 23 ms build).
 constexpr int kBlockRows = 256;
 
+// Rows of a wide level at least: with more rows than warps (16 on each of 152
+// SMs) a level takes several rounds, and a round of packed rows four at a time
+// (see k_rows_pack).  Below, a level is one round either way and a row is
+// faster with 32 lanes.
+constexpr int kWideRows = 2432;
+constexpr int kWideLevels = 4;  // levels of a packed stretch at least (a launch of its own)
+constexpr int kPackLanes = 8;
+constexpr int kPackRows = 32 / kPackLanes;
+
 __host__ __device__ __forceinline__ int64_t tri(int64_t m) { return m * (m + 1) / 2; }
 
 // ---------------------------------------------------------------------------
@@ -213,13 +222,21 @@ __global__ void __launch_bounds__(32) k_block_invert(const SolveBlock* __restric
     }
 }
 
-// Thread per position: its row as k_rows takes it.
-__global__ void k_fill_rows(int32_t n, const int32_t* __restrict__ order, const int32_t* __restrict__ last,
-                            const int64_t* __restrict__ rp, SolveRow* rows) {
+// Thread per position: its row as the row solves take it, in the slot of its
+// level (padding slots stay all ones: no row, no entries).
+__global__ void k_fill_rows(int32_t n, int32_t depth, const int64_t* __restrict__ lptr,
+                            const int64_t* __restrict__ slot0, const int32_t* __restrict__ order,
+                            const int32_t* __restrict__ last, const int64_t* __restrict__ rp, SolveRow* rows) {
     for (int32_t p = blockIdx.x * blockDim.x + threadIdx.x; p < n; p += gridDim.x * blockDim.x) {
+        int lo = 0, hi = depth - 1;  // the level of position p
+        while (lo < hi) {
+            const int mid = (lo + hi + 1) >> 1;
+            if (lptr[mid] <= p) lo = mid;
+            else hi = mid - 1;
+        }
         const int32_t row = order[p];
         const int64_t s = rp[row];
-        rows[p] = SolveRow{s, (int32_t)(rp[row + 1] - s), row, last[row], 0};
+        rows[slot0[lo] + (p - lptr[lo])] = SolveRow{s, (int32_t)(rp[row + 1] - s), row, last[row], 0};
     }
 }
 
@@ -242,36 +259,65 @@ rw_status build_schedule(rw_context* ctx, int32_t n, const int64_t* rp, const in
                          "copy")))
         return rc;
     if ((rc = check_cuda(cudaStreamSynchronize(s), "sync"))) return rc;
-    // stretches: narrow ones as blocks, the rows between them row by row
+    // stretches: narrow ones as blocks, the others row by row, the widest levels packed
     std::vector<SolveBlock> blocks;
-    int64_t pos = 0;
-    auto rows_until = [&](int64_t end) {
-        if (end > pos) S.stretches.push_back(SolveStretch{pos, end, 0, 0});
-        pos = end;
+    std::vector<int64_t> slot0((size_t)depth);  // of each level in the rows array
+    int64_t slots = 0;
+    auto kind_of = [&](int32_t l) {
+        const int64_t w = S.lptr_h[l + 1] - S.lptr_h[l];
+        return w <= kNarrow ? 0 : w < kWideRows ? 1 : 2;
     };
     for (int32_t l = 0; l < depth;) {
-        int32_t e = l;
-        while (e < depth && S.lptr_h[e + 1] - S.lptr_h[e] <= kNarrow) ++e;
-        if (e - l >= kNarrowLevels) {
-            rows_until(S.lptr_h[l]);
-            SolveStretch st{pos, S.lptr_h[e], (int32_t)blocks.size(), 0};
-            for (int64_t prev = pos; pos < st.pos1;) {
+        // the longest stretch of one kind; one too short for a launch of its own joins the row by row levels
+        int kind = kind_of(l);
+        int32_t e = l + 1;
+        auto stretch_end = [&](int32_t f, int k) {
+            while (f < depth && kind_of(f) == k) ++f;
+            return f;
+        };
+        e = stretch_end(l, kind);
+        if ((kind == 0 && e - l < kNarrowLevels) || (kind == 2 && e - l < kWideLevels)) kind = 1;
+        if (kind == 1) {  // up to the next long enough stretch of another kind
+            while (e < depth) {
+                const int k = kind_of(e);
+                const int32_t f = stretch_end(e, k);
+                if ((k == 0 && f - e >= kNarrowLevels) || (k == 2 && f - e >= kWideLevels)) break;
+                e = f;
+            }
+        }
+        if (kind == 2) slots = (slots + kPackRows - 1) / kPackRows * kPackRows;
+        SolveStretch st{S.lptr_h[l], S.lptr_h[e], slots, 0, (int32_t)blocks.size(), 0, kind == 2};
+        for (int32_t i = l; i < e; ++i) {
+            slot0[i] = slots;
+            slots += S.lptr_h[i + 1] - S.lptr_h[i];
+            if (kind == 2) slots = (slots + kPackRows - 1) / kPackRows * kPackRows;
+        }
+        st.slot1 = slots;
+        if (kind == 0) {
+            for (int64_t pos = st.pos0, prev = pos; pos < st.pos1;) {
                 const int32_t r = (int32_t)std::min<int64_t>(kBlockRows, st.pos1 - pos);
                 blocks.push_back(SolveBlock{pos, prev, st.pos0, r, 0});
                 prev = pos;
                 pos += r;
             }
             st.nblocks = (int32_t)blocks.size() - st.block0;
-            S.stretches.push_back(st);
         }
-        l = e > l ? e : e + 1;
+        S.stretches.push_back(st);
+        l = e;
     }
-    rows_until(n);
+    S.nrows = slots;
     const int g = grid_for(n, 256, ctx->num_sms * 8);
-    S.rows = alloc_n<SolveRow>(pool, n);
-    if (!S.rows) return RW_ERR_ALLOC;
+    S.rows = alloc_n<SolveRow>(pool, slots);
+    int64_t* d_slot0 = alloc_n<int64_t>(scratch, depth);
+    if (!S.rows || !d_slot0) return RW_ERR_ALLOC;
+    if ((rc = check_cuda(cudaMemcpyAsync(d_slot0, slot0.data(), sizeof(int64_t) * (size_t)depth,
+                                         cudaMemcpyHostToDevice, s),
+                         "copy")) ||
+        (slots > n &&
+         (rc = check_cuda(cudaMemsetAsync(S.rows, 0xFF, sizeof(SolveRow) * (size_t)slots, s), "memset"))))
+        return rc;
     RW_COUNT_LAUNCH();
-    k_fill_rows<<<g, 256, 0, s>>>(n, order, last, rp, S.rows);
+    k_fill_rows<<<g, 256, 0, s>>>(n, depth, lptr_dev, d_slot0, order, last, rp, S.rows);
     if ((rc = check_launch("schedule rows"))) return rc;
     const int64_t nb = (int64_t)blocks.size(), nslots = nb * kBlockRows;
     if (nb == 0) return RW_OK;
@@ -738,7 +784,7 @@ __global__ void __launch_bounds__(512, sizeof(T) == 4 ? 2 : 1) k_rows(const RowP
         }
 #pragma unroll
         for (int o = NR; o < 32; o <<= 1) acc += __shfl_xor_sync(kFull, acc, o);
-        if (es == 0 && jok) st_relaxed(P.x + (size_t)cur.d.row * nr + j, cur.b - acc);
+        if (es == 0 && jok && cur.d.row >= 0) st_relaxed(P.x + (size_t)cur.d.row * nr + j, cur.b - acc);
     }
 }
 
@@ -857,8 +903,10 @@ __global__ void __launch_bounds__(512, MINB) k_rows_vec(const RowParams<T> P) {
                 wait_vec(src, cur.d.last, w);
 #pragma unroll
                 for (int u = 0; u < U; ++u)
-                    if (base + lane + u * 32 < cnt && any_pending<T, NR>(v[u], P.nrhs))
-                        xload_relaxed<T, NR>(src, P.nrhs, c[u], v[u]);
+                    if (base + lane + u * 32 < cnt && any_pending<T, NR>(v[u], P.nrhs)) {
+                        if (NR == 1 && c[u] == cur.d.last) v[u][0] = w[0];
+                        else xload_relaxed<T, NR>(src, P.nrhs, c[u], v[u]);
+                    }
                 first = false;
             }
 #pragma unroll
@@ -871,23 +919,119 @@ __global__ void __launch_bounds__(512, MINB) k_rows_vec(const RowParams<T> P) {
             }
         }
         const T sum = warp_sums_spread<T, NR>(acc);
-        if (owner) st_relaxed(P.x + (size_t)cur.d.row * P.nrhs + jo, cur.b - sum);
+        if (owner && cur.d.row >= 0) st_relaxed(P.x + (size_t)cur.d.row * P.nrhs + jo, cur.b - sum);
+    }
+}
+
+// Rows of the widest levels (at least kWideRows, more rows than warps), one
+// right-hand side: a warp takes four rows of one level, eight lanes each, so
+// that every FP64 instruction serves four rows and a level takes a quarter of
+// the rounds.  The rows array pads the levels of such a stretch to whole groups
+// of four; rows of different levels never share a warp (one could wait for
+// another).  Latency of the loads bounds it.  61x64x67 asymmetric grid, FP64:
+// these levels and the rest 219 us per application with a row per warp, 204 us
+// packed (227 us with two thread blocks per SM, more polls than work); 10^6
+// nodes, FP32: 25.4 ms of a PCG solve, 24.4 packed, 23.9 with two per SM.  With
+// four right-hand sides it was the slower one (64^3 7-point grid: 17.99 ->
+// 18.52 ms of PCG): the vector loads of k_rows_vec fill the lanes.
+template <typename T>
+__global__ void __launch_bounds__(512, sizeof(T) == 4 ? 2 : 1) k_rows_pack(const RowParams<T> P) {
+    constexpr int U = kPreEntries, L = kPackLanes, R = kPackRows;
+    const int lane = (int)lane_id(), l = lane % L;
+    const int64_t gw = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const int64_t step = (((int64_t)gridDim.x * blockDim.x) >> 5) * R;
+    const unsigned spin_limit = P.st->spin_limit;
+    auto wait_value = [&](int32_t c, T v) -> T {
+        unsigned spins = 0;
+        while (is_pending(v)) {
+            if (wait_gives_up(spins, spin_limit, &P.st->timeout)) return T(0);
+            if (spins > 4) __nanosleep(32);
+            v = ld_relaxed(P.x + c);
+        }
+        return v;
+    };
+    struct Pre {
+        SolveRow d;
+        int32_t c[U];
+        T y[U];
+        T b;
+    };
+    auto load = [&](const SolveRow& d, Pre& A) {
+        A.d = d;
+#pragma unroll
+        for (int u = 0; u < U; ++u) row_entry(P, d, l + u * L, A.c[u], A.y[u]);
+        A.b = l == 0 && d.row >= 0 ? P.rhs[d.row] : T(0);
+    };
+    const int64_t first = gw * R + lane / L;
+    Pre pre[2];
+    load(row_at(P, first), pre[0]);
+    load(row_at(P, first + step), pre[1]);
+    SolveRow after = row_at(P, first + 2 * step);
+    for (int64_t pos = first; pos - lane / L < P.n; pos += step) {  // (warp-uniform)
+        const Pre cur = pre[0];
+        pre[0] = pre[1];
+        load(after, pre[1]);
+        after = row_at(P, pos + 3 * step);
+        const int cnt = cur.d.cnt;
+        T acc = T(0);
+        int32_t c[U];
+        T y[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            c[u] = cur.c[u];
+            y[u] = cur.y[u];
+        }
+        const int most = __reduce_max_sync(kFull, cnt);
+        for (int base = 0; base < most; base += U * L) {
+            if (base > 0) {
+#pragma unroll
+                for (int u = 0; u < U; ++u) row_entry(P, cur.d, base + l + u * L, c[u], y[u]);
+            }
+            T v[U];
+            bool pend = false;
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                v[u] = base + l + u * L < cnt ? ld_relaxed(P.x + c[u]) : T(0);
+                pend |= is_pending(v[u]);
+            }
+            if (__any_sync(kFull, pend)) {
+                if (cur.d.last >= 0) wait_value(cur.d.last, ld_relaxed(P.x + cur.d.last));
+#pragma unroll
+                for (int u = 0; u < U; ++u)
+                    if (is_pending(v[u])) v[u] = ld_relaxed(P.x + c[u]);
+            }
+#pragma unroll
+            for (int u = 0; u < U; ++u)
+                if (base + u * L < most) acc += y[u] * wait_value(c[u], v[u]);
+        }
+#pragma unroll
+        for (int o = L / 2; o >= 1; o >>= 1) acc += __shfl_xor_sync(kFull, acc, o);
+        if (l == 0 && cur.d.row >= 0) st_relaxed(P.x + cur.d.row, cur.b - acc);
     }
 }
 
 template <typename T, int NR, bool VEC>
-static rw_status launch_rows(rw_context* ctx, const RowParams<T>& P) {
-    const int two = VEC && ctx->opt.solve_blocks_per_sm >= 2 ? 1 : 0;
+static rw_status launch_rows(rw_context* ctx, const RowParams<T>& P, bool pack) {
+    int which = VEC && ctx->opt.solve_blocks_per_sm >= 2 ? 1 : 0;
     const void* kern;
-    if constexpr (VEC) kern = two ? (const void*)k_rows_vec<T, NR, 2> : (const void*)k_rows_vec<T, NR, 1>;
-    else kern = (const void*)k_rows<T, NR>;
-    static int per_sm_of[2] = {-1, -1};
-    int& per_sm = per_sm_of[two];
+    if constexpr (VEC) {
+        kern = which ? (const void*)k_rows_vec<T, NR, 2> : (const void*)k_rows_vec<T, NR, 1>;
+        if constexpr (NR == 1) {
+            if (pack) {
+                which = 2;
+                kern = (const void*)k_rows_pack<T>;
+            }
+        }
+    } else {
+        kern = (const void*)k_rows<T, NR>;
+    }
+    static int per_sm_of[3] = {-1, -1, -1};
+    int& per_sm = per_sm_of[which];
     if (per_sm < 0) {
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 512, 0);
         if (per_sm < 1) per_sm = 1;
     }
-    int64_t blocks = (int64_t)std::min(per_sm, 2) * ctx->num_sms;
+    int64_t blocks = (int64_t)std::min(per_sm, which == 2 && sizeof(T) == 8 ? 1 : 2) * ctx->num_sms;
     const int64_t need = (P.n + 15) / 16;
     if (blocks > need) blocks = need;
     if (blocks < 1) blocks = 1;
@@ -1329,20 +1473,27 @@ static rw_status solve_runs_nr(rw_context* ctx, const SolveSchedule& S, const in
         if ((rc = check_launch("solve begin"))) return rc;
     }
     if (rows) {
-        // the rows at positions [pos0, pos1); vector entries while one entry's
+        // the rows in slots [slot0, slot1); vector entries while one entry's
         // right-hand sides fit in 32 bytes of registers
-        auto solve_rows = [&](int64_t pos0, int64_t pos1) -> rw_status {
-            const RowParams<T> P{pos1 - pos0, S.rows + pos0, col, val, rhs, x, nrhs, ctx->d_status};
+        auto solve_rows = [&](int64_t slot0, int64_t slot1, bool pack) -> rw_status {
+            const RowParams<T> P{slot1 - slot0, S.rows + slot0, col, val, rhs, x, nrhs, ctx->d_status};
             if constexpr (NR * sizeof(T) <= 32) {
-                if (ctx->opt.wide_slices < 0) return launch_rows<T, NR, true>(ctx, P);
+                if (ctx->opt.wide_slices < 0) return launch_rows<T, NR, true>(ctx, P, pack);
             }
-            return launch_rows<T, NR, false>(ctx, P);
+            return launch_rows<T, NR, false>(ctx, P, false);
         };
-        if (mode == 1 || ctx->num_sms <= kMainBlocks) return solve_rows(0, S.n);
+        if (mode == 1 || ctx->num_sms <= kMainBlocks) return solve_rows(0, S.nrows, false);
         unsigned epoch = 0, mid = 0;
-        for (const SolveStretch& st : S.stretches) {
+        const bool packs = NR == 1 && ctx->opt.wide_slices < 0;
+        for (size_t i = 0; i < S.stretches.size(); ++i) {
+            const SolveStretch& st = S.stretches[i];
             if (st.nblocks == 0) {
-                if ((rc = solve_rows(st.pos0, st.pos1))) return rc;
+                const bool pack = packs && st.pack;
+                int64_t slot1 = st.slot1;  // unpacked neighbours in one launch
+                while (!pack && i + 1 < S.stretches.size() && S.stretches[i + 1].nblocks == 0 &&
+                       !(packs && S.stretches[i + 1].pack))
+                    slot1 = S.stretches[++i].slot1;
+                if ((rc = solve_rows(st.slot0, slot1, pack))) return rc;
                 continue;
             }
             BlockParams<T> P{};
