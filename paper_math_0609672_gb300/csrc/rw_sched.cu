@@ -71,6 +71,9 @@ __global__ void k_pos_of(int32_t n, const int32_t* __restrict__ order, int32_t* 
 // The entries of a block slot's row, by where their column lies: in the block
 // (0), in the block before it (1), earlier in the stretch (2), before it (3).
 constexpr int kClasses = 4;
+// Place of a class in the common numbering of the entries: the in-block ones,
+// which only the inversion reads, come last.
+__host__ __device__ __forceinline__ int class_place(int k) { return (k + kClasses - 1) % kClasses; }
 __device__ __forceinline__ int entry_class(int64_t p, const SolveBlock& b) {
     return p >= b.pos0 ? 0 : p >= b.prev0 ? 1 : p >= b.stretch0 ? 2 : 3;
 }
@@ -102,19 +105,21 @@ __global__ void __launch_bounds__(256) k_block_count(int64_t nslots, const Solve
         }
         if (lane == 0) {
 #pragma unroll
-            for (int k = 0; k < kClasses; ++k) cnt[k * nslots + t] = c[k];
+            for (int k = 0; k < kClasses; ++k) cnt[class_place(k) * nslots + t] = c[k];
             trow[t] = row;
         }
     }
 }
 
 // The entries of each class, in the row's order: slots and values inside the
-// block, columns, values and FP32 copies of the others.
+// block (from `inside` of the common numbering on), columns, values and FP32
+// copies of the others.
 struct BlockEntries {
     const int64_t* ptr[kClasses];  // [nslots + 1] first entry of each slot
-    int32_t* idx[kClasses];
-    double* val[kClasses];
-    float* val32[kClasses];        // (NULL inside the block, or without FP32 copies)
+    int64_t inside;
+    int32_t *slot, *col;
+    double *yval, *val;
+    float* val32;  // (NULL without FP32 copies)
 };
 
 __global__ void __launch_bounds__(256) k_block_split(int64_t nslots, const SolveBlock* __restrict__ blocks,
@@ -145,9 +150,14 @@ __global__ void __launch_bounds__(256) k_block_split(int64_t nslots, const Solve
                 const unsigned m = __ballot_sync(kFull, cl == k);
                 if (cl == k) {
                     const int64_t at = o[k] + __popc(m & lt);
-                    E.idx[k][at] = k == 0 ? (int32_t)(p - b.pos0) : c;
-                    E.val[k][at] = val[q];
-                    if (E.val32[k]) E.val32[k][at] = val32[q];
+                    if (k == 0) {
+                        E.slot[at - E.inside] = (int32_t)(p - b.pos0);
+                        E.yval[at - E.inside] = val[q];
+                    } else {
+                        E.col[at] = c;
+                        E.val[at] = val[q];
+                        if (E.val32) E.val32[at] = val32[q];
+                    }
                 }
                 o[k] += __popc(m);
             }
@@ -164,7 +174,7 @@ __global__ void __launch_bounds__(256) k_block_split(int64_t nslots, const Solve
 // spread over many SMs.
 constexpr int kPanel = 8;
 __global__ void __launch_bounds__(32) k_block_invert(const SolveBlock* __restrict__ blocks,
-                                                     const int64_t* __restrict__ iptr,
+                                                     const int64_t* __restrict__ iptr, int64_t inside,
                                                      const int32_t* __restrict__ islot,
                                                      const double* __restrict__ ival, double* inv, float* inv32) {
     __shared__ double X[kBlockRows * kPanel];  // [rows - c0][kPanel]
@@ -180,8 +190,8 @@ __global__ void __launch_bounds__(32) k_block_invert(const SolveBlock* __restric
     auto fetch = [&](int r) {
         e0 = e1 = 0;
         if (r < rows) {
-            e0 = iptr[t0 + r];
-            e1 = iptr[t0 + r + 1];
+            e0 = iptr[t0 + r] - inside;
+            e1 = iptr[t0 + r + 1] - inside;
         }
 #pragma unroll
         for (int u = 0; u < U; ++u) {
@@ -323,7 +333,7 @@ rw_status build_schedule(rw_context* ctx, int32_t n, const int64_t* rp, const in
     if (nb == 0) return RW_OK;
     int32_t* pos_of = alloc_n<int32_t>(scratch, n);
     uint32_t* cnt = alloc_n<uint32_t>(scratch, kClasses * nslots);
-    int64_t* ptr = alloc_n<int64_t>(pool, kClasses * (nslots + 1));
+    int64_t* ptr = alloc_n<int64_t>(pool, kClasses * nslots + 1);
     S.blocks = alloc_n<SolveBlock>(pool, nb);
     S.trow = alloc_n<int32_t>(pool, nslots);
     S.inv = alloc_n<double>(pool, nb * tri(kBlockRows));
@@ -342,24 +352,20 @@ rw_status build_schedule(rw_context* ctx, int32_t n, const int64_t* rp, const in
     if ((rc = check_launch("schedule count"))) return rc;
     BlockEntries E{};
     int64_t* h64 = static_cast<int64_t*>(ctx->h_small);
-    for (int k = 0; k < kClasses; ++k) {
-        int64_t* p = ptr + k * (nslots + 1);
-        E.ptr[k] = p;
-        if ((rc = check_cuda(scan_u32_to_i64(cnt + k * nslots, p, nslots, s, scratch), "scan")) ||
-            (rc = check_cuda(cudaMemcpyAsync(h64 + k, p + nslots, 8, cudaMemcpyDeviceToHost, s), "copy")))
-            return rc;
-    }
-    if ((rc = check_cuda(cudaStreamSynchronize(s), "sync"))) return rc;
-    int64_t total[kClasses];
-    for (int k = 0; k < kClasses; ++k) total[k] = h64[k];
-    for (int k = 0; k < kClasses; ++k) {
-        Pool& where = k == 0 ? scratch : pool;
-        E.idx[k] = alloc_n<int32_t>(where, total[k]);
-        E.val[k] = alloc_n<double>(where, total[k]);
-        E.val32[k] = k > 0 && val32 ? alloc_n<float>(where, total[k]) : nullptr;
-        if (!E.idx[k] || !E.val[k] || (k > 0 && val32 && !E.val32[k])) return RW_ERR_ALLOC;
-    }
-    for (int k = 0; k + 1 < kClasses; ++k) S.ext[k] = SolveEntries{E.ptr[k + 1], E.idx[k + 1], E.val[k + 1], E.val32[k + 1]};
+    if ((rc = check_cuda(scan_u32_to_i64(cnt, ptr, kClasses * nslots, s, scratch), "scan")) ||
+        (rc = check_cuda(cudaMemcpyAsync(h64, ptr + class_place(0) * nslots, 8, cudaMemcpyDeviceToHost, s), "copy")) ||
+        (rc = check_cuda(cudaMemcpyAsync(h64 + 1, ptr + kClasses * nslots, 8, cudaMemcpyDeviceToHost, s), "copy")) ||
+        (rc = check_cuda(cudaStreamSynchronize(s), "sync")))
+        return rc;
+    for (int k = 0; k < kClasses; ++k) E.ptr[k] = ptr + class_place(k) * nslots;
+    E.inside = h64[0];
+    E.slot = alloc_n<int32_t>(scratch, h64[1] - E.inside);
+    E.yval = alloc_n<double>(scratch, h64[1] - E.inside);
+    E.col = alloc_n<int32_t>(pool, E.inside);
+    E.val = alloc_n<double>(pool, E.inside);
+    E.val32 = val32 ? alloc_n<float>(pool, E.inside) : nullptr;
+    if (!E.slot || !E.yval || !E.col || !E.val || (val32 && !E.val32)) return RW_ERR_ALLOC;
+    for (int k = 0; k + 1 < kClasses; ++k) S.ext[k] = SolveEntries{E.ptr[k + 1], E.col, E.val, E.val32};
     RW_COUNT_LAUNCH();
     k_block_split<<<gw, 256, 0, s>>>(nslots, S.blocks, S.trow, rp, col, val, val32, pos_of, E);
     if ((rc = check_launch("schedule split"))) return rc;
@@ -367,7 +373,7 @@ rw_status build_schedule(rw_context* ctx, int32_t n, const int64_t* rp, const in
         const unsigned nbl = (unsigned)std::min<int64_t>(nb - b0, 65535);
         RW_COUNT_LAUNCH();
         k_block_invert<<<dim3(kBlockRows / kPanel, nbl), 32, 0, s>>>(
-            S.blocks + b0, E.ptr[0] + b0 * kBlockRows, E.idx[0], E.val[0], S.inv + b0 * tri(kBlockRows),
+            S.blocks + b0, E.ptr[0] + b0 * kBlockRows, E.inside, E.slot, E.yval, S.inv + b0 * tri(kBlockRows),
             S.inv32 ? S.inv32 + b0 * tri(kBlockRows) : nullptr);
     }
     return check_launch("block inverses");
