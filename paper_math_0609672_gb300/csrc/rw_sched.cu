@@ -58,6 +58,8 @@ constexpr int kWideLevels = 4;  // levels of a packed stretch at least (a launch
 constexpr int kPackLanes = 8;
 constexpr int kPackRows = 32 / kPackLanes;
 
+__device__ __forceinline__ bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; }
+
 __host__ __device__ __forceinline__ int64_t tri(int64_t m) { return m * (m + 1) / 2; }
 
 // ---------------------------------------------------------------------------
@@ -503,11 +505,11 @@ struct RowVec {
             R0.y[u] = q < R0.e ? P.val[q] : T(0);
         }
     }
-    // the nrhs values of x at node c (vector loads when nrhs == NR)
+    // the nrhs values of x at node c (vector loads when nrhs == NR and x is aligned for them)
     __device__ __forceinline__ void xload(const WideParams<T>& P, int32_t c, T (&v)[NR]) const {
         const T* p = P.x + (size_t)c * P.nrhs;
         if constexpr (NR >= 2 && sizeof(T) == 8) {
-            if (P.nrhs == NR) {
+            if (P.nrhs == NR && aligned16(P.x)) {
 #pragma unroll
                 for (int j = 0; j < NR; j += 2) {
                     const double2 d = __ldcg(reinterpret_cast<const double2*>(p + j));
@@ -517,7 +519,7 @@ struct RowVec {
                 return;
             }
         } else if constexpr (NR >= 4 && sizeof(T) == 4) {
-            if (P.nrhs == NR) {
+            if (P.nrhs == NR && aligned16(P.x)) {
 #pragma unroll
                 for (int j = 0; j < NR; j += 4) {
                     const float4 d = __ldcg(reinterpret_cast<const float4*>(p + j));
@@ -802,13 +804,13 @@ template <typename T, int NR>
 __device__ __forceinline__ void xload_relaxed(const T* x, int nrhs, int32_t c, T (&v)[NR]) {
     const T* p = x + (size_t)c * nrhs;
     if constexpr (NR >= 2 && sizeof(T) == 8) {
-        if (nrhs == NR) {
+        if (nrhs == NR && aligned16(x)) {
 #pragma unroll
             for (int j = 0; j < NR; j += 2) ld_relaxed_v2(reinterpret_cast<const double*>(p + j), v[j], v[j + 1]);
             return;
         }
     } else if constexpr (NR >= 4 && sizeof(T) == 4) {
-        if (nrhs == NR) {
+        if (nrhs == NR && aligned16(x)) {
 #pragma unroll
             for (int j = 0; j < NR; j += 4)
                 ld_relaxed_v4(reinterpret_cast<const float*>(p + j), v[j], v[j + 1], v[j + 2], v[j + 3]);
@@ -1110,12 +1112,13 @@ __device__ __forceinline__ bool blocks_barrier(unsigned* count, unsigned target,
     return give_up == 0;
 }
 
-// The nrhs values at node c (vector loads when nrhs == NR), from L2.
+// The nrhs values at node c (vector loads when nrhs == NR and x is aligned for
+// them: a caller's vector need not be), from L2.
 template <typename T, int NR>
 __device__ __forceinline__ void xload_cg(const T* x, int nrhs, int64_t c, T (&v)[NR]) {
     const T* p = x + c * nrhs;
     if constexpr (NR >= 2 && sizeof(T) == 8) {
-        if (nrhs == NR) {
+        if (nrhs == NR && aligned16(x)) {
 #pragma unroll
             for (int j = 0; j < NR; j += 2) {
                 const double2 d = __ldcg(reinterpret_cast<const double2*>(p + j));
@@ -1125,7 +1128,7 @@ __device__ __forceinline__ void xload_cg(const T* x, int nrhs, int64_t c, T (&v)
             return;
         }
     } else if constexpr (NR >= 4 && sizeof(T) == 4) {
-        if (nrhs == NR) {
+        if (nrhs == NR && aligned16(x)) {
 #pragma unroll
             for (int j = 0; j < NR; j += 4) {
                 const float4 d = __ldcg(reinterpret_cast<const float4*>(p + j));

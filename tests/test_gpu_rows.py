@@ -102,3 +102,26 @@ def test_packed_rows_in_single_precision(P, name):
         F.destroy()
     finally:
         c.close()
+
+
+@pytest.mark.parametrize("offset", [0, 1])
+@pytest.mark.parametrize("nrhs", [2, 4, 5, 8, 9, 12, 13, 16])
+def test_unaligned_vectors(P, nrhs, offset):
+    # vectors that start 8 bytes after a 16-byte boundary
+    import torch
+    A = W.grid3d(11, 10, 9, 7, np.random.default_rng(4), excess_frac=1e-3)
+    for mode in (0, 1, 2):
+        c = P.Context(options=P.rw_options_default(solve_mode=mode))
+        try:
+            F = P.rw_build_factor(c, P.CSR.from_host(A), 60, 3, 0.0)
+            r = np.random.default_rng(nrhs).standard_normal((A.n, nrhs))
+            store = torch.empty(A.n * nrhs + 1, dtype=torch.float64, device="cuda")
+            z = store[offset:offset + A.n * nrhs].view(A.n, nrhs)
+            P.rw_precond_apply(c, F, torch.as_tensor(r).cuda(), z)
+            t = {k: v.cpu().numpy() for k, v in F.tensors().items()}
+            y = _matvec(t["y_row_ptr"], t["y_col"], t["y_val"], z.cpu().numpy())
+            back = _matvec(t["yt_row_ptr"], t["yt_col"], t["yt_val"], y * t["d"][:, None])
+            assert np.abs(back - r).max() / np.abs(r).max() < 1e-11
+            F.destroy()
+        finally:
+            c.close()
