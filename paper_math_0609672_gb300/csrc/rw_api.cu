@@ -311,11 +311,10 @@ rw_status rw::complete_factor(rw_context* ctx, rw_factor* F, const FactorOut& fo
     }
     F->bar = static_cast<unsigned*>(F->pool.get((size_t)kSolveWorkspaceBytes));
     if (!F->bar) return RW_ERR_ALLOC;
-    if ((rc = build_schedule(ctx, n, fo.y_rp, fo.y_col, fo.y_val, y32, F->fwd_order, last, fwd_lptr,
-                             d.fwd_levels, F->fwd_sched, F->pool, scratch)))
-        return rc;
-    if ((rc = build_schedule(ctx, n, yt_rp, yt_col, yt_val, yt32, F->bwd_order, last + n, bwd_lptr,
-                             d.bwd_levels, F->bwd_sched, F->pool, scratch)))
+    if ((rc = build_schedules(
+             ctx, n, ScheduleInput{fo.y_rp, fo.y_col, fo.y_val, y32, F->fwd_order, last, fwd_lptr, d.fwd_levels},
+             F->fwd_sched, ScheduleInput{yt_rp, yt_col, yt_val, yt32, F->bwd_order, last + n, bwd_lptr, d.bwd_levels},
+             F->bwd_sched, F->pool, scratch)))
         return rc;
     if (timing) cudaEventRecord(ctx->ev[14], s);
     d.nnz = fo.nnz;

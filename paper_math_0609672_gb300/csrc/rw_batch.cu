@@ -820,10 +820,13 @@ rw_status rw_batch_create(rw_context* ctx, int32_t nmat, const rw_csr* As, const
     if ((rc = compute_levels_pair(
              ctx, (int32_t)N, LevelDag{B->y_rp, B->y_col, false, B->fwd_order, last, &B->fwd_depth, &fwd_lptr},
              LevelDag{B->yt_rp, B->yt_col, true, B->bwd_order, last + N, &B->bwd_depth, &bwd_lptr}, P, sc)) ||
-        (rc = build_schedule(ctx, (int32_t)N, B->y_rp, B->y_col, B->y_val, B->y_val32, B->fwd_order, last, fwd_lptr,
-                             B->fwd_depth, B->fwd_sched, P, sc)) ||
-        (rc = build_schedule(ctx, (int32_t)N, B->yt_rp, B->yt_col, B->yt_val, B->yt_val32, B->bwd_order, last + N,
-                             bwd_lptr, B->bwd_depth, B->bwd_sched, P, sc)))
+        (rc = build_schedules(ctx, (int32_t)N,
+                              ScheduleInput{B->y_rp, B->y_col, B->y_val, B->y_val32, B->fwd_order, last, fwd_lptr,
+                                            B->fwd_depth},
+                              B->fwd_sched,
+                              ScheduleInput{B->yt_rp, B->yt_col, B->yt_val, B->yt_val32, B->bwd_order, last + N,
+                                            bwd_lptr, B->bwd_depth},
+                              B->bwd_sched, P, sc)))
         return fail(rc);
     if ((rc = read_status(ctx, "batch create"))) return fail(rc);
     *out = B;

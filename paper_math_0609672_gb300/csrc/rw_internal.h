@@ -314,10 +314,18 @@ struct SolveSchedule {
     void* t = nullptr;               // workspace: [slots][nrhs] gathered right-hand sides
 };
 
-rw_status build_schedule(rw_context* ctx, int32_t n, const int64_t* rp, const int32_t* col,
-                         const double* val, const float* val32, const int32_t* order,
-                         const int32_t* last, const int64_t* lptr_dev, int32_t depth, SolveSchedule& S, Pool& pool,
-                         Pool& scratch);
+// One direction's triangle with its level order.
+struct ScheduleInput {
+    const int64_t* rp;
+    const int32_t* col;
+    const double* val;
+    const float* val32;  // NULL without FP32 copies
+    const int32_t *order, *last;
+    const int64_t* lptr;
+    int32_t depth;
+};
+rw_status build_schedules(rw_context* ctx, int32_t n, const ScheduleInput& fwd, SolveSchedule& F,
+                          const ScheduleInput& bwd, SolveSchedule& B, Pool& pool, Pool& scratch);
 
 // Device workspace of the solves, owned by the factor: two grid-barrier words.
 constexpr int64_t kSolveWorkspaceBytes = 256;

@@ -174,16 +174,35 @@ __global__ void __launch_bounds__(256) k_block_split(int64_t nslots, const Solve
 // FP64 pipe's latency along the rows bounds it (an FP64 FMA waits 64 cycles), so
 // the panels are narrow: many warps per SM, and the columns of a block are
 // spread over many SMs.
+// One direction's blocks leave most SMs idle on small factors, so both
+// directions share a launch (24 factors of random geometric
+// graphs: 50 launches of 152 us, now 25 of 157 us).
 constexpr int kPanel = 8;
-__global__ void __launch_bounds__(32) k_block_invert(const SolveBlock* __restrict__ blocks,
-                                                     const int64_t* __restrict__ iptr, int64_t inside,
-                                                     const int32_t* __restrict__ islot,
-                                                     const double* __restrict__ ival, double* inv, float* inv32) {
+struct InvertJob {
+    int64_t nb;
+    const SolveBlock* blocks;
+    const int64_t* ptr;  // first entry of each slot, the in-block ones from `inside` on
+    int64_t inside;
+    const int32_t* slot;
+    const double* val;
+    double* inv;
+    float* inv32;
+};
+
+__global__ void __launch_bounds__(32) k_block_invert(const InvertJob J0, const InvertJob J1, int64_t b0) {
     __shared__ double X[kBlockRows * kPanel];  // [rows - c0][kPanel]
     const int lane = (int)lane_id(), j = lane % kPanel, q = lane / kPanel;
-    const int64_t b = blockIdx.y;
-    const int rows = blocks[b].rows, c0 = (int)blockIdx.x * kPanel;
+    const InvertJob& J = blockIdx.z ? J1 : J0;
+    const int64_t b = b0 + blockIdx.y;
+    if (b >= J.nb) return;
+    const int rows = J.blocks[b].rows, c0 = (int)blockIdx.x * kPanel;
     if (c0 >= rows) return;
+    const int64_t* __restrict__ iptr = J.ptr;
+    const int32_t* __restrict__ islot = J.slot;
+    const double* __restrict__ ival = J.val;
+    const int64_t inside = J.inside;
+    double* const inv = J.inv;
+    float* const inv32 = J.inv32;
     const int64_t t0 = b * kBlockRows, out0 = b * tri(kBlockRows);
     constexpr int U = 4;  // entries per lane read ahead
     int32_t sl[U];
@@ -252,27 +271,22 @@ __global__ void k_fill_rows(int32_t n, int32_t depth, const int64_t* __restrict_
     }
 }
 
-rw_status build_schedule(rw_context* ctx, int32_t n, const int64_t* rp, const int32_t* col,
-                         const double* val, const float* val32, const int32_t* order,
-                         const int32_t* last, const int64_t* lptr_dev, int32_t depth, SolveSchedule& S, Pool& pool,
-                         Pool& scratch) {
-    NvtxRange nvtx_range("rw_schedule");
+// A schedule under construction.
+struct ScheduleWork {
+    std::vector<SolveBlock> blocks;
+    int32_t* pos_of = nullptr;
+    int64_t* ptr = nullptr;
+};
+
+// The stretches, rows and blocks of one direction, and (on their way to
+// totals[0..1]) the numbers of its blocks' entries outside and in all.
+static rw_status schedule_plan(rw_context* ctx, const ScheduleInput& in, SolveSchedule& S, ScheduleWork& W,
+                               int64_t* totals, Pool& pool, Pool& scratch) {
     cudaStream_t s = ctx->stream;
     rw_status rc;
-    S = SolveSchedule{};
-    S.n = n;
-    S.depth = depth;
-    S.order = order;
-    S.lptr = lptr_dev;
-    if (n == 0) return RW_OK;
-    S.lptr_h.resize((size_t)depth + 1);
-    if ((rc = check_cuda(cudaMemcpyAsync(S.lptr_h.data(), lptr_dev, sizeof(int64_t) * (depth + 1),
-                                         cudaMemcpyDeviceToHost, s),
-                         "copy")))
-        return rc;
-    if ((rc = check_cuda(cudaStreamSynchronize(s), "sync"))) return rc;
     // stretches: narrow ones as blocks, the others row by row, the widest levels packed
-    std::vector<SolveBlock> blocks;
+    std::vector<SolveBlock>& blocks = W.blocks;
+    const int32_t n = S.n, depth = S.depth;
     std::vector<int64_t> slot0((size_t)depth);  // of each level in the rows array
     int64_t slots = 0;
     auto kind_of = [&](int32_t l) {
@@ -329,54 +343,98 @@ rw_status build_schedule(rw_context* ctx, int32_t n, const int64_t* rp, const in
          (rc = check_cuda(cudaMemsetAsync(S.rows, 0xFF, sizeof(SolveRow) * (size_t)slots, s), "memset"))))
         return rc;
     RW_COUNT_LAUNCH();
-    k_fill_rows<<<g, 256, 0, s>>>(n, depth, lptr_dev, d_slot0, order, last, rp, S.rows);
+    k_fill_rows<<<g, 256, 0, s>>>(n, depth, S.lptr, d_slot0, S.order, in.last, in.rp, S.rows);
     if ((rc = check_launch("schedule rows"))) return rc;
     const int64_t nb = (int64_t)blocks.size(), nslots = nb * kBlockRows;
     if (nb == 0) return RW_OK;
-    int32_t* pos_of = alloc_n<int32_t>(scratch, n);
+    const bool fp32 = in.val32 != nullptr;
+    int32_t* const pos_of = W.pos_of = alloc_n<int32_t>(scratch, n);
     uint32_t* cnt = alloc_n<uint32_t>(scratch, kClasses * nslots);
-    int64_t* ptr = alloc_n<int64_t>(pool, kClasses * nslots + 1);
+    int64_t* const ptr = W.ptr = alloc_n<int64_t>(pool, kClasses * nslots + 1);
     S.blocks = alloc_n<SolveBlock>(pool, nb);
     S.trow = alloc_n<int32_t>(pool, nslots);
     S.inv = alloc_n<double>(pool, nb * tri(kBlockRows));
-    S.inv32 = val32 ? alloc_n<float>(pool, nb * tri(kBlockRows)) : nullptr;
+    S.inv32 = fp32 ? alloc_n<float>(pool, nb * tri(kBlockRows)) : nullptr;
     S.t = pool.get((size_t)nslots * 16 * sizeof(double));
-    if (!pos_of || !cnt || !ptr || !S.blocks || !S.trow || !S.inv || (val32 && !S.inv32) || !S.t) return RW_ERR_ALLOC;
+    if (!pos_of || !cnt || !ptr || !S.blocks || !S.trow || !S.inv || (fp32 && !S.inv32) || !S.t) return RW_ERR_ALLOC;
     if ((rc = check_cuda(cudaMemcpyAsync(S.blocks, blocks.data(), sizeof(SolveBlock) * (size_t)nb,
                                          cudaMemcpyHostToDevice, s),
                          "copy")))
         return rc;
     const int gw = grid_for(nslots * 32, 256, ctx->num_sms * 8);
     RW_COUNT_LAUNCH();
-    k_pos_of<<<g, 256, 0, s>>>(n, order, pos_of);
+    k_pos_of<<<g, 256, 0, s>>>(n, S.order, pos_of);
     RW_COUNT_LAUNCH();
-    k_block_count<<<gw, 256, 0, s>>>(nslots, S.blocks, order, rp, col, pos_of, cnt, S.trow);
+    k_block_count<<<gw, 256, 0, s>>>(nslots, S.blocks, S.order, in.rp, in.col, pos_of, cnt, S.trow);
     if ((rc = check_launch("schedule count"))) return rc;
-    BlockEntries E{};
-    int64_t* h64 = static_cast<int64_t*>(ctx->h_small);
     if ((rc = check_cuda(scan_u32_to_i64(cnt, ptr, kClasses * nslots, s, scratch), "scan")) ||
-        (rc = check_cuda(cudaMemcpyAsync(h64, ptr + class_place(0) * nslots, 8, cudaMemcpyDeviceToHost, s), "copy")) ||
-        (rc = check_cuda(cudaMemcpyAsync(h64 + 1, ptr + kClasses * nslots, 8, cudaMemcpyDeviceToHost, s), "copy")) ||
-        (rc = check_cuda(cudaStreamSynchronize(s), "sync")))
+        (rc = check_cuda(cudaMemcpyAsync(totals, ptr + class_place(0) * nslots, 8, cudaMemcpyDeviceToHost, s),
+                         "copy")))
         return rc;
-    for (int k = 0; k < kClasses; ++k) E.ptr[k] = ptr + class_place(k) * nslots;
-    E.inside = h64[0];
-    E.slot = alloc_n<int32_t>(scratch, h64[1] - E.inside);
-    E.yval = alloc_n<double>(scratch, h64[1] - E.inside);
+    return check_cuda(cudaMemcpyAsync(totals + 1, ptr + kClasses * nslots, 8, cudaMemcpyDeviceToHost, s), "copy");
+}
+
+// The entries of the blocks by class; J: the inversion of their triangles.
+static rw_status schedule_split(rw_context* ctx, const ScheduleInput& in, SolveSchedule& S, const ScheduleWork& W,
+                                const int64_t* totals, InvertJob& J, Pool& pool, Pool& scratch) {
+    cudaStream_t s = ctx->stream;
+    const int64_t nb = (int64_t)W.blocks.size(), nslots = nb * kBlockRows;
+    if (nb == 0) return RW_OK;
+    const int gw = grid_for(nslots * 32, 256, ctx->num_sms * 8);
+    BlockEntries E{};
+    for (int k = 0; k < kClasses; ++k) E.ptr[k] = W.ptr + class_place(k) * nslots;
+    E.inside = totals[0];
+    E.slot = alloc_n<int32_t>(scratch, totals[1] - E.inside);
+    E.yval = alloc_n<double>(scratch, totals[1] - E.inside);
     E.col = alloc_n<int32_t>(pool, E.inside);
     E.val = alloc_n<double>(pool, E.inside);
-    E.val32 = val32 ? alloc_n<float>(pool, E.inside) : nullptr;
-    if (!E.slot || !E.yval || !E.col || !E.val || (val32 && !E.val32)) return RW_ERR_ALLOC;
+    E.val32 = in.val32 ? alloc_n<float>(pool, E.inside) : nullptr;
+    if (!E.slot || !E.yval || !E.col || !E.val || (in.val32 && !E.val32)) return RW_ERR_ALLOC;
     for (int k = 0; k + 1 < kClasses; ++k) S.ext[k] = SolveEntries{E.ptr[k + 1], E.col, E.val, E.val32};
     RW_COUNT_LAUNCH();
-    k_block_split<<<gw, 256, 0, s>>>(nslots, S.blocks, S.trow, rp, col, val, val32, pos_of, E);
-    if ((rc = check_launch("schedule split"))) return rc;
+    k_block_split<<<gw, 256, 0, s>>>(nslots, S.blocks, S.trow, in.rp, in.col, in.val, in.val32, W.pos_of, E);
+    J = InvertJob{nb, S.blocks, E.ptr[0], E.inside, E.slot, E.yval, S.inv, S.inv32};
+    return check_launch("schedule split");
+}
+
+rw_status build_schedules(rw_context* ctx, int32_t n, const ScheduleInput& fwd, SolveSchedule& F,
+                          const ScheduleInput& bwd, SolveSchedule& B, Pool& pool, Pool& scratch) {
+    NvtxRange nvtx_range("rw_schedule");
+    cudaStream_t s = ctx->stream;
+    rw_status rc;
+    const ScheduleInput* in[2] = {&fwd, &bwd};
+    SolveSchedule* S[2] = {&F, &B};
+    for (int k = 0; k < 2; ++k) {
+        *S[k] = SolveSchedule{};
+        S[k]->n = n;
+        S[k]->depth = in[k]->depth;
+        S[k]->order = in[k]->order;
+        S[k]->lptr = in[k]->lptr;
+    }
+    if (n == 0) return RW_OK;
+    for (int k = 0; k < 2; ++k) {
+        S[k]->lptr_h.resize((size_t)S[k]->depth + 1);
+        if ((rc = check_cuda(cudaMemcpyAsync(S[k]->lptr_h.data(), S[k]->lptr, sizeof(int64_t) * (S[k]->depth + 1),
+                                             cudaMemcpyDeviceToHost, s),
+                             "copy")))
+            return rc;
+    }
+    if ((rc = check_cuda(cudaStreamSynchronize(s), "sync"))) return rc;
+    ScheduleWork W[2];
+    InvertJob J[2]{};
+    int64_t* totals = static_cast<int64_t*>(ctx->h_small);
+    for (int k = 0; k < 2; ++k)
+        if ((rc = schedule_plan(ctx, *in[k], *S[k], W[k], totals + 2 * k, pool, scratch))) return rc;
+    const int64_t nb = (int64_t)std::max(W[0].blocks.size(), W[1].blocks.size());
+    if (nb == 0) return RW_OK;
+    if ((rc = check_cuda(cudaStreamSynchronize(s), "sync"))) return rc;
+    const int64_t counts[4] = {totals[0], totals[1], totals[2], totals[3]};
+    for (int k = 0; k < 2; ++k)
+        if ((rc = schedule_split(ctx, *in[k], *S[k], W[k], counts + 2 * k, J[k], pool, scratch))) return rc;
     for (int64_t b0 = 0; b0 < nb; b0 += 65535) {
         const unsigned nbl = (unsigned)std::min<int64_t>(nb - b0, 65535);
         RW_COUNT_LAUNCH();
-        k_block_invert<<<dim3(kBlockRows / kPanel, nbl), 32, 0, s>>>(
-            S.blocks + b0, E.ptr[0] + b0 * kBlockRows, E.inside, E.slot, E.yval, S.inv + b0 * tri(kBlockRows),
-            S.inv32 ? S.inv32 + b0 * tri(kBlockRows) : nullptr);
+        k_block_invert<<<dim3(kBlockRows / kPanel, nbl, 2), 32, 0, s>>>(J[0], J[1], b0);
     }
     return check_launch("block inverses");
 }
