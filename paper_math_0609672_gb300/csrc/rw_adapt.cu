@@ -21,6 +21,7 @@
 // whose estimate moves by a few walks is decided again in the same round.
 // Walks beyond the final count are discarded; the counts and the decision
 // count are those of the one-decision-per-round schedule.
+#include <algorithm>
 #include <cmath>
 
 #include "rw_internal.h"
@@ -125,12 +126,19 @@ __global__ void k_adapt_chain(int32_t nw, const int4* __restrict__ wrow, const i
 __global__ void k_adapt_budget(int32_t n, uint32_t* budget) {
     for (int32_t k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) budget[k] = 0u;
 }
-// Every walk row: first decision after `first` walks, run ahead of it.
-__global__ void k_adapt_first(int32_t nw, const int4* __restrict__ wrow, uint32_t first, uint32_t pct,
+// Every walk row: first decision after `first` walks, run ahead of it.  The
+// first kDeepRows rows (a sixteenth of the rows at most) run at least `deep`
+// walks in the first round: with few homes below them their walks are the long
+// ones that every launch round waits for, and few in number.  Decided in one
+// round, they leave the later rounds to rows of short walks (48^3 27-point
+// grid, 20 walks at least, three rounds: 57 ms of walks before, 31 ms now).
+constexpr int32_t kDeepRows = 1024;
+__global__ void k_adapt_first(int32_t nw, const int4* __restrict__ wrow, uint32_t first, uint32_t pct, uint32_t deep,
                               uint32_t max_walks, uint32_t* T, uint32_t* inc) {
     for (int32_t r = blockIdx.x * blockDim.x + threadIdx.x; r < nw; r += gridDim.x * blockDim.x) {
         T[r] = first;
-        inc[wrow[r].x] = adapt_ahead(first, pct, max_walks);
+        const uint32_t a = adapt_ahead(first, pct, max_walks);
+        inc[wrow[r].x] = r < min(kDeepRows, nw / 16) ? max(a, min(deep, max_walks)) : a;
     }
 }
 __global__ void k_adapt_budget_rows(int32_t nw, const int4* __restrict__ wrow, const uint32_t* __restrict__ M,
@@ -193,9 +201,11 @@ rw_status rw_adaptive_budget(rw_context* ctx, const rw_csr* A, uint64_t seed, do
     const int gw = grid_for(nw, 256, ctx->num_sms * 8);
     const uint32_t pct = ctx->opt.adapt_ahead > 0 ? (uint32_t)ctx->opt.adapt_ahead : 0u;
     RW_COUNT_LAUNCH();
-    k_adapt_first<<<gw, 256, 0, s>>>(nw, T.wrow, min_walks, pct, max_walks, R.T, inc);
-    if ((rc = check_launch("adaptive start"))) return rc;
     const double d2 = delta * delta, z2 = z * z;
+    // twice the count of a row whose walk lengths are geometric (standard deviation = mean), 512 at most
+    const uint32_t deep = pct > 0 ? (uint32_t)std::min(512.0, std::ceil(2.0 * z2 / d2)) : 0u;
+    k_adapt_first<<<gw, 256, 0, s>>>(nw, T.wrow, min_walks, pct, deep, max_walks, R.T, inc);
+    if ((rc = check_launch("adaptive start"))) return rc;
     unsigned* hp = static_cast<unsigned*>(ctx->h_small);
     hp[0] = hp[1] = 0u;
     // Every launch round reaches each pending row's decision point at least
