@@ -271,9 +271,11 @@ __global__ void k_fill_rows(int32_t n, int32_t depth, const int64_t* __restrict_
     }
 }
 
-// A schedule under construction.
+// A schedule under construction.  The host arrays live until their uploads are
+// done (a GPU that shares the CPU's page tables may read them in place).
 struct ScheduleWork {
     std::vector<SolveBlock> blocks;
+    std::vector<int64_t> slot0;  // of each level in the rows array
     int32_t* pos_of = nullptr;
     int64_t* ptr = nullptr;
 };
@@ -287,7 +289,8 @@ static rw_status schedule_plan(rw_context* ctx, const ScheduleInput& in, SolveSc
     // stretches: narrow ones as blocks, the others row by row, the widest levels packed
     std::vector<SolveBlock>& blocks = W.blocks;
     const int32_t n = S.n, depth = S.depth;
-    std::vector<int64_t> slot0((size_t)depth);  // of each level in the rows array
+    std::vector<int64_t>& slot0 = W.slot0;
+    slot0.resize((size_t)depth);
     int64_t slots = 0;
     auto kind_of = [&](int32_t l) {
         const int64_t w = S.lptr_h[l + 1] - S.lptr_h[l];
@@ -426,8 +429,7 @@ rw_status build_schedules(rw_context* ctx, int32_t n, const ScheduleInput& fwd, 
     for (int k = 0; k < 2; ++k)
         if ((rc = schedule_plan(ctx, *in[k], *S[k], W[k], totals + 2 * k, pool, scratch))) return rc;
     const int64_t nb = (int64_t)std::max(W[0].blocks.size(), W[1].blocks.size());
-    if (nb == 0) return RW_OK;
-    if ((rc = check_cuda(cudaStreamSynchronize(s), "sync"))) return rc;
+    if ((rc = check_cuda(cudaStreamSynchronize(s), "sync")) || nb == 0) return rc;
     const int64_t counts[4] = {totals[0], totals[1], totals[2], totals[3]};
     for (int k = 0; k < 2; ++k)
         if ((rc = schedule_split(ctx, *in[k], *S[k], W[k], counts + 2 * k, J[k], pool, scratch))) return rc;
