@@ -428,8 +428,8 @@ def _walk_roofline(P, ctx, peaks, peak_kind, As, hops, walk_ms, l2_bytes, tag):
 def _solve_kernels(opt):
     """Names of the triangular-solve kernels the tuned options run."""
     def one(mode):
-        free = "k_syncfree_vec" if opt.get("wide_slices") == -1 else "k_syncfree"
-        return free if mode == 1 else f"k_thin/{free}" if mode == 2 else "k_thin/k_wide"
+        free = "k_rows_vec" if opt.get("wide_slices") == -1 else "k_rows"
+        return free if mode == 1 else f"k_blocks/{free}" if mode == 2 else "k_wide"
     fwd = one(opt.get("solve_mode", 0))
     bwd = one(opt.get("solve_mode_bwd", -1) if opt.get("solve_mode_bwd", -1) >= 0 else opt.get("solve_mode", 0))
     return f"{fwd} (forward) + {bwd} (backward)"
