@@ -331,8 +331,9 @@ __device__ __forceinline__ void drain_walks(const WalkParams& P, bool& active, W
     for (uint32_t round = 0;; ++round) {
         const bool near_cap = run && S.h + 4u > P.max_steps;
         if (!__any_sync(kFull, run) || __any_sync(kFull, near_cap)) break;
-        if ((round & 1023u) == 0u && ld_relaxed_u32(&P.st->walk_cap) != 0u) {
-            // another walk hit the step cap: stop (the build reports the error)
+        if ((round & 1023u) == 0u && __any_sync(kFull, ld_relaxed_u32(&P.st->walk_cap) != 0u)) {
+            // another walk hit the step cap: stop (the build reports the error), all lanes together: the
+            // loads of the lanes need not see one value, and the rounds' shuffles take the whole warp
             if (run && q == 0u) P.rec[S.widx] = walk_record(P.record_lengths, -2, S.h, S.ret);
             run = false;
             break;
