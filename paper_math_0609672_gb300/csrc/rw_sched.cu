@@ -20,7 +20,10 @@
 //     (k_rows).
 // Y = I - N with N >= 0 for an R-matrix, so the blocks' inverses have no
 // negative entries and are computed and applied without cancellation; they are
-// computed in FP64 whatever the solve's precision.
+// computed in FP64 whatever the solve's precision.  An entry of an inverse is
+// zero exactly where its row does not depend on its column, and zero entries
+// are not multiplied: 0 x infinity or NaN would carry a non-finite value to rows
+// that do not depend on it (of other matrices, in a batch).
 // One application of the preconditioner, before (narrow levels one after the
 // other in one thread block, the others sync-free with every lane polling its
 // own values) and now: 32^2 grid, 709 levels each way, 1.65 -> 0.076 ms; 300^2
@@ -61,6 +64,11 @@ constexpr int kPackRows = 32 / kPackLanes;
 __device__ __forceinline__ bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; }
 
 __host__ __device__ __forceinline__ int64_t tri(int64_t m) { return m * (m + 1) / 2; }
+
+// An entry of an inverse that is not the structural zero (integer tests: the
+// FP64 pipe is what bounds these kernels).
+__device__ __forceinline__ bool nonzero(double v) { return __double_as_longlong(v) != 0; }
+__device__ __forceinline__ bool nonzero(float v) { return __float_as_uint(v) != 0u; }
 
 // ---------------------------------------------------------------------------
 // Schedule construction
@@ -174,6 +182,8 @@ __global__ void __launch_bounds__(256) k_block_split(int64_t nslots, const Solve
 // FP64 pipe's latency along the rows bounds it (an FP64 FMA waits 64 cycles), so
 // the panels are narrow: many warps per SM, and the columns of a block are
 // spread over many SMs.
+// An entry to which some product contributes is stored as the least positive
+// number when it underflows, so that zero means that no product does.
 // One direction's blocks leave most SMs idle on small factors, so both
 // directions share a launch (24 factors of random geometric
 // graphs: 50 launches of 152 us, now 25 of 157 us).
@@ -233,22 +243,33 @@ __global__ void __launch_bounds__(32) k_block_invert(const InvertJob J0, const I
         const int64_t p0 = e0, p1 = e1;
         fetch(r + 1);  // in flight while this row is summed
         double acc = 0.0;
+        bool hit = false;
+        auto term = [&](int s, double yv) {
+            const double xv = X[(s - c0) * kPanel + j];
+            acc += yv * xv;
+            hit |= nonzero(xv);
+        };
 #pragma unroll
         for (int u = 0; u < U; ++u)
-            if (cs[u] >= c0) acc += cy[u] * X[(cs[u] - c0) * kPanel + j];
+            if (cs[u] >= c0) term(cs[u], cy[u]);
         for (int64_t p = p0 + q + 4 * U; p < p1; p += 4) {
             const int s = islot[p];
-            if (s >= c0) acc += ival[p] * X[(s - c0) * kPanel + j];
+            if (s >= c0) term(s, ival[p]);
         }
         acc += __shfl_xor_sync(kFull, acc, 8);
         acc += __shfl_xor_sync(kFull, acc, 16);
         const int c = c0 + j;
-        const double v = (r == c ? 1.0 : 0.0) - (r >= c ? acc : 0.0);
+        double v = (r == c ? 1.0 : 0.0) - (r >= c ? acc : 0.0);
+        hit = ((__ballot_sync(kFull, hit) >> j) & 0x01010101u) != 0u;  // in any of the column's four lanes
+        if (hit && !nonzero(v)) v = __longlong_as_double(1);
         if (q == 0) X[(r - c0) * kPanel + j] = v;
         __syncwarp();
         if (q == 0 && c <= r) {
             inv[out0 + tri(r) + c] = v;
-            if (inv32) inv32[out0 + tri(r) + c] = (float)v;
+            if (inv32) {
+                const float f = (float)v;
+                inv32[out0 + tri(r) + c] = nonzero(v) && !nonzero(f) ? __uint_as_float(1u) : f;
+            }
         }
     }
 }
@@ -1359,14 +1380,14 @@ __global__ void __launch_bounds__(256, 1) k_blocks(const BlockParams<T> P) {
                     T v[W][NR];
 #pragma unroll
                     for (int k = 0; k < W; ++k)
-                        if (lane + 32 * (k0 + k) <= slot)
+                        if (nonzero(iv[k0 + k]))
                             xload_cg<T, NR>(P.t, nr, b * kBlockRows + lane + 32 * (k0 + k), v[k]);
 #pragma unroll
                     for (int k = 0; k < W; ++k)
                         if (32 * (k0 + k) <= slot) {  // (FP64 instructions only for what the row holds)
 #pragma unroll
                             for (int j = 0; j < NR; ++j)
-                                acc[j] += lane + 32 * (k0 + k) <= slot ? iv[k0 + k] * v[k][j] : T(0);
+                                acc[j] += nonzero(iv[k0 + k]) ? iv[k0 + k] * v[k][j] : T(0);
                         }
                 }
                 const T sum = warp_sums_spread<T, NR>(acc);
