@@ -196,6 +196,12 @@ void rw_context_destroy(rw_context* ctx);
  * Philox-4x32-10 with counter (s/4, w, k, tag) and key (lo32(seed), hi32(seed)),
  * tag = (matrix_index << 2), matrix_index = 0 here.  Entries with
  * |Y_ki| < drop_tol are dropped (drop_tol >= 0; 0 keeps every entry).
+ * Memory beside the factor itself: the schedule of the solves takes 24 bytes per
+ * row and, for the rows on narrow levels (at most 96 rows), about 1.7 KB per row
+ * and direction (1.2 KB without FP32 copies) and a copy of their entries; these
+ * blocks end at a sixteenth of the device's memory per direction, and beyond
+ * 32 MB per direction they are given up when their memory cannot be allocated
+ * (the rows are then solved one by one).
  * On success *out receives a new factor (rw_factor_destroy releases it). */
 rw_status rw_build_factor(rw_context* ctx, const rw_csr* A, uint32_t walks_per_row, uint64_t seed,
                           double drop_tol, rw_factor** out);

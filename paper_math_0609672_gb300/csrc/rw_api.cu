@@ -219,6 +219,11 @@ rw_status rw_context_create(rw_context** out, void* stream, rw_alloc_fn alloc, r
         }
     }
     c->l2_bytes = (size_t)(l2 > 0 ? l2 : 0);
+    size_t free_bytes = 0;
+    if ((rc = check_cuda(cudaMemGetInfo(&free_bytes, &c->mem_bytes), "cudaMemGetInfo"))) {
+        rw_context_destroy(c);
+        return rc;
+    }
     // a fresh context reports no error until a call sets one
     if ((rc = reset_status(c)) || (rc = check_cuda(cudaStreamSynchronize(c->stream), "sync"))) {
         rw_context_destroy(c);

@@ -25,6 +25,7 @@ struct rw_context {
     void* h_small = nullptr;            // pinned host scratch (256 bytes)
     double reuse_ratio = 8.0;           // walk reuse: extra records per walk to allocate for
     size_t l2_bytes = 0;                // L2 cache size of the device
+    size_t mem_bytes = 0;               // memory of the device
     cudaEvent_t ev[16] = {};
 };
 
@@ -64,6 +65,10 @@ struct Pool {
     void* get(size_t bytes);   // nullptr on failure (error message set)
     void release(void* p);     // free one allocation now
     void release_all();
+    void absorb(Pool& o) {     // takes over the allocations of a pool of the same context
+        bufs.insert(bufs.end(), o.bufs.begin(), o.bufs.end());
+        o.bufs.clear();
+    }
     ~Pool() { release_all(); }
     Pool(const Pool&) = delete;
     Pool& operator=(const Pool&) = delete;
@@ -282,9 +287,9 @@ struct SolveStretch {
 
 // Block of a narrow stretch: positions [pos0, pos0 + rows); prev0: the first
 // position of the block before it (pos0 in the stretch's first block);
-// stretch0: the first position of the stretch.
+// stretch0: the first position of the stretch; inv0: where its inverse starts.
 struct SolveBlock {
-    int64_t pos0, prev0, stretch0;
+    int64_t pos0, prev0, stretch0, inv0;
     int32_t rows, pad;
 };
 

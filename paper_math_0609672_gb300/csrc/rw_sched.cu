@@ -51,6 +51,20 @@ constexpr int kNarrowLevels = 16;
 // Rows of a block.  With 512 the inversion takes twice as long (both directions
 // of the 64^3 7-point grid: 2.3 against 1.2 ms of a 23 ms build).
 constexpr int kBlockRows = 256;
+// Thread blocks that solve a block's slots (see k_blocks); smaller devices take
+// every row by itself.
+constexpr int kMainBlocks = 64;
+
+// Memory of the blocks of one direction, in bytes of inverses and workspace
+// (a full block: 263 KB of FP64 inverse, 132 KB of FP32 copies and 42 KB of
+// slots, 1.7 KB per row; beside it the schedule holds at most one more copy of
+// the rows' entries).  A factor whose levels are all narrow would take several
+// times its own size, so the blocks end at a sixteenth of the device's memory
+// (10 million rows on 284 GB) and the rows after them are solved one by one.
+// Beyond kBlockBytesSure they are also given up when their memory is not to be
+// had: the factor then keeps the blocks of that many bytes only.
+constexpr int64_t kBlockBytesSure = (int64_t)32 << 20;
+constexpr int kBlockMemoryPart = 16;
 
 // Rows of a wide level at least: with more rows than warps (16 on each of 152
 // SMs) a level takes several rounds, and a round of packed rows four at a time
@@ -213,7 +227,7 @@ __global__ void __launch_bounds__(32) k_block_invert(const InvertJob J0, const I
     const int64_t inside = J.inside;
     double* const inv = J.inv;
     float* const inv32 = J.inv32;
-    const int64_t t0 = b * kBlockRows, out0 = b * tri(kBlockRows);
+    const int64_t t0 = b * kBlockRows, out0 = J.blocks[b].inv0;
     constexpr int U = 4;  // entries per lane read ahead
     int32_t sl[U];
     double y[U];
@@ -296,15 +310,29 @@ __global__ void k_fill_rows(int32_t n, int32_t depth, const int64_t* __restrict_
 // done (a GPU that shares the CPU's page tables may read them in place).
 struct ScheduleWork {
     std::vector<SolveBlock> blocks;
+    int64_t inverse = 0;         // entries of the blocks' inverses
     std::vector<int64_t> slot0;  // of each level in the rows array
     int32_t* pos_of = nullptr;
     int64_t* ptr = nullptr;
 };
 
-// The stretches, rows and blocks of one direction, and (on their way to
-// totals[0..1]) the numbers of its blocks' entries outside and in all.
+// Entries of the inverses of a stretch of `rows` rows, and the bytes that its
+// blocks take (see kBlockBytesSure).
+static int64_t inverse_entries(int64_t rows) {
+    return rows / kBlockRows * tri(kBlockRows) + tri(rows % kBlockRows);
+}
+static int64_t block_bytes(int64_t rows, bool fp32) {
+    const int64_t nb = (rows + kBlockRows - 1) / kBlockRows;
+    return inverse_entries(rows) * (fp32 ? 12 : 8) +
+           nb * (int64_t)(kBlockRows * (16 * sizeof(double) + kClasses * sizeof(int64_t) + sizeof(int32_t)) +
+                          sizeof(SolveBlock));
+}
+
+// The stretches, rows and blocks (of `room` bytes at most; *used receives them)
+// of one direction, and (on their way to totals[0..1]) the numbers of its
+// blocks' entries outside and in all.
 static rw_status schedule_plan(rw_context* ctx, const ScheduleInput& in, SolveSchedule& S, ScheduleWork& W,
-                               int64_t* totals, Pool& pool, Pool& scratch) {
+                               int64_t* totals, int64_t room, int64_t* used, Pool& pool, Pool& scratch) {
     cudaStream_t s = ctx->stream;
     rw_status rc;
     // stretches: narrow ones as blocks, the others row by row, the widest levels packed
@@ -313,9 +341,11 @@ static rw_status schedule_plan(rw_context* ctx, const ScheduleInput& in, SolveSc
     std::vector<int64_t>& slot0 = W.slot0;
     slot0.resize((size_t)depth);
     int64_t slots = 0;
+    bool full = ctx->num_sms <= kMainBlocks;  // no (further) blocks
+    const bool fp32 = in.val32 != nullptr;
     auto kind_of = [&](int32_t l) {
         const int64_t w = S.lptr_h[l + 1] - S.lptr_h[l];
-        return w <= kNarrow ? 0 : w < kWideRows ? 1 : 2;
+        return w <= kNarrow && !full ? 0 : w < kWideRows ? 1 : 2;
     };
     for (int32_t l = 0; l < depth;) {
         // the longest stretch of one kind; one too short for a launch of its own joins the row by row levels
@@ -326,6 +356,16 @@ static rw_status schedule_plan(rw_context* ctx, const ScheduleInput& in, SolveSc
             return f;
         };
         e = stretch_end(l, kind);
+        if (kind == 0 && *used + block_bytes(S.lptr_h[e] - S.lptr_h[l], fp32) > room) {
+            int32_t lo = l, hi = e;  // the last level that still has room, by bisection
+            while (hi - lo > 1) {
+                const int32_t mid = lo + (hi - lo) / 2;
+                (*used + block_bytes(S.lptr_h[mid] - S.lptr_h[l], fp32) > room ? hi : lo) = mid;
+            }
+            full = true;
+            if (lo - l < kNarrowLevels) continue;
+            e = lo;
+        }
         if ((kind == 0 && e - l < kNarrowLevels) || (kind == 2 && e - l < kWideLevels)) kind = 1;
         if (kind == 1) {  // up to the next long enough stretch of another kind
             while (e < depth) {
@@ -346,11 +386,13 @@ static rw_status schedule_plan(rw_context* ctx, const ScheduleInput& in, SolveSc
         if (kind == 0) {
             for (int64_t pos = st.pos0, prev = pos; pos < st.pos1;) {
                 const int32_t r = (int32_t)std::min<int64_t>(kBlockRows, st.pos1 - pos);
-                blocks.push_back(SolveBlock{pos, prev, st.pos0, r, 0});
+                blocks.push_back(SolveBlock{pos, prev, st.pos0, W.inverse, r, 0});
+                W.inverse += tri(r);
                 prev = pos;
                 pos += r;
             }
             st.nblocks = (int32_t)blocks.size() - st.block0;
+            *used += block_bytes(st.pos1 - st.pos0, fp32);
         }
         S.stretches.push_back(st);
         l = e;
@@ -371,14 +413,13 @@ static rw_status schedule_plan(rw_context* ctx, const ScheduleInput& in, SolveSc
     if ((rc = check_launch("schedule rows"))) return rc;
     const int64_t nb = (int64_t)blocks.size(), nslots = nb * kBlockRows;
     if (nb == 0) return RW_OK;
-    const bool fp32 = in.val32 != nullptr;
     int32_t* const pos_of = W.pos_of = alloc_n<int32_t>(scratch, n);
     uint32_t* cnt = alloc_n<uint32_t>(scratch, kClasses * nslots);
     int64_t* const ptr = W.ptr = alloc_n<int64_t>(pool, kClasses * nslots + 1);
     S.blocks = alloc_n<SolveBlock>(pool, nb);
     S.trow = alloc_n<int32_t>(pool, nslots);
-    S.inv = alloc_n<double>(pool, nb * tri(kBlockRows));
-    S.inv32 = fp32 ? alloc_n<float>(pool, nb * tri(kBlockRows)) : nullptr;
+    S.inv = alloc_n<double>(pool, W.inverse);
+    S.inv32 = fp32 ? alloc_n<float>(pool, W.inverse) : nullptr;
     S.t = pool.get((size_t)nslots * 16 * sizeof(double));
     if (!pos_of || !cnt || !ptr || !S.blocks || !S.trow || !S.inv || (fp32 && !S.inv32) || !S.t) return RW_ERR_ALLOC;
     if ((rc = check_cuda(cudaMemcpyAsync(S.blocks, blocks.data(), sizeof(SolveBlock) * (size_t)nb,
@@ -421,13 +462,42 @@ static rw_status schedule_split(rw_context* ctx, const ScheduleInput& in, SolveS
     return check_launch("schedule split");
 }
 
+// Both directions with blocks of `room` bytes each at most; *used: the larger
+// of what they take.
+static rw_status schedules_in(rw_context* ctx, const ScheduleInput* const in[2], SolveSchedule* const S[2],
+                              int64_t room, int64_t* used, ScheduleWork (&W)[2], Pool& pool, Pool& scratch) {
+    cudaStream_t s = ctx->stream;
+    const int32_t n = S[0]->n;
+    rw_status rc;
+    InvertJob J[2]{};
+    int64_t* totals = static_cast<int64_t*>(ctx->h_small);
+    for (int k = 0; k < 2; ++k) {
+        *S[k] = SolveSchedule{n, in[k]->depth, in[k]->order, in[k]->lptr, std::move(S[k]->lptr_h)};
+        int64_t bytes = 0;
+        rc = schedule_plan(ctx, *in[k], *S[k], W[k], totals + 2 * k, room, &bytes, pool, scratch);
+        *used = std::max(*used, bytes);
+        if (rc) return rc;
+    }
+    const int64_t nb = (int64_t)std::max(W[0].blocks.size(), W[1].blocks.size());
+    if ((rc = check_cuda(cudaStreamSynchronize(s), "sync")) || nb == 0) return rc;
+    const int64_t counts[4] = {totals[0], totals[1], totals[2], totals[3]};
+    for (int k = 0; k < 2; ++k)
+        if ((rc = schedule_split(ctx, *in[k], *S[k], W[k], counts + 2 * k, J[k], pool, scratch))) return rc;
+    for (int64_t b0 = 0; b0 < nb; b0 += 65535) {
+        const unsigned nbl = (unsigned)std::min<int64_t>(nb - b0, 65535);
+        RW_COUNT_LAUNCH();
+        k_block_invert<<<dim3(kBlockRows / kPanel, nbl, 2), 32, 0, s>>>(J[0], J[1], b0);
+    }
+    return check_launch("block inverses");
+}
+
 rw_status build_schedules(rw_context* ctx, int32_t n, const ScheduleInput& fwd, SolveSchedule& F,
                           const ScheduleInput& bwd, SolveSchedule& B, Pool& pool, Pool& scratch) {
     NvtxRange nvtx_range("rw_schedule");
     cudaStream_t s = ctx->stream;
     rw_status rc;
-    const ScheduleInput* in[2] = {&fwd, &bwd};
-    SolveSchedule* S[2] = {&F, &B};
+    const ScheduleInput* const in[2] = {&fwd, &bwd};
+    SolveSchedule* const S[2] = {&F, &B};
     for (int k = 0; k < 2; ++k) {
         *S[k] = SolveSchedule{};
         S[k]->n = n;
@@ -444,22 +514,21 @@ rw_status build_schedules(rw_context* ctx, int32_t n, const ScheduleInput& fwd, 
             return rc;
     }
     if ((rc = check_cuda(cudaStreamSynchronize(s), "sync"))) return rc;
-    ScheduleWork W[2];
-    InvertJob J[2]{};
-    int64_t* totals = static_cast<int64_t*>(ctx->h_small);
-    for (int k = 0; k < 2; ++k)
-        if ((rc = schedule_plan(ctx, *in[k], *S[k], W[k], totals + 2 * k, pool, scratch))) return rc;
-    const int64_t nb = (int64_t)std::max(W[0].blocks.size(), W[1].blocks.size());
-    if ((rc = check_cuda(cudaStreamSynchronize(s), "sync")) || nb == 0) return rc;
-    const int64_t counts[4] = {totals[0], totals[1], totals[2], totals[3]};
-    for (int k = 0; k < 2; ++k)
-        if ((rc = schedule_split(ctx, *in[k], *S[k], W[k], counts + 2 * k, J[k], pool, scratch))) return rc;
-    for (int64_t b0 = 0; b0 < nb; b0 += 65535) {
-        const unsigned nbl = (unsigned)std::min<int64_t>(nb - b0, 65535);
-        RW_COUNT_LAUNCH();
-        k_block_invert<<<dim3(kBlockRows / kPanel, nbl, 2), 32, 0, s>>>(J[0], J[1], b0);
+    for (int64_t room = std::max(kBlockBytesSure, (int64_t)(ctx->mem_bytes / kBlockMemoryPart));;
+         room = kBlockBytesSure) {
+        ScheduleWork W[2];
+        Pool mine(ctx), work(ctx);
+        int64_t used = 0;
+        rc = schedules_in(ctx, in, S, room, &used, W, mine, work);
+        if (rc == RW_OK) {
+            pool.absorb(mine);
+            scratch.absorb(work);
+            return RW_OK;
+        }
+        cudaStreamSynchronize(s);  // nothing reads the host arrays any more
+        if (rc != RW_ERR_ALLOC || used <= kBlockBytesSure) return rc;
+        cudaGetLastError();  // (the failed allocation's)
     }
-    return check_launch("block inverses");
 }
 
 // ---------------------------------------------------------------------------
@@ -1145,7 +1214,7 @@ static rw_status launch_rows(rw_context* ctx, const RowParams<T>& P, bool pack) 
 // (k_stretch_begin).  The chain per block is then two barriers and two rounds
 // of loads.
 // ---------------------------------------------------------------------------
-constexpr int kMainBlocks = 64;  // 256 slots: four warps of each (see k_blocks)
+static_assert(kBlockRows % kMainBlocks == 0 && kBlockRows / kMainBlocks <= 8, "a warp of a solving block per slot");
 constexpr int kLongGather = 512;
 
 template <typename T>
@@ -1319,6 +1388,7 @@ __global__ void __launch_bounds__(256, 1) k_blocks(const BlockParams<T> P) {
     int64_t q1 = 0, q0 = 0;
     T y[U], iv[V];
     auto fetch = [&](int64_t b) {
+        const int64_t inv0 = P.blocks[b].inv0;
         mine = slot < P.blocks[b].rows;
         const int64_t t = b * kBlockRows + slot;
         q0 = q1 = 0;
@@ -1333,7 +1403,7 @@ __global__ void __launch_bounds__(256, 1) k_blocks(const BlockParams<T> P) {
             c[u] = ok ? P.prev.idx[q0 + 32 * u] : -1;
             y[u] = ok ? P.prev.val[q0 + 32 * u] : T(0);
         }
-        const T* inv = P.inv + b * tri(kBlockRows) + tri(slot);
+        const T* inv = P.inv + inv0 + tri(slot);
 #pragma unroll
         for (int k = 0; k < V; ++k) iv[k] = mine && lane + 32 * k <= slot ? inv[lane + 32 * k] : T(0);
     };
