@@ -106,8 +106,9 @@ typedef struct {
     int32_t cluster_width;   /* level schedule: levels of at most this many rows run on one thread-block
                                 cluster with hardware barriers; 0 = never */
     int32_t cluster_size;    /* CTAs of that cluster (2..16; 0 = 16) */
-    int32_t solve_mode;      /* triangular solves: 0 = level schedule (the whole grid level by level),
-                                1 = sync-free (each row waits only for its own dependencies),
+    int32_t solve_mode;      /* triangular solves: 0 = level schedule (the whole grid level by level;
+                                stretches of narrow levels in blocks as with 2), 1 = sync-free (each row
+                                waits only for its own dependencies),
                                 2 = stretches of narrow levels in blocks of rows with inverted
                                 triangles, the other rows sync-free (default 2) */
     int32_t reuse;           /* 1: walk reuse (Algorithm 2 of Sec. 5.3) in single-matrix builds:

@@ -276,11 +276,12 @@ struct SolveRow {
     int32_t pad;
 };
 
-// Positions [pos0, pos1) solved together: as blocks, or (nblocks 0) row by row
-// from slots [slot0, slot1) of the rows array; pack: levels padded to whole
-// groups of rows.
+// Positions [pos0, pos1), levels [lev0, lev1), solved together: as blocks, or
+// (nblocks 0) row by row from slots [slot0, slot1) of the rows array, or level
+// by level; pack: levels padded to whole groups of rows.
 struct SolveStretch {
     int64_t pos0, pos1, slot0, slot1;
+    int32_t lev0, lev1;
     int32_t block0, nblocks;
     bool pack;
 };

@@ -31,9 +31,11 @@
 // levels, four right-hand sides 6.9 -> 2.5 ms, sixteen 28 -> 6.3 ms; 1000^2
 // with long-range edges, 2229 levels, FP32 8.5 -> 6.4 ms.
 //
-// solve_mode 1 takes every row as in a wide stretch; solve_mode 0 is
-// level-synchronous over the whole grid.  Every row sums its terms in a fixed
-// order, so results do not depend on timing.
+// solve_mode 1 takes every row as in a wide stretch; solve_mode 0 solves the
+// narrow stretches as blocks too and the other levels one after another over the
+// whole grid (with the narrow levels one after another too, a 100^2 grid of 5,594
+// levels takes 26.1 ms per application; with blocks 0.48 ms).  Every row sums its
+// terms in a fixed order, so results do not depend on timing.
 #include <algorithm>
 
 #include "rw_internal.h"
@@ -376,7 +378,7 @@ static rw_status schedule_plan(rw_context* ctx, const ScheduleInput& in, SolveSc
             }
         }
         if (kind == 2) slots = (slots + kPackRows - 1) / kPackRows * kPackRows;
-        SolveStretch st{S.lptr_h[l], S.lptr_h[e], slots, 0, (int32_t)blocks.size(), 0, kind == 2};
+        SolveStretch st{S.lptr_h[l], S.lptr_h[e], slots, 0, l, e, (int32_t)blocks.size(), 0, kind == 2};
         for (int32_t i = l; i < e; ++i) {
             slot0[i] = slots;
             slots += S.lptr_h[i + 1] - S.lptr_h[i];
@@ -1586,18 +1588,17 @@ static rw_status launch_cluster(rw_context* ctx, const SolveSchedule& S, int32_t
     }
 }
 
-// The level schedule: consecutive levels up to the cluster width go to one
-// cluster, the rest to the whole grid.
+// Levels [l, end) one after another: consecutive levels up to the cluster width
+// go to one cluster, the rest to the whole grid.
 template <typename T, int NR, int ES>
-static rw_status launch_levels(rw_context* ctx, const SolveSchedule& S, const int64_t* rp, const int32_t* col,
-                               const T* val, const T* rhs, T* x, int nrhs, unsigned* bar) {
+static rw_status launch_levels(rw_context* ctx, const SolveSchedule& S, int32_t l, int32_t end, const int64_t* rp,
+                               const int32_t* col, const T* val, const T* rhs, T* x, int nrhs, unsigned* bar) {
     const int64_t cw = ctx->opt.cluster_width > 0 ? ctx->opt.cluster_width : 0;
     const int csize = ctx->opt.cluster_size > 0 ? ctx->opt.cluster_size : 16;
-    int32_t l = 0;
-    while (l < S.depth) {
+    while (l < end) {
         const bool narrow = cw > 0 && S.lptr_h[l + 1] - S.lptr_h[l] <= cw;
         int32_t e = l + 1;
-        while (e < S.depth && (cw > 0 && S.lptr_h[e + 1] - S.lptr_h[e] <= cw) == narrow) ++e;
+        while (e < end && (cw > 0 && S.lptr_h[e + 1] - S.lptr_h[e] <= cw) == narrow) ++e;
         // cluster runs (1024-thread blocks, 64 registers) keep lane groups
         constexpr int CES = ES == 0 ? 32 / NR : ES;
         rw_status rc = narrow ? launch_cluster<T, NR, CES>(ctx, S, l, e, rp, col, val, rhs, x, nrhs, bar, csize)
@@ -1632,78 +1633,91 @@ static rw_status solve_runs_nr(rw_context* ctx, const SolveSchedule& S, const in
         k_solve_begin<T><<<grid_for(cnt, 256, ctx->num_sms * 8), 256, 0, s>>>(rows ? x : nullptr, cnt, w, d, nrhs, bar);
         if ((rc = check_launch("solve begin"))) return rc;
     }
-    if (rows) {
-        // the rows in slots [slot0, slot1); vector entries while one entry's
-        // right-hand sides fit in 32 bytes of registers
-        auto solve_rows = [&](int64_t slot0, int64_t slot1, bool pack) -> rw_status {
-            const RowParams<T> P{slot1 - slot0, S.rows + slot0, col, val, rhs, x, nrhs, ctx->d_status};
-            if constexpr (NR * sizeof(T) <= 32) {
-                // One FP32 right-hand side backward: the entries of the long rows of Y^T over lane groups, two thread
-                // blocks per SM (k_rows), 3.8 -> 3.2 ms per solve of 10^6 nodes with long-range edges, 1.19 -> 1.12 ms
-                // on a 56^3 27-point grid; forward the same costs 2.4 -> 2.9 ms.
-                const bool groups = sizeof(T) * NR == 4 && backward && !pack;
-                if (ctx->opt.wide_slices < 0 && !groups) return launch_rows<T, NR, true>(ctx, P, pack);
-            }
-            return launch_rows<T, NR, false>(ctx, P, false);
-        };
-        if (mode == 1 || ctx->num_sms <= kMainBlocks) return solve_rows(0, S.nrows, false);
-        unsigned epoch = 0, mid = 0;
-        const bool packs = NR == 1 && ctx->opt.wide_slices < 0;
-        for (size_t i = 0; i < S.stretches.size(); ++i) {
-            const SolveStretch& st = S.stretches[i];
-            if (st.nblocks == 0) {
-                const bool pack = packs && st.pack;
-                int64_t slot1 = st.slot1;  // unpacked neighbours in one launch
-                while (!pack && i + 1 < S.stretches.size() && S.stretches[i + 1].nblocks == 0 &&
-                       !(packs && S.stretches[i + 1].pack))
-                    slot1 = S.stretches[++i].slot1;
-                if ((rc = solve_rows(st.slot0, slot1, pack))) return rc;
-                continue;
-            }
-            BlockParams<T> P{};
-            P.blocks = S.blocks;
-            P.block0 = st.block0;
-            P.nblocks = st.nblocks;
-            P.trow = S.trow;
-            P.prev = block_sums<T>(S.ext[0]);
-            P.older = block_sums<T>(S.ext[1]);
-            P.from_rhs = st.pos0 == 0;
-            P.inv = schedule_values<T>(S.inv, S.inv32);
-            P.rhs = rhs;
-            P.x = x;
-            P.t = static_cast<T*>(S.t);
-            P.nrhs = nrhs;
-            P.bar = bar;
-            P.epoch0 = epoch;
-            P.mid0 = mid;
-            P.st = ctx->d_status;
-            if (st.pos0 > 0) {
-                const int64_t t0 = (int64_t)st.block0 * kBlockRows, t1 = t0 + (int64_t)st.nblocks * kBlockRows;
-                RW_COUNT_LAUNCH();
-                k_stretch_begin<T, NR><<<grid_for((t1 - t0) / 8, 1, ctx->num_sms * 8), 256, 0, s>>>(
-                    t0, t1, S.blocks, block_sums<T>(S.ext[2]), x, rhs, S.trow, P.t, nrhs);
-                if ((rc = check_launch("stretch begin"))) return rc;
-            }
-            if ((rc = launch_blocks<T, NR>(ctx, P))) return rc;
-            epoch += (unsigned)st.nblocks - 1;
-            mid += (unsigned)st.nblocks;
+    // the rows in slots [slot0, slot1); vector entries while one entry's
+    // right-hand sides fit in 32 bytes of registers
+    auto solve_rows = [&](int64_t slot0, int64_t slot1, bool pack) -> rw_status {
+        const RowParams<T> P{slot1 - slot0, S.rows + slot0, col, val, rhs, x, nrhs, ctx->d_status};
+        if constexpr (NR * sizeof(T) <= 32) {
+            // One FP32 right-hand side backward: the entries of the long rows of Y^T over lane groups, two thread
+            // blocks per SM (k_rows), 3.8 -> 3.2 ms per solve of 10^6 nodes with long-range edges, 1.19 -> 1.12 ms
+            // on a 56^3 27-point grid; forward the same costs 2.4 -> 2.9 ms.
+            const bool groups = sizeof(T) * NR == 4 && backward && !pack;
+            if (ctx->opt.wide_slices < 0 && !groups) return launch_rows<T, NR, true>(ctx, P, pack);
         }
-        return RW_OK;
+        return launch_rows<T, NR, false>(ctx, P, false);
+    };
+    if (mode == 1) return solve_rows(0, S.nrows, false);
+    // the levels [l, end) one after another
+    auto solve_levels = [&](int32_t l, int32_t end) -> rw_status {
+        switch (lane_slices(ctx->opt.wide_slices, NR)) {
+            case 0: {
+                // vector rows while one entry's right-hand sides fit in 64 bytes of registers
+                constexpr int ES = NR * sizeof(T) <= 64 ? 0 : 32 / NR;
+                return launch_levels<T, NR, ES>(ctx, S, l, end, rp, col, val, rhs, x, nrhs, bar);
+            }
+            case 1: return launch_levels<T, NR, 1>(ctx, S, l, end, rp, col, val, rhs, x, nrhs, bar);
+            case 2: return launch_levels<T, NR, 2>(ctx, S, l, end, rp, col, val, rhs, x, nrhs, bar);
+            case 4: return launch_levels<T, NR, 4>(ctx, S, l, end, rp, col, val, rhs, x, nrhs, bar);
+            case 8: return launch_levels<T, NR, 8>(ctx, S, l, end, rp, col, val, rhs, x, nrhs, bar);
+            case 16: return launch_levels<T, NR, 16>(ctx, S, l, end, rp, col, val, rhs, x, nrhs, bar);
+            default: return launch_levels<T, NR, 32>(ctx, S, l, end, rp, col, val, rhs, x, nrhs, bar);
+        }
+    };
+    unsigned epoch = 0, mid = 0;
+    bool clear = rows || w;  // the barrier words hold the epochs
+    const bool packs = rows && NR == 1 && ctx->opt.wide_slices < 0;
+    for (size_t i = 0; i < S.stretches.size(); ++i) {
+        const SolveStretch& st = S.stretches[i];
+        if (st.nblocks == 0) {
+            const bool pack = packs && st.pack;
+            size_t e = i;  // unpacked neighbours in one launch
+            while (!pack && e + 1 < S.stretches.size() && S.stretches[e + 1].nblocks == 0 &&
+                   !(packs && S.stretches[e + 1].pack))
+                ++e;
+            i = e;
+            if (rows) {
+                rc = solve_rows(st.slot0, S.stretches[e].slot1, pack);
+            } else {
+                rc = solve_levels(st.lev0, S.stretches[e].lev1);
+                clear = false;
+            }
+            if (rc) return rc;
+            continue;
+        }
+        if (!clear) {
+            if ((rc = check_cuda(cudaMemsetAsync(bar, 0, 2 * sizeof(unsigned), s), "memset"))) return rc;
+            epoch = mid = 0;
+            clear = true;
+        }
+        BlockParams<T> P{};
+        P.blocks = S.blocks;
+        P.block0 = st.block0;
+        P.nblocks = st.nblocks;
+        P.trow = S.trow;
+        P.prev = block_sums<T>(S.ext[0]);
+        P.older = block_sums<T>(S.ext[1]);
+        P.from_rhs = st.pos0 == 0;
+        P.inv = schedule_values<T>(S.inv, S.inv32);
+        P.rhs = rhs;
+        P.x = x;
+        P.t = static_cast<T*>(S.t);
+        P.nrhs = nrhs;
+        P.bar = bar;
+        P.epoch0 = epoch;
+        P.mid0 = mid;
+        P.st = ctx->d_status;
+        if (st.pos0 > 0) {
+            const int64_t t0 = (int64_t)st.block0 * kBlockRows, t1 = t0 + (int64_t)st.nblocks * kBlockRows;
+            RW_COUNT_LAUNCH();
+            k_stretch_begin<T, NR><<<grid_for((t1 - t0) / 8, 1, ctx->num_sms * 8), 256, 0, s>>>(
+                t0, t1, S.blocks, block_sums<T>(S.ext[2]), x, rhs, S.trow, P.t, nrhs);
+            if ((rc = check_launch("stretch begin"))) return rc;
+        }
+        if ((rc = launch_blocks<T, NR>(ctx, P))) return rc;
+        epoch += (unsigned)st.nblocks - 1;
+        mid += (unsigned)st.nblocks;
     }
-    switch (lane_slices(ctx->opt.wide_slices, NR)) {
-        case 0:
-            // vector rows while one entry's right-hand sides fit in 64 bytes of registers
-            if constexpr (NR * sizeof(T) <= 64)
-                return launch_levels<T, NR, 0>(ctx, S, rp, col, val, rhs, x, nrhs, bar);
-            else
-                return launch_levels<T, NR, 32 / NR>(ctx, S, rp, col, val, rhs, x, nrhs, bar);
-        case 1: return launch_levels<T, NR, 1>(ctx, S, rp, col, val, rhs, x, nrhs, bar);
-        case 2: return launch_levels<T, NR, 2>(ctx, S, rp, col, val, rhs, x, nrhs, bar);
-        case 4: return launch_levels<T, NR, 4>(ctx, S, rp, col, val, rhs, x, nrhs, bar);
-        case 8: return launch_levels<T, NR, 8>(ctx, S, rp, col, val, rhs, x, nrhs, bar);
-        case 16: return launch_levels<T, NR, 16>(ctx, S, rp, col, val, rhs, x, nrhs, bar);
-        default: return launch_levels<T, NR, 32>(ctx, S, rp, col, val, rhs, x, nrhs, bar);
-    }
+    return RW_OK;
 }
 
 template <typename T>
