@@ -36,7 +36,8 @@ constexpr int kDotParts = 1024;  // blocks of the dot-product producing kernels
 // sides and 406 us with one; now 249 and 237 us (1.0e11 gathers/s).
 // Passes whose entries exceed the copy or that hold a row of more than
 // kLongRow entries per lane sum their rows with all 32 lanes each, straight
-// from memory.
+// from memory; matrices of long rows take no passes (rows_per_pass 0: a warp per
+// row throughout).
 //
 // DIFF (the FP32 operator of the mixed mode): val holds A_ij (j != i) and, at
 // the diagonal position, the excess e_i = A_ii + sum_j A_ij, and the row is
@@ -48,6 +49,14 @@ constexpr int kDotParts = 1024;  // blocks of the dot-product producing kernels
 constexpr int kSpmvEntries = 2048;  // entries of a pass (24 KB of columns and FP64 values: eight blocks per SM)
 constexpr int kSpmvRows = 512;      // rows of a pass
 constexpr int kLongRow = 64;
+// Average entries per row times right-hand sides (four at least) from which
+// every row is summed by a warp, straight from memory.  A pass then holds too
+// few rows for the copy to pay, and from 1000 entries a row only one or two, so
+// that most of the block idles.  Warp per row against the copy, us: 6000 rows of
+// 920 entries 27 | 70 (one right-hand side), 176 | 507 (16); 30,000 of 129 37 | 34
+// and 128 | 154; 200,000 of 65 134 | 89, 206 | 146 (three), 271 | 285 (eight) and
+// 420 | 467 (16); 60,000 of 33 46 | 27 and 83 | 88.
+constexpr int kLongRows = 512;
 
 // RES: the true residual b - A x of PCG instead of A x: stored as FP32
 // (out32) or FP64 where y is given, its squares in place of the dot products.
@@ -83,7 +92,23 @@ __global__ void __launch_bounds__(256) k_spmv(int32_t n, const int32_t* __restri
             if (part) dot += (double)x[at] * (double)acc;
         }
     };
-    const int64_t npass = ((int64_t)n + rows_per_pass - 1) / rows_per_pass;
+    // row `row`, entries [s, e), by the warp, straight from memory
+    auto warp_row = [&](int32_t row, int32_t s, int32_t e) {
+        constexpr int EW = 32 / NR;
+        const int j = lane % NR, es = lane / NR;
+        const bool jok = j < nrhs;
+        const TV xi = (DIFF && jok) ? x[(size_t)row * nrhs + j] : TV(0);
+        TV acc = TV(0);
+        if (jok)
+            for (int32_t p = s + es; p < e; p += EW) acc += term(col[p], val[p], row, j, xi);
+#pragma unroll
+        for (int o = NR; o < 32; o <<= 1) acc += __shfl_xor_sync(kFull, acc, o);
+        if (es == 0 && jok) finish((size_t)row * nrhs + j, acc, wdot);
+    };
+    const int64_t npass = rows_per_pass ? ((int64_t)n + rows_per_pass - 1) / rows_per_pass : 0;
+    if (npass == 0)
+        for (int64_t row = (int64_t)blockIdx.x * 8 + (tid >> 5); row < n; row += (int64_t)gridDim.x * 8)
+            warp_row((int32_t)row, rp[row], rp[row + 1]);
     for (int64_t ps = blockIdx.x; ps < npass; ps += gridDim.x) {
         const int32_t base = (int32_t)(ps * rows_per_pass);
         const int nr = min(rows_per_pass, n - base);
@@ -135,19 +160,7 @@ __global__ void __launch_bounds__(256) k_spmv(int32_t n, const int32_t* __restri
                 if (r < nr && jok && es == 0) finish((size_t)(base + r) * nrhs + j, acc, mydot);
             }
         } else {
-            constexpr int EW = 32 / NR;
-            const int j = lane % NR, es = lane / NR;
-            const bool jok = j < nrhs;
-            for (int r = tid >> 5; r < nr; r += 8) {
-                const int32_t row = base + r;
-                const TV xi = (DIFF && jok) ? x[(size_t)row * nrhs + j] : TV(0);
-                TV acc = TV(0);
-                if (jok)
-                    for (int32_t p = srp[r] + es; p < srp[r + 1]; p += EW) acc += term(col[p], val[p], row, j, xi);
-#pragma unroll
-                for (int o = NR; o < 32; o <<= 1) acc += __shfl_xor_sync(kFull, acc, o);
-                if (es == 0 && jok) finish((size_t)row * nrhs + j, acc, wdot);
-            }
+            for (int r = tid >> 5; r < nr; r += 8) warp_row(base + r, srp[r], srp[r + 1]);
         }
         __syncthreads();
     }
@@ -403,7 +416,9 @@ static void launch_spmv_es(const rw_context* ctx, int32_t n, int64_t nnz, const 
         // (a small matrix: at least two passes per SM)
         rows = std::max(std::min(rows, set), std::min(rows, n / (2 * ctx->num_sms)));
         if (rows > set) rows -= rows % set;
-        const int64_t passes = ((int64_t)n + rows - 1) / rows;
+        // long rows: a warp each (see kLongRows); slices that fill the warp ask for that too
+        const bool whole = ctx->opt.spmv_slices > 0 ? NR * ES == 32 : avg * std::max(NR, 4) >= kLongRows;
+        const int64_t passes = whole ? ((int64_t)n + 7) / 8 : ((int64_t)n + rows - 1) / rows;
         static int per_sm = 0;
         if (per_sm < 1) {
             cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_spmv<TA, TV, NR, ES, sizeof(TA) == 4, RES>, 256, 0);
@@ -415,7 +430,7 @@ static void launch_spmv_es(const rw_context* ctx, int32_t n, int64_t nnz, const 
         RW_COUNT_LAUNCH();
         // FP32 values are always the excess + difference form of the mixed mode
         k_spmv<TA, TV, NR, ES, sizeof(TA) == 4, RES>
-            <<<blocks, 256, 0, s>>>(n, rp, col, val, x, y, nrhs, rows, part, b, out32);
+            <<<blocks, 256, 0, s>>>(n, rp, col, val, x, y, nrhs, whole ? 0 : rows, part, b, out32);
     }
 }
 
