@@ -509,8 +509,8 @@ rw_status rw_budget_predict(rw_context* ctx, const rw_csr* A, const rw_mlp* M, d
  *   h_rounds host, optional: the most decisions any row took (the rounds of
  *   a schedule that decides every row once per round).
  * Errors: RW_ERR_ARG (delta, z <= 0; min_walks < 2; max_walks < min_walks or
- * > 65535; max_rounds < 1), RW_ERR_NOT_RMATRIX, RW_ERR_WALK_CAP (a walk hit
- * rw_options.max_steps), RW_ERR_ALLOC, RW_ERR_CUDA.  Synchronous. */
+ * > 65535; max_rounds < 1), RW_ERR_NOT_RMATRIX, RW_ERR_WALK_CAP (a walk that a
+ * decision uses hit rw_options.max_steps), RW_ERR_ALLOC, RW_ERR_CUDA.  Synchronous. */
 rw_status rw_adaptive_budget(rw_context* ctx, const rw_csr* A, uint64_t seed, double delta, double z,
                              uint32_t min_walks, uint32_t max_walks, int32_t max_rounds, uint32_t* d_budget,
                              int32_t* h_rounds);

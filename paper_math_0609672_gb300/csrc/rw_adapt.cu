@@ -147,6 +147,68 @@ __global__ void k_adapt_budget_rows(int32_t nw, const int4* __restrict__ wrow, c
         budget[wrow[r].x] = M[r];
 }
 
+// The launch rounds: each row's walks up to its decision points, `pct` percent
+// past them and the first rows' first round `deep` walks far, until every row is
+// decided; *decisions: the most of a row.
+static rw_status adaptive_rounds(rw_context* ctx, const Tables& T, const AdaptRows& R, uint64_t seed, double d2,
+                                 double z2, uint32_t min_walks, uint32_t max_walks, int32_t max_rounds, uint32_t pct,
+                                 uint32_t deep, uint32_t* inc, unsigned* flags, unsigned long long* hops,
+                                 unsigned* decisions) {
+    cudaStream_t s = ctx->stream;
+    const int32_t n = T.n, nw = T.n_walk_rows;
+    const int gw = grid_for(nw, 256, ctx->num_sms * 8);
+    rw_status rc;
+    if ((rc = check_cuda(cudaMemsetAsync(R.A, 0, sizeof(uint32_t) * (size_t)nw, s), "memset")) ||
+        (rc = check_cuda(cudaMemsetAsync(R.M, 0, sizeof(uint32_t) * (size_t)nw, s), "memset")) ||
+        (rc = check_cuda(cudaMemsetAsync(R.D, 0, sizeof(uint32_t) * (size_t)nw, s), "memset")) ||
+        (rc = check_cuda(cudaMemsetAsync(R.S1, 0, sizeof(unsigned long long) * (size_t)nw, s), "memset")) ||
+        (rc = check_cuda(cudaMemsetAsync(R.S2, 0, sizeof(unsigned long long) * (size_t)nw, s), "memset")) ||
+        (rc = check_cuda(cudaMemsetAsync(inc, 0, sizeof(uint32_t) * (size_t)n, s), "memset")) ||
+        (rc = check_cuda(cudaMemsetAsync(flags, 0, sizeof(unsigned) * 2, s), "memset")))
+        return rc;
+    RW_COUNT_LAUNCH();
+    k_adapt_first<<<gw, 256, 0, s>>>(nw, T.wrow, min_walks, pct, deep, max_walks, R.T, inc);
+    if ((rc = check_launch("adaptive start"))) return rc;
+    unsigned* hp = static_cast<unsigned*>(ctx->h_small);
+    hp[0] = hp[1] = 0u;
+    // Every launch round reaches each pending row's decision point at least
+    // once, so max_rounds launch rounds decide every row.
+    for (int32_t round = 0; round < max_rounds; ++round) {
+        Pool rp(ctx);  // this launch round's walk space and records
+        WalkSpace ws;
+        if ((rc = build_walk_space(ctx, T, 0, inc, ws, rp, true))) return rc;
+        if (ws.total == 0) break;
+        int2* rec = alloc_n<int2>(rp, ws.total);
+        if (!rec) return RW_ERR_ALLOC;
+        WalkBatch wb;
+        wb.m0 = mat_walk(T, seed, 0, 0);  // factor walks: the ones rw_build_factor_budget runs
+        wb.table_bytes = table_bytes(T);
+        wb.huge = has_huge_nodes(T);
+        wb.nrows = T.n_walk_rows;
+        wb.wrow = T.wrow;
+        wb.wbase = ws.wbase;
+        wb.wofs = R.A;  // walks A, A+1, ... of each row
+        wb.chunk_row = ws.chunk_row;
+        wb.total = ws.total;
+        WalkLaunch wl;
+        wl.max_steps = ctx->opt.max_steps;
+        wl.record_lengths = 1;
+        if ((rc = run_walks(ctx, wb, wl, rec, hops, rp, nullptr)) || (rc = read_status(ctx, "adaptive walks")))
+            return rc;
+        if ((rc = check_cuda(cudaMemsetAsync(flags, 0, sizeof(unsigned), s), "memset"))) return rc;
+        RW_COUNT_LAUNCH();
+        k_adapt_chain<<<grid_for((int64_t)nw * 32, 256, ctx->num_sms * 8), 256, 0, s>>>(
+            nw, T.wrow, ws.wbase, rec, R, d2, z2, max_walks, pct, max_rounds, inc, flags, flags + 1);
+        if ((rc = check_launch("adaptive decisions"))) return rc;
+        if ((rc = check_cuda(cudaMemcpyAsync(hp, flags, 2 * sizeof(unsigned), cudaMemcpyDeviceToHost, s), "copy")) ||
+            (rc = check_cuda(cudaStreamSynchronize(s), "sync")))
+            return rc;
+        if (hp[0] == 0u) break;
+    }
+    *decisions = hp[1];
+    return RW_OK;
+}
+
 }  // namespace rw
 
 using namespace rw;
@@ -190,62 +252,26 @@ rw_status rw_adaptive_budget(rw_context* ctx, const rw_csr* A, uint64_t seed, do
     unsigned* flags = alloc_n<unsigned>(sc, 2);  // pending rows, most decisions of a row
     unsigned long long* hops = alloc_n<unsigned long long>(sc, 1);
     if (!R.A || !R.T || !R.M || !R.D || !R.S1 || !R.S2 || !inc || !flags || !hops) return RW_ERR_ALLOC;
-    if ((rc = check_cuda(cudaMemsetAsync(R.A, 0, sizeof(uint32_t) * (size_t)nw, s), "memset")) ||
-        (rc = check_cuda(cudaMemsetAsync(R.M, 0, sizeof(uint32_t) * (size_t)nw, s), "memset")) ||
-        (rc = check_cuda(cudaMemsetAsync(R.D, 0, sizeof(uint32_t) * (size_t)nw, s), "memset")) ||
-        (rc = check_cuda(cudaMemsetAsync(R.S1, 0, sizeof(unsigned long long) * (size_t)nw, s), "memset")) ||
-        (rc = check_cuda(cudaMemsetAsync(R.S2, 0, sizeof(unsigned long long) * (size_t)nw, s), "memset")) ||
-        (rc = check_cuda(cudaMemsetAsync(inc, 0, sizeof(uint32_t) * (size_t)n, s), "memset")) ||
-        (rc = check_cuda(cudaMemsetAsync(flags, 0, sizeof(unsigned) * 2, s), "memset")))
-        return rc;
     const int gw = grid_for(nw, 256, ctx->num_sms * 8);
     const uint32_t pct = ctx->opt.adapt_ahead > 0 ? (uint32_t)ctx->opt.adapt_ahead : 0u;
-    RW_COUNT_LAUNCH();
     const double d2 = delta * delta, z2 = z * z;
     // twice the count of a row whose walk lengths are geometric (standard deviation = mean), 512 at most
     const uint32_t deep = pct > 0 ? (uint32_t)std::min(512.0, std::ceil(2.0 * z2 / d2)) : 0u;
-    k_adapt_first<<<gw, 256, 0, s>>>(nw, T.wrow, min_walks, pct, deep, max_walks, R.T, inc);
-    if ((rc = check_launch("adaptive start"))) return rc;
-    unsigned* hp = static_cast<unsigned*>(ctx->h_small);
-    hp[0] = hp[1] = 0u;
-    // Every launch round reaches each pending row's decision point at least
-    // once, so max_rounds launch rounds decide every row.
-    for (int32_t round = 0; round < max_rounds; ++round) {
-        Pool rp(ctx);  // this launch round's walk space and records
-        WalkSpace ws;
-        if ((rc = build_walk_space(ctx, T, 0, inc, ws, rp, true))) return rc;
-        if (ws.total == 0) break;
-        int2* rec = alloc_n<int2>(rp, ws.total);
-        if (!rec) return RW_ERR_ALLOC;
-        WalkBatch wb;
-        wb.m0 = mat_walk(T, seed, 0, 0);  // factor walks: the ones rw_build_factor_budget runs
-        wb.table_bytes = table_bytes(T);
-        wb.huge = has_huge_nodes(T);
-        wb.nrows = T.n_walk_rows;
-        wb.wrow = T.wrow;
-        wb.wbase = ws.wbase;
-        wb.wofs = R.A;  // walks A, A+1, ... of each row
-        wb.chunk_row = ws.chunk_row;
-        wb.total = ws.total;
-        WalkLaunch wl;
-        wl.max_steps = ctx->opt.max_steps;
-        wl.record_lengths = 1;
-        if ((rc = run_walks(ctx, wb, wl, rec, hops, rp, nullptr)) || (rc = read_status(ctx, "adaptive walks")))
-            return rc;
-        if ((rc = check_cuda(cudaMemsetAsync(flags, 0, sizeof(unsigned), s), "memset"))) return rc;
-        RW_COUNT_LAUNCH();
-        k_adapt_chain<<<grid_for((int64_t)nw * 32, 256, ctx->num_sms * 8), 256, 0, s>>>(
-            nw, T.wrow, ws.wbase, rec, R, d2, z2, max_walks, pct, max_rounds, inc, flags, flags + 1);
-        if ((rc = check_launch("adaptive decisions"))) return rc;
-        if ((rc = check_cuda(cudaMemcpyAsync(hp, flags, 2 * sizeof(unsigned), cudaMemcpyDeviceToHost, s), "copy")) ||
-            (rc = check_cuda(cudaStreamSynchronize(s), "sync")))
-            return rc;
-        if (hp[0] == 0u) break;
+    unsigned decisions = 0u;
+    rc = adaptive_rounds(ctx, T, R, seed, d2, z2, min_walks, max_walks, max_rounds, pct, deep, inc, flags, hops,
+                         &decisions);
+    // A walk that reached the step cap may be one that no decision asks for: only the walks up to the decision
+    // points decide whether the call fails.
+    if (rc == RW_ERR_WALK_CAP && pct > 0u) {
+        if ((rc = reset_status(ctx))) return rc;
+        rc = adaptive_rounds(ctx, T, R, seed, d2, z2, min_walks, max_walks, max_rounds, 0u, 0u, inc, flags, hops,
+                             &decisions);
     }
+    if (rc) return rc;
     RW_COUNT_LAUNCH();
     k_adapt_budget_rows<<<gw, 256, 0, s>>>(nw, T.wrow, R.M, d_budget);
     if ((rc = check_launch("adaptive budget"))) return rc;
-    if (h_rounds) *h_rounds = (int32_t)hp[1];
+    if (h_rounds) *h_rounds = (int32_t)decisions;
     return read_status(ctx, "adaptive budget");
 }
 
