@@ -362,9 +362,10 @@ rw_status rw_probe_gather(rw_context* ctx, uint64_t buffer_bytes, int32_t access
  * scaling by 1/D, forward solve with Y).
  * Concurrency: every solve on a factor (this call, rw_precond_apply_static,
  * pcg_solve, rw_precond_apply_ldu, bicgstab_solve) uses the factor's own solve
- * workspace (grid-barrier words and gathered right-hand sides), so two of them on the same
- * factor must not overlap on the GPU (different streams or threads); calls on
- * different factors may. */
+ * workspace (grid-barrier words and gathered right-hand sides), so two of them on
+ * the same factor must not overlap on the GPU (different streams or threads);
+ * calls on different factors may.  The two-game calls use F_A's workspace and
+ * only read F_AT. */
 rw_status rw_precond_apply(rw_context* ctx, const rw_factor* F, const double* d_r, double* d_z,
                            int32_t nrhs);
 

@@ -674,8 +674,9 @@ static FactorView view_of(const rw_factor* F) {
 }
 
 // The two-game factor of Sec. 7.1: forward data (Y, its schedule, D) from the
-// game on A, backward data (Y^T and its schedule) from the game on A^T.
-static rw_status ldu_view(const rw_factor* FA, const rw_factor* FAT, FactorView* v) {
+// game on A, backward data (Y^T and its schedule) from the game on A^T.  The
+// backward solve's workspace comes from sc, so that F_AT is only read.
+static rw_status ldu_view(const rw_factor* FA, const rw_factor* FAT, int nrhs, FactorView* v, Pool& sc) {
     if (!FA || !FAT || FA->desc.n != FAT->desc.n) {
         set_error("two-game factor: factors missing or of different sizes");
         return RW_ERR_ARG;
@@ -688,6 +689,10 @@ static rw_status ldu_view(const rw_factor* FA, const rw_factor* FAT, FactorView*
     v->yt_val32 = t.yt_val32;
     v->bwd_order = t.bwd_order;
     v->bwd_sched = t.bwd_sched;
+    if (t.bwd_sched->slots > 0) {
+        v->bwd_t = alloc_n<double>(sc, t.bwd_sched->slots * nrhs);
+        if (!v->bwd_t) return RW_ERR_ALLOC;
+    }
     return RW_OK;
 }
 
@@ -712,11 +717,11 @@ rw_status rw_precond_apply_ldu(rw_context* ctx, const rw_factor* F_A, const rw_f
         return RW_ERR_ARG;
     }
     FactorView v;
-    rw_status rc = ldu_view(F_A, F_AT, &v);
+    Pool sc(ctx);
+    rw_status rc = ldu_view(F_A, F_AT, nrhs, &v, sc);
     if (rc) return rc;
     if (v.n == 0) return RW_OK;
     if ((rc = reset_status(ctx))) return rc;
-    Pool sc(ctx);
     rc = precond_fp64(ctx, v, d_r, d_z, nrhs, sc);
     sc.release_all();
     cudaStreamSynchronize(ctx->stream);
@@ -732,7 +737,8 @@ rw_status bicgstab_solve(rw_context* ctx, const rw_csr* A, const rw_factor* F_A,
     rw_status rc = check_csr(A);
     if (rc) return rc;
     FactorView v;
-    if ((rc = ldu_view(F_A, F_AT, &v))) return rc;
+    Pool sc(ctx);
+    if ((rc = ldu_view(F_A, F_AT, 1, &v, sc))) return rc;
     if (v.n != A->n) {
         set_error("bicgstab_solve: matrix and factors do not match");
         return RW_ERR_ARG;

@@ -317,6 +317,7 @@ struct SolveSchedule {
     SolveEntries ext[3];             // entries in the block before, earlier in the stretch, before it
     double* inv = nullptr;           // inverses of the blocks' unit triangles
     float* inv32 = nullptr;
+    int64_t slots = 0;               // of all blocks
     void* t = nullptr;               // workspace: [slots][nrhs] gathered right-hand sides
 };
 
@@ -340,11 +341,12 @@ constexpr int64_t kSolveWorkspaceBytes = 256;
 // (rw_options.solve_mode_bwd may choose its mode).  w, d: when given, w <- w / d
 // row by row (w node-major [n][nrhs]) before the solve starts -- the D^-1 step
 // between the two solves, so that the forward solve's rows need no division of
-// their own; IEEE division as the solve would do it.
+// their own; IEEE division as the solve would do it.  t: workspace of S.slots * nrhs
+// values instead of the schedule's own (NULL).
 template <typename T>
 rw_status solve_runs(rw_context* ctx, const SolveSchedule& S, const int64_t* rp, const int32_t* col,
                      const T* val, const T* rhs, T* x, int nrhs, unsigned* bar, bool backward = false,
-                     T* w = nullptr, const T* d = nullptr);
+                     T* w = nullptr, const T* d = nullptr, void* t = nullptr);
 
 // ---- solve path (rw_solve.cu) ----------------------------------------------
 
@@ -366,6 +368,8 @@ struct FactorView {
     const SolveSchedule* fwd_sched;
     const SolveSchedule* bwd_sched;
     unsigned* bar;  // grid-barrier words of the solves (owned by the factor)
+    // workspace of the backward solve's blocks; NULL: the schedule's own
+    void* bwd_t = nullptr;
 };
 
 void launch_to_fp32(const double* in, float* out, int64_t cnt, cudaStream_t s, int num_sms);

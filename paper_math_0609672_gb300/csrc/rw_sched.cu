@@ -422,6 +422,7 @@ static rw_status schedule_plan(rw_context* ctx, const ScheduleInput& in, SolveSc
     S.trow = alloc_n<int32_t>(pool, nslots);
     S.inv = alloc_n<double>(pool, W.inverse);
     S.inv32 = fp32 ? alloc_n<float>(pool, W.inverse) : nullptr;
+    S.slots = nslots;
     S.t = pool.get((size_t)nslots * 16 * sizeof(double));
     if (!pos_of || !cnt || !ptr || !S.blocks || !S.trow || !S.inv || (fp32 && !S.inv32) || !S.t) return RW_ERR_ALLOC;
     if ((rc = check_cuda(cudaMemcpyAsync(S.blocks, blocks.data(), sizeof(SolveBlock) * (size_t)nb,
@@ -1623,7 +1624,7 @@ static BlockSums<T> block_sums(const SolveEntries& E) {
 template <typename T, int NR>
 static rw_status solve_runs_nr(rw_context* ctx, const SolveSchedule& S, const int64_t* rp,
                                const int32_t* col, const T* val, const T* rhs, T* x, int nrhs, unsigned* bar, int mode,
-                               bool backward, T* w, const T* d) {
+                               bool backward, T* w, const T* d, void* t) {
     cudaStream_t s = ctx->stream;
     rw_status rc;
     const bool rows = mode == 1 || mode == 2;
@@ -1700,7 +1701,7 @@ static rw_status solve_runs_nr(rw_context* ctx, const SolveSchedule& S, const in
         P.inv = schedule_values<T>(S.inv, S.inv32);
         P.rhs = rhs;
         P.x = x;
-        P.t = static_cast<T*>(S.t);
+        P.t = static_cast<T*>(t ? t : S.t);
         P.nrhs = nrhs;
         P.bar = bar;
         P.epoch0 = epoch;
@@ -1722,25 +1723,27 @@ static rw_status solve_runs_nr(rw_context* ctx, const SolveSchedule& S, const in
 
 template <typename T>
 rw_status solve_runs(rw_context* ctx, const SolveSchedule& S, const int64_t* rp, const int32_t* col,
-                     const T* val, const T* rhs, T* x, int nrhs, unsigned* bar, bool backward, T* w, const T* d) {
+                     const T* val, const T* rhs, T* x, int nrhs, unsigned* bar, bool backward, T* w, const T* d,
+                     void* t) {
     NvtxRange nvtx_range(backward ? "rw_solve_bwd" : "rw_solve_fwd");
     if (S.n == 0) return RW_OK;
     const int mode = backward && ctx->opt.solve_mode_bwd >= 0 ? ctx->opt.solve_mode_bwd : ctx->opt.solve_mode;
     int nr = 1;
     while (nr < nrhs) nr <<= 1;
     switch (nr) {
-        case 1: return solve_runs_nr<T, 1>(ctx, S, rp, col, val, rhs, x, nrhs, bar, mode, backward, w, d);
-        case 2: return solve_runs_nr<T, 2>(ctx, S, rp, col, val, rhs, x, nrhs, bar, mode, backward, w, d);
-        case 4: return solve_runs_nr<T, 4>(ctx, S, rp, col, val, rhs, x, nrhs, bar, mode, backward, w, d);
-        case 8: return solve_runs_nr<T, 8>(ctx, S, rp, col, val, rhs, x, nrhs, bar, mode, backward, w, d);
-        default: return solve_runs_nr<T, 16>(ctx, S, rp, col, val, rhs, x, nrhs, bar, mode, backward, w, d);
+        case 1: return solve_runs_nr<T, 1>(ctx, S, rp, col, val, rhs, x, nrhs, bar, mode, backward, w, d, t);
+        case 2: return solve_runs_nr<T, 2>(ctx, S, rp, col, val, rhs, x, nrhs, bar, mode, backward, w, d, t);
+        case 4: return solve_runs_nr<T, 4>(ctx, S, rp, col, val, rhs, x, nrhs, bar, mode, backward, w, d, t);
+        case 8: return solve_runs_nr<T, 8>(ctx, S, rp, col, val, rhs, x, nrhs, bar, mode, backward, w, d, t);
+        default: return solve_runs_nr<T, 16>(ctx, S, rp, col, val, rhs, x, nrhs, bar, mode, backward, w, d, t);
     }
 }
 
 template rw_status solve_runs<double>(rw_context*, const SolveSchedule&, const int64_t*, const int32_t*,
                                       const double*, const double*, double*, int, unsigned*, bool, double*,
-                                      const double*);
+                                      const double*, void*);
 template rw_status solve_runs<float>(rw_context*, const SolveSchedule&, const int64_t*, const int32_t*,
-                                     const float*, const float*, float*, int, unsigned*, bool, float*, const float*);
+                                     const float*, const float*, float*, int, unsigned*, bool, float*, const float*,
+                                     void*);
 
 }  // namespace rw

@@ -504,7 +504,8 @@ static rw_status precond_t(rw_context* ctx, const FactorView& F, const T* yv, co
                            const T* d, const T* r, T* w, T* z, int nrhs, SolveTimes* tm = nullptr) {
     NvtxRange nvtx_range("rw_precond");
     if (tm && tm->on) cudaEventRecord(ctx->ev[5], ctx->stream);
-    rw_status rc = solve_runs<T>(ctx, *F.bwd_sched, F.yt_rp, F.yt_col, ytv, r, w, nrhs, F.bar, true);
+    rw_status rc = solve_runs<T>(ctx, *F.bwd_sched, F.yt_rp, F.yt_col, ytv, r, w, nrhs, F.bar, true, nullptr, nullptr,
+                                 F.bwd_t);
     if (rc) return rc;
     if (tm && tm->on) cudaEventRecord(ctx->ev[6], ctx->stream);
     rc = solve_runs<T>(ctx, *F.fwd_sched, F.y_rp, F.y_col, yv, w, z, nrhs, F.bar, false, w, d);
