@@ -26,8 +26,12 @@ namespace {
 struct Candidate {
     int wide_slices, solve_blocks_per_sm, cluster_width, spmv_slices, solve_mode;
     int solve_mode_bwd = -1;  // -1: as solve_mode
-    int thin_cluster = 0, thin_flags = 0, thin_lanes = 0;  // without effect: options and cache lines that hold them
 };
+
+// Generation of the kernels that the options choose among: part of the cache
+// key, raised whenever an option selects other code than before, so that a line
+// timed on kernels that are gone is not installed.
+constexpr int kTuneGeneration = 2;
 
 std::string shape_key(const rw_context* ctx, const TuneTarget& T, int nrhs) {
     cudaDeviceProp prop{};
@@ -37,10 +41,12 @@ std::string shape_key(const rw_context* ctx, const TuneTarget& T, int nrhs) {
     const int lg_n = (int)std::lround(std::log2(std::max(1, T.n)));
     const double per_row = T.n > 0 ? (double)T.nnz_y / T.n : 0.0;
     const int lg_per_row = (int)std::lround(std::log2(std::max(1.0, per_row)) * 2.0);
+    const double per_row_a = T.n > 0 ? (double)T.nnz_a / T.n : 0.0;  // (the SpMV's slices depend on it)
+    const int lg_per_row_a = (int)std::lround(std::log2(std::max(1.0, per_row_a)) * 2.0);
     const int lg_depth = (int)std::lround(std::log2(std::max(1, T.depth)) * 2.0);
     char buf[512];
-    snprintf(buf, sizeof buf, "%s|sm%d|n2^%d|ypr%d|depth%d|nrhs%d", prop.name, prop.multiProcessorCount, lg_n,
-             lg_per_row, lg_depth, nr);
+    snprintf(buf, sizeof buf, "%s|sm%d|gen%d|n2^%d|apr%d|ypr%d|depth%d|nrhs%d", prop.name, prop.multiProcessorCount,
+             kTuneGeneration, lg_n, lg_per_row_a, lg_per_row, lg_depth, nr);
     for (char* p = buf; *p; ++p)
         if (*p == '"' || *p == '\\') *p = '_';
     return buf;
@@ -68,9 +74,7 @@ bool cache_lookup(const char* path, const std::string& key, Candidate* c) {
         Candidate t{};
         if (json_int(line, "wide_slices", &t.wide_slices) && json_int(line, "solve_blocks_per_sm", &t.solve_blocks_per_sm) &&
             json_int(line, "cluster_width", &t.cluster_width) && json_int(line, "spmv_slices", &t.spmv_slices) &&
-            json_int(line, "solve_mode", &t.solve_mode) && json_int(line, "solve_mode_bwd", &t.solve_mode_bwd) &&
-            json_int(line, "thin_cluster", &t.thin_cluster) && json_int(line, "thin_flags", &t.thin_flags)) {
-            json_int(line, "thin_lanes", &t.thin_lanes);  // absent in older cache lines: 0
+            json_int(line, "solve_mode", &t.solve_mode) && json_int(line, "solve_mode_bwd", &t.solve_mode_bwd)) {
             *c = t;  // the last matching line wins
             found = true;
         }
@@ -84,10 +88,10 @@ void cache_store(const char* path, const std::string& key, const Candidate& c, f
     FILE* f = fopen(path, "a");
     if (!f) return;
     fprintf(f,
-            "{\"key\":\"%s\",\"solve_mode\":%d,\"solve_mode_bwd\":%d,\"thin_cluster\":%d,\"thin_flags\":%d,\"thin_lanes\":%d,\"wide_slices\":%d,\"solve_blocks_per_sm\":%d,\"cluster_width\":%d,"
-            "\"spmv_slices\":%d,\"precond_ms\":%.4f,\"spmv_ms\":%.4f}\n",
-            key.c_str(), c.solve_mode, c.solve_mode_bwd, c.thin_cluster, c.thin_flags, c.thin_lanes, c.wide_slices, c.solve_blocks_per_sm, c.cluster_width, c.spmv_slices, ms_pre,
-            ms_spmv);
+            "{\"key\":\"%s\",\"solve_mode\":%d,\"solve_mode_bwd\":%d,\"wide_slices\":%d,\"solve_blocks_per_sm\":%d,"
+            "\"cluster_width\":%d,\"spmv_slices\":%d,\"precond_ms\":%.4f,\"spmv_ms\":%.4f}\n",
+            key.c_str(), c.solve_mode, c.solve_mode_bwd, c.wide_slices, c.solve_blocks_per_sm, c.cluster_width,
+            c.spmv_slices, ms_pre, ms_spmv);
     fclose(f);
 }
 
@@ -174,9 +178,6 @@ rw_status tune_t(rw_context* ctx, const TuneTarget& X, int nrhs, const T* av, co
     for (const Candidate& c : cands) {
         ctx->opt.solve_mode = c.solve_mode;
         ctx->opt.solve_mode_bwd = c.solve_mode_bwd;
-        ctx->opt.thin_cluster = c.thin_cluster;
-        ctx->opt.thin_flags = c.thin_flags;
-        ctx->opt.thin_lanes = c.thin_lanes;
         ctx->opt.wide_slices = c.wide_slices;
         ctx->opt.solve_blocks_per_sm = c.solve_blocks_per_sm;
         ctx->opt.cluster_width = c.cluster_width;
@@ -189,9 +190,6 @@ rw_status tune_t(rw_context* ctx, const TuneTarget& X, int nrhs, const T* av, co
             bp = ms;
             b.solve_mode = c.solve_mode;
             b.solve_mode_bwd = c.solve_mode_bwd;
-            b.thin_cluster = c.thin_cluster;
-            b.thin_flags = c.thin_flags;
-            b.thin_lanes = c.thin_lanes;
             b.wide_slices = c.wide_slices;
             b.solve_blocks_per_sm = c.solve_blocks_per_sm;
             b.cluster_width = c.cluster_width;
@@ -235,9 +233,6 @@ rw_status autotune(rw_context* ctx, const TuneTarget& X, int nrhs, rw_precision 
     }
     ctx->opt.solve_mode = c.solve_mode;
     ctx->opt.solve_mode_bwd = c.solve_mode_bwd;
-    ctx->opt.thin_cluster = c.thin_cluster;
-    ctx->opt.thin_flags = c.thin_flags;
-    ctx->opt.thin_lanes = c.thin_lanes;
     ctx->opt.wide_slices = c.wide_slices;
     ctx->opt.solve_blocks_per_sm = c.solve_blocks_per_sm;
     ctx->opt.cluster_width = c.cluster_width;
