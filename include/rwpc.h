@@ -93,9 +93,10 @@ typedef struct {
     int32_t refine_every;    /* FP32 PCG: true-residual replacement period (default 50) */
     int32_t walk_blocks_per_sm; /* 0 = from the occupancy calculator */
     int32_t timing;          /* 1: record per-phase device times (default 1) */
-    int32_t solve_blocks_per_sm; /* level schedule and row solves with vector rows: 512-thread blocks
-                                    per SM (0 = 1; 2 = a register-capped row kernel, two blocks
-                                    resident per SM) */
+    int32_t solve_blocks_per_sm; /* 512-thread blocks per SM.  Level schedule: 0 = 1.  Row solves with
+                                    vector rows: 1 = as many as the kernel's registers admit (two at
+                                    most), 2 = a register-capped kernel, two resident per SM, 0 = as 1,
+                                    but lane groups for the backward solve of one FP32 right-hand side */
     int32_t graphs;          /* 1: batched PCG replays each iteration from a CUDA graph (default 1) */
     int32_t wide_slices;     /* wide-level solves: entry slices per row (lanes per row = slices x
                                 right-hand sides, power of two <= 32); 0 = one row per warp;
@@ -322,9 +323,9 @@ rw_status rw_permute_csr(rw_context* ctx, const rw_csr* A, const int32_t* d_perm
  * SpMV entry slices -- and installs the fastest in the context's options
  * (rw_options.solve_mode, wide_slices, solve_blocks_per_sm, cluster_width,
  * spmv_slices), also copied to *out if not NULL.  cache_path (may be NULL): a
- * JSON-lines file; a line whose key matches the device and the problem's
- * shape (log2 n, stored entries per row, depth, nrhs, precision) is used
- * without timing, otherwise the result is appended.  h_ms (host [2], may be
+ * JSON-lines file; a line whose key matches the device, the generation of the
+ * library's kernels and the problem's shape (log2 n, stored entries per row of
+ * A and Y, depth, nrhs, precision) is used without timing, otherwise the result is appended.  h_ms (host [2], may be
  * NULL): the best preconditioner and SpMV times in ms (0 when read from the
  * cache).  The factor and the results of later solves are unchanged; only
  * their speed depends on these options. */

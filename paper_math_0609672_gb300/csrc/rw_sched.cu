@@ -1639,10 +1639,10 @@ static rw_status solve_runs_nr(rw_context* ctx, const SolveSchedule& S, const in
     auto solve_rows = [&](int64_t slot0, int64_t slot1, bool pack) -> rw_status {
         const RowParams<T> P{slot1 - slot0, S.rows + slot0, col, val, rhs, x, nrhs, ctx->d_status};
         if constexpr (NR * sizeof(T) <= 32) {
-            // One FP32 right-hand side backward: the entries of the long rows of Y^T over lane groups, two thread
-            // blocks per SM (k_rows), 3.8 -> 3.2 ms per solve of 10^6 nodes with long-range edges, 1.19 -> 1.12 ms
-            // on a 56^3 27-point grid; forward the same costs 2.4 -> 2.9 ms.
-            const bool groups = sizeof(T) * NR == 4 && backward && !pack;
+            // One FP32 right-hand side backward, blocks per SM left to the library: the entries of the long rows of
+            // Y^T over lane groups, two thread blocks per SM (k_rows), 3.8 -> 3.2 ms per solve of 10^6 nodes with
+            // long-range edges, 1.19 -> 1.12 ms on a 56^3 27-point grid; forward the same costs 2.4 -> 2.9 ms.
+            const bool groups = sizeof(T) * NR == 4 && backward && !pack && ctx->opt.solve_blocks_per_sm <= 0;
             if (ctx->opt.wide_slices < 0 && !groups) return launch_rows<T, NR, true>(ctx, P, pack);
         }
         return launch_rows<T, NR, false>(ctx, P, false);

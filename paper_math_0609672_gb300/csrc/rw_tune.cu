@@ -31,7 +31,7 @@ struct Candidate {
 // Generation of the kernels that the options choose among: part of the cache
 // key, raised whenever an option selects other code than before, so that a line
 // timed on kernels that are gone is not installed.
-constexpr int kTuneGeneration = 2;
+constexpr int kTuneGeneration = 3;
 
 std::string shape_key(const rw_context* ctx, const TuneTarget& T, int nrhs) {
     cudaDeviceProp prop{};
@@ -175,6 +175,8 @@ rw_status tune_t(rw_context* ctx, const TuneTarget& X, int nrhs, const T* av, co
     cands.push_back(Candidate{-1, 2, 0, 0, 2});     // the same, two blocks per SM
     cands.push_back(Candidate{slices[0], 1, 0, 0, 2});  // the same, lane groups
     cands.push_back(Candidate{-1, 1, 0, 0, 1, 2});  // sync-free forward, blocks backward
+    if (sizeof(T) == 4 && nr == 1)  // vector rows forward, lane groups backward
+        for (int mode : {1, 2}) cands.push_back(Candidate{-1, 0, 0, 0, mode});
     for (const Candidate& c : cands) {
         ctx->opt.solve_mode = c.solve_mode;
         ctx->opt.solve_mode_bwd = c.solve_mode_bwd;
