@@ -425,14 +425,27 @@ def _walk_roofline(P, ctx, peaks, peak_kind, As, hops, walk_ms, l2_bytes, tag):
                        "dram_gbs": (tph * hops / (walk_ms * 1e-3) / 1e9) if tph else None}}
 
 
-def _solve_kernels(opt):
-    """Names of the triangular-solve kernels the tuned options run."""
-    def one(mode):
-        free = "k_rows_vec" if opt.get("wide_slices") == -1 else "k_rows"
-        return free if mode == 1 else f"k_blocks/{free}" if mode == 2 else "k_wide"
-    fwd = one(opt.get("solve_mode", 0))
-    bwd = one(opt.get("solve_mode_bwd", -1) if opt.get("solve_mode_bwd", -1) >= 0 else opt.get("solve_mode", 0))
-    return f"{fwd} (forward) + {bwd} (backward)"
+def _solve_kernels(opt, nrhs, mixed):
+    """Names of the triangular-solve kernels the tuned options run: blocks of
+    narrow levels (modes 0 and 2), and for the other rows vector rows while an
+    entry's right-hand sides fit in 32 bytes (the widest levels packed for one
+    of them, mode 2), lane groups otherwise and for the backward solve of one
+    FP32 right-hand side with the blocks per SM left open; or level by level
+    (mode 0)."""
+    nr = 1 << (nrhs - 1).bit_length()
+    vec = opt.get("wide_slices") == -1 and nr * (4 if mixed else 8) <= 32
+
+    def one(mode, backward):
+        if mode not in (1, 2):
+            return "k_blocks/k_wide"
+        groups = backward and mixed and nr == 1 and opt.get("solve_blocks_per_sm", 0) <= 0
+        free = "k_rows_vec" if vec and not groups else "k_rows"
+        pack = "/k_rows_pack" if mode == 2 and vec and nr == 1 else ""
+        return free if mode == 1 else f"k_blocks/{free}{pack}"
+
+    mode = opt.get("solve_mode", 0)
+    bwd = opt.get("solve_mode_bwd", -1)
+    return f"{one(mode, False)} (forward) + {one(bwd if bwd >= 0 else mode, True)} (backward)"
 
 
 def _solve_roofline(peaks, napply, nnz_y, n, nrhs, tri_ms, vbytes, ybytes, kernels="triangular solves"):
@@ -544,7 +557,7 @@ def run_gpu_single(args, P, torch, dev, stream, ws, rank, local):
     tri_ms = statistics.mean(i["bwd_ms"] + i["fwd_ms"] for i in infos)
     solve_roof = _solve_roofline(peaks, napply, infos[-1]["nnz"], A.n, nrhs, tri_ms,
                                  4.0 if mixed else 8.0, 8.0 if mixed else 12.0,
-                                 _solve_kernels(tuned))
+                                 _solve_kernels(tuned, nrhs, mixed))
     # latency view of the solves: each level of a solve waits for at least one
     # value stored by another SM, so one SM-to-SM hand-off per level is a floor
     nlev = infos[-1]["fwd"] + infos[-1]["bwd"]
