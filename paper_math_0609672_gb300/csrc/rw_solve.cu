@@ -36,8 +36,7 @@ constexpr int kDotParts = 1024;  // blocks of the dot-product producing kernels
 // sides and 406 us with one; now 249 and 237 us (1.0e11 gathers/s).
 // Passes whose entries exceed the copy or that hold a row of more than
 // kLongRow entries per lane sum their rows with all 32 lanes each, straight
-// from memory; matrices of long rows take no passes (rows_per_pass 0: a warp per
-// row throughout).
+// from memory; matrices of long rows take a warp per row throughout (k_spmv_rows).
 //
 // DIFF (the FP32 operator of the mixed mode): val holds A_ij (j != i) and, at
 // the diagonal position, the excess e_i = A_ii + sum_j A_ij, and the row is
@@ -50,12 +49,13 @@ constexpr int kSpmvEntries = 2048;  // entries of a pass (24 KB of columns and F
 constexpr int kSpmvRows = 512;      // rows of a pass
 constexpr int kLongRow = 64;
 // Average entries per row times right-hand sides (four at least) from which
-// every row is summed by a warp, straight from memory.  A pass then holds too
+// every row is summed by a warp (k_spmv_rows).  A pass of k_spmv then holds too
 // few rows for the copy to pay, and from 1000 entries a row only one or two, so
-// that most of the block idles.  Warp per row against the copy, us: 6000 rows of
-// 920 entries 27 | 70 (one right-hand side), 176 | 507 (16); 30,000 of 129 37 | 34
-// and 128 | 154; 200,000 of 65 134 | 89, 206 | 146 (three), 271 | 285 (eight) and
-// 420 | 467 (16); 60,000 of 33 46 | 27 and 83 | 88.
+// that most of the block idles.  k_spmv | k_spmv_rows, us: 6000 rows of 920
+// entries 60 | 27 (one right-hand side), 430 | 180 (16); 8000 of 497 35 | 27 and
+// 163 | 141; 30,000 of 129 42 | 36 and 154 | 132; 16 right-hand sides on 40,000 of
+// 65 100 | 96 and on 60,000 of 33 88 | 83.  Below the line: 200,000 of 65 with one
+// 89 | 134, with three 146 | 206.
 constexpr int kLongRows = 512;
 
 // RES: the true residual b - A x of PCG instead of A x: stored as FP32
@@ -92,23 +92,7 @@ __global__ void __launch_bounds__(256) k_spmv(int32_t n, const int32_t* __restri
             if (part) dot += (double)x[at] * (double)acc;
         }
     };
-    // row `row`, entries [s, e), by the warp, straight from memory
-    auto warp_row = [&](int32_t row, int32_t s, int32_t e) {
-        constexpr int EW = 32 / NR;
-        const int j = lane % NR, es = lane / NR;
-        const bool jok = j < nrhs;
-        const TV xi = (DIFF && jok) ? x[(size_t)row * nrhs + j] : TV(0);
-        TV acc = TV(0);
-        if (jok)
-            for (int32_t p = s + es; p < e; p += EW) acc += term(col[p], val[p], row, j, xi);
-#pragma unroll
-        for (int o = NR; o < 32; o <<= 1) acc += __shfl_xor_sync(kFull, acc, o);
-        if (es == 0 && jok) finish((size_t)row * nrhs + j, acc, wdot);
-    };
-    const int64_t npass = rows_per_pass ? ((int64_t)n + rows_per_pass - 1) / rows_per_pass : 0;
-    if (npass == 0)
-        for (int64_t row = (int64_t)blockIdx.x * 8 + (tid >> 5); row < n; row += (int64_t)gridDim.x * 8)
-            warp_row((int32_t)row, rp[row], rp[row + 1]);
+    const int64_t npass = ((int64_t)n + rows_per_pass - 1) / rows_per_pass;
     for (int64_t ps = blockIdx.x; ps < npass; ps += gridDim.x) {
         const int32_t base = (int32_t)(ps * rows_per_pass);
         const int nr = min(rows_per_pass, n - base);
@@ -160,7 +144,19 @@ __global__ void __launch_bounds__(256) k_spmv(int32_t n, const int32_t* __restri
                 if (r < nr && jok && es == 0) finish((size_t)(base + r) * nrhs + j, acc, mydot);
             }
         } else {
-            for (int r = tid >> 5; r < nr; r += 8) warp_row(base + r, srp[r], srp[r + 1]);
+            constexpr int EW = 32 / NR;
+            const int j = lane % NR, es = lane / NR;
+            const bool jok = j < nrhs;
+            for (int r = tid >> 5; r < nr; r += 8) {
+                const int32_t row = base + r;
+                const TV xi = (DIFF && jok) ? x[(size_t)row * nrhs + j] : TV(0);
+                TV acc = TV(0);
+                if (jok)
+                    for (int32_t p = srp[r] + es; p < srp[r + 1]; p += EW) acc += term(col[p], val[p], row, j, xi);
+#pragma unroll
+                for (int o = NR; o < 32; o <<= 1) acc += __shfl_xor_sync(kFull, acc, o);
+                if (es == 0 && jok) finish((size_t)row * nrhs + j, acc, wdot);
+            }
         }
         __syncthreads();
     }
@@ -178,6 +174,58 @@ __global__ void __launch_bounds__(256) k_spmv(int32_t n, const int32_t* __restri
             for (int i = tid; i < 256; i += lanes) t += sdot[i];
             for (int i = tid; i < 256; i += NR) t += sdot[256 + i];
             part[(size_t)blockIdx.x * 16 + tid] = t;
+        }
+    }
+}
+
+// Matrices of long rows: a warp per row, straight from memory.  A kernel of its
+// own: in k_spmv the loop cost every other matrix registers (spills, 253 -> 263 us
+// on the 27-point grid above), and without the copy's shared memory L1 holds more
+// of x.
+template <typename TA, typename TV, int NR, bool DIFF, bool RES>
+__global__ void __launch_bounds__(256) k_spmv_rows(int32_t n, const int32_t* __restrict__ rp,
+                                                   const int32_t* __restrict__ col, const TA* __restrict__ val,
+                                                   const TV* __restrict__ x, TV* __restrict__ y, int nrhs,
+                                                   double* part, const double* __restrict__ b, int out32) {
+    constexpr int EW = 32 / NR;
+    __shared__ double sdot[8][NR];
+    const int lane = (int)lane_id(), warp = (int)threadIdx.x >> 5;
+    const int j = lane % NR, es = lane / NR;
+    const bool jok = j < nrhs;
+    double dot = 0.0;
+    for (int64_t row = (int64_t)blockIdx.x * 8 + warp; row < n; row += (int64_t)gridDim.x * 8) {
+        const int32_t s = rp[row], e = rp[row + 1];
+        const size_t at = (size_t)row * nrhs + j;
+        const TV xi = (DIFF && jok) ? x[at] : TV(0);
+        TV acc = TV(0);
+        if (jok)
+            for (int32_t p = s + es; p < e; p += EW) {
+                const int32_t c = col[p];
+                const TV a = (TV)val[p], xc = x[(size_t)c * nrhs + j];
+                if (DIFF) acc += c == row ? a * xi : a * (xc - xi);
+                else acc += a * xc;
+            }
+#pragma unroll
+        for (int o = NR; o < 32; o <<= 1) acc += __shfl_xor_sync(kFull, acc, o);
+        if (es == 0 && jok) {
+            if constexpr (RES) {
+                const double t = b[at] - (double)acc;
+                if (y && out32) reinterpret_cast<float*>(y)[at] = (float)t;
+                else if (y) y[at] = (TV)t;
+                dot += t * t;
+            } else {
+                y[at] = acc;
+                if (part) dot += (double)x[at] * (double)acc;
+            }
+        }
+    }
+    if (part) {
+        if (es == 0) sdot[warp][j] = dot;
+        __syncthreads();
+        if ((int)threadIdx.x < nrhs) {
+            double t = 0.0;
+            for (int w = 0; w < 8; ++w) t += sdot[w][threadIdx.x];
+            part[(size_t)blockIdx.x * 16 + threadIdx.x] = t;
         }
     }
 }
@@ -416,9 +464,7 @@ static void launch_spmv_es(const rw_context* ctx, int32_t n, int64_t nnz, const 
         // (a small matrix: at least two passes per SM)
         rows = std::max(std::min(rows, set), std::min(rows, n / (2 * ctx->num_sms)));
         if (rows > set) rows -= rows % set;
-        // long rows: a warp each (see kLongRows); slices that fill the warp ask for that too
-        const bool whole = ctx->opt.spmv_slices > 0 ? NR * ES == 32 : avg * std::max(NR, 4) >= kLongRows;
-        const int64_t passes = whole ? ((int64_t)n + 7) / 8 : ((int64_t)n + rows - 1) / rows;
+        const int64_t passes = ((int64_t)n + rows - 1) / rows;
         static int per_sm = 0;
         if (per_sm < 1) {
             cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_spmv<TA, TV, NR, ES, sizeof(TA) == 4, RES>, 256, 0);
@@ -430,8 +476,20 @@ static void launch_spmv_es(const rw_context* ctx, int32_t n, int64_t nnz, const 
         RW_COUNT_LAUNCH();
         // FP32 values are always the excess + difference form of the mixed mode
         k_spmv<TA, TV, NR, ES, sizeof(TA) == 4, RES>
-            <<<blocks, 256, 0, s>>>(n, rp, col, val, x, y, nrhs, whole ? 0 : rows, part, b, out32);
+            <<<blocks, 256, 0, s>>>(n, rp, col, val, x, y, nrhs, rows, part, b, out32);
     }
+}
+
+template <typename TA, typename TV, int NR, bool RES>
+static void launch_spmv_rows(const rw_context* ctx, int32_t n, const int32_t* rp, const int32_t* col, const TA* val,
+                             const TV* x, TV* y, int nrhs, double* part, int* blocks_out, cudaStream_t s,
+                             const double* b, int out32) {
+    int blocks = grid_for(n, 8, ctx->num_sms * 8);
+    if (part && blocks > kDotParts) blocks = kDotParts;
+    if (blocks_out) *blocks_out = blocks;
+    RW_COUNT_LAUNCH();
+    k_spmv_rows<TA, TV, NR, sizeof(TA) == 4, RES>
+        <<<blocks, 256, 0, s>>>(n, rp, col, val, x, y, nrhs, part, b, out32);
 }
 
 // Entry slices per row: the option, else one, doubled until the rows that the
@@ -442,6 +500,9 @@ template <typename TA, typename TV, int NR, bool RES>
 static void launch_spmv_nr(const rw_context* ctx, int32_t n, int64_t nnz, const int32_t* rp, const int32_t* col,
                            const TA* val, const TV* x, TV* y, int nrhs, double* part, int* blocks, cudaStream_t s,
                            const double* b, int out32) {
+    // long rows: a warp each (see kLongRows); slices that fill the warp ask for that too
+    if (ctx->opt.spmv_slices > 0 ? ctx->opt.spmv_slices >= 32 / NR : nnz * std::max(NR, 4) >= (int64_t)kLongRows * n)
+        return launch_spmv_rows<TA, TV, NR, RES>(ctx, n, rp, col, val, x, y, nrhs, part, blocks, s, b, out32);
     int p = 1;
     if (ctx->opt.spmv_slices > 0) {
         while (p * 2 <= ctx->opt.spmv_slices && p * 2 * NR <= 32) p *= 2;
