@@ -281,6 +281,7 @@ struct SolveRow {
 // by level; pack: levels padded to whole groups of rows.
 struct SolveStretch {
     int64_t pos0, pos1, slot0, slot1;
+    int64_t inv0;  // where its blocks' inverses start
     int32_t lev0, lev1;
     int32_t block0, nblocks;
     bool pack;

@@ -259,25 +259,22 @@ __global__ void __launch_bounds__(32) k_block_invert(const InvertJob J0, const I
         const int64_t p0 = e0, p1 = e1;
         fetch(r + 1);  // in flight while this row is summed
         double acc = 0.0;
-        bool hit = false;
+        int bits = 0;  // of the factors: zero when no product contributes (no branches: they cost more than the products)
         auto term = [&](int s, double yv) {
-            const double xv = X[(s - c0) * kPanel + j];
+            const double xv = s >= c0 ? X[(s - c0) * kPanel + j] : 0.0;
             acc += yv * xv;
-            hit |= nonzero(xv);
+            bits |= __double2hiint(xv) | __double2loint(xv);
         };
 #pragma unroll
-        for (int u = 0; u < U; ++u)
-            if (cs[u] >= c0) term(cs[u], cy[u]);
-        for (int64_t p = p0 + q + 4 * U; p < p1; p += 4) {
-            const int s = islot[p];
-            if (s >= c0) term(s, ival[p]);
-        }
+        for (int u = 0; u < U; ++u) term(cs[u], cy[u]);
+        for (int64_t p = p0 + q + 4 * U; p < p1; p += 4) term(islot[p], ival[p]);
+        const unsigned hits = __ballot_sync(kFull, bits != 0);
         acc += __shfl_xor_sync(kFull, acc, 8);
         acc += __shfl_xor_sync(kFull, acc, 16);
         const int c = c0 + j;
         double v = (r == c ? 1.0 : 0.0) - (r >= c ? acc : 0.0);
-        hit = ((__ballot_sync(kFull, hit) >> j) & 0x01010101u) != 0u;  // in any of the column's four lanes
-        if (hit && !nonzero(v)) v = __longlong_as_double(1);
+        const bool hit = ((hits >> j) & 0x01010101u) != 0u;  // in any of the column's four lanes
+        v = __hiloint2double(__double2hiint(v), __double2loint(v) | (hit && !nonzero(v) ? 1 : 0));
         if (q == 0) X[(r - c0) * kPanel + j] = v;
         __syncwarp();
         if (q == 0 && c <= r) {
@@ -378,7 +375,8 @@ static rw_status schedule_plan(rw_context* ctx, const ScheduleInput& in, SolveSc
             }
         }
         if (kind == 2) slots = (slots + kPackRows - 1) / kPackRows * kPackRows;
-        SolveStretch st{S.lptr_h[l], S.lptr_h[e], slots, 0, l, e, (int32_t)blocks.size(), 0, kind == 2};
+        SolveStretch st{S.lptr_h[l], S.lptr_h[e], slots, 0, W.inverse, l, e, (int32_t)blocks.size(), 0,
+                        kind == 2};
         for (int32_t i = l; i < e; ++i) {
             slot0[i] = slots;
             slots += S.lptr_h[i + 1] - S.lptr_h[i];
@@ -1391,7 +1389,6 @@ __global__ void __launch_bounds__(256, 1) k_blocks(const BlockParams<T> P) {
     int64_t q1 = 0, q0 = 0;
     T y[U], iv[V];
     auto fetch = [&](int64_t b) {
-        const int64_t inv0 = P.blocks[b].inv0;
         mine = slot < P.blocks[b].rows;
         const int64_t t = b * kBlockRows + slot;
         q0 = q1 = 0;
@@ -1406,7 +1403,7 @@ __global__ void __launch_bounds__(256, 1) k_blocks(const BlockParams<T> P) {
             c[u] = ok ? P.prev.idx[q0 + 32 * u] : -1;
             y[u] = ok ? P.prev.val[q0 + 32 * u] : T(0);
         }
-        const T* inv = P.inv + inv0 + tri(slot);
+        const T* inv = P.inv + (b - P.block0) * tri(kBlockRows) + tri(slot);  // (every block before is full)
 #pragma unroll
         for (int k = 0; k < V; ++k) iv[k] = mine && lane + 32 * k <= slot ? inv[lane + 32 * k] : T(0);
     };
@@ -1453,11 +1450,12 @@ __global__ void __launch_bounds__(256, 1) k_blocks(const BlockParams<T> P) {
                     T v[W][NR];
 #pragma unroll
                     for (int k = 0; k < W; ++k)
-                        if (nonzero(iv[k0 + k]))
+                        if (lane + 32 * (k0 + k) <= slot)
                             xload_cg<T, NR>(P.t, nr, b * kBlockRows + lane + 32 * (k0 + k), v[k]);
 #pragma unroll
                     for (int k = 0; k < W; ++k)
                         if (32 * (k0 + k) <= slot) {  // (FP64 instructions only for what the row holds)
+                            // (the loads above do not wait for the inverse)
 #pragma unroll
                             for (int j = 0; j < NR; ++j)
                                 acc[j] += nonzero(iv[k0 + k]) ? iv[k0 + k] * v[k][j] : T(0);
@@ -1698,7 +1696,7 @@ static rw_status solve_runs_nr(rw_context* ctx, const SolveSchedule& S, const in
         P.prev = block_sums<T>(S.ext[0]);
         P.older = block_sums<T>(S.ext[1]);
         P.from_rhs = st.pos0 == 0;
-        P.inv = schedule_values<T>(S.inv, S.inv32);
+        P.inv = schedule_values<T>(S.inv, S.inv32) + st.inv0;
         P.rhs = rhs;
         P.x = x;
         P.t = static_cast<T*>(t ? t : S.t);
