@@ -208,7 +208,7 @@ rw_status rw_context_create(rw_context** out, void* stream, rw_alloc_fn alloc, r
         (rc = check_cuda(cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, c->device), "device attribute")) ||
         (rc = check_cuda(cudaMalloc(&c->d_status, sizeof(DevStatus)), "cudaMalloc status")) ||
         (rc = check_cuda(cudaMallocHost(&c->h_status, sizeof(DevStatus)), "cudaMallocHost")) ||
-        (rc = check_cuda(cudaMallocHost(&c->h_small, 4096), "cudaMallocHost"))) {
+        (rc = check_cuda(cudaMallocHost(&c->h_small, kSmallBytes), "cudaMallocHost"))) {
         rw_context_destroy(c);
         return rc;
     }

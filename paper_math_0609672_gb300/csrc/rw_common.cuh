@@ -101,8 +101,8 @@ __device__ __forceinline__ void st_relaxed(int* p, int v) {
 }
 
 // Bit patterns marking "not yet computed" in the sync-free triangular solves.
-// They are NaN payloads that arithmetic never produces (GPU arithmetic returns
-// the canonical NaN), and inputs are checked to be finite.
+// They are signalling NaNs, which arithmetic never produces (its NaNs are quiet),
+// whatever the inputs hold: every value published is the result of a subtraction.
 __device__ __forceinline__ double pending_value(double) {
     return __longlong_as_double(0x7FF4C0DEC0DE0001LL);
 }

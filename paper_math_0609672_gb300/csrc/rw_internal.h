@@ -22,7 +22,7 @@ struct rw_context {
     int num_sms = 0;
     rw::DevStatus* d_status = nullptr;  // device copy
     rw::DevStatus* h_status = nullptr;  // pinned host copy
-    void* h_small = nullptr;            // pinned host scratch (256 bytes)
+    void* h_small = nullptr;            // pinned host scratch (rw::kSmallBytes)
     double reuse_ratio = 8.0;           // walk reuse: extra records per walk to allocate for
     size_t l2_bytes = 0;                // L2 cache size of the device
     size_t mem_bytes = 0;               // memory of the device
@@ -41,6 +41,8 @@ struct NvtxRange {
     NvtxRange(const NvtxRange&) = delete;
     NvtxRange& operator=(const NvtxRange&) = delete;
 };
+
+constexpr size_t kSmallBytes = 4096;  // rw_context::h_small
 
 constexpr int kFeatures = RW_NUM_FEATURES;
 constexpr int kFeatStride = RW_FEATURE_STRIDE;

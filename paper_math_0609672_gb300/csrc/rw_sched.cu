@@ -28,8 +28,8 @@
 // other in one thread block, the others sync-free with every lane polling its
 // own values) and now: 32^2 grid, 709 levels each way, 1.65 -> 0.076 ms; 300^2
 // grid in natural order, 48,350 levels, 109 -> 4.0 ms; 64^3 7-point, 1198
-// levels, four right-hand sides 6.9 -> 2.5 ms, sixteen 28 -> 6.3 ms; 1000^2
-// with long-range edges, 2229 levels, FP32 8.5 -> 6.4 ms.
+// levels, four right-hand sides 6.9 -> 2.4 ms, sixteen 28 -> 6.3 ms; 1000^2
+// with long-range edges, 2229 levels, FP32 8.5 -> 4.6 ms.
 //
 // solve_mode 1 takes every row as in a wide stretch; solve_mode 0 solves the
 // narrow stretches as blocks too and the other levels one after another over the

@@ -268,6 +268,7 @@ struct PcgScalars {
     int any_check;
     int pad;
 };
+static_assert(sizeof(PcgScalars) <= kSmallBytes, "the host copy lies in the context's pinned scratch");
 
 // Threads of a block that work on an [n][nrhs] array element by element, each
 // on one right-hand side (tid % nrhs): whole groups of nrhs threads.

@@ -94,16 +94,7 @@ constexpr int kRefill = 8;
 constexpr int kTeamLanes = 8;
 constexpr int kTeams = 32 / kTeamLanes;
 
-// 32 bytes (eight words) in one load; p must be 32-byte aligned (sectors are).
-__device__ __forceinline__ void ld_nc8(const uint32_t* p, uint4& lo, uint4& hi) {
-    asm("ld.global.nc.v8.u32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-        : "=r"(lo.x), "=r"(lo.y), "=r"(lo.z), "=r"(lo.w), "=r"(hi.x), "=r"(hi.y), "=r"(hi.z), "=r"(hi.w)
-        : "l"(p));
-}
-
-// The same with an L2 cache-policy operand (createpolicy): evict_last keeps
-// the summaries and group bases in L2 while the group sectors stream through
-// with evict_first, when the tables are larger than the L2.
+// 32 bytes (eight words) in one load with a cache policy; p must be 32-byte aligned (sectors are).
 __device__ __forceinline__ void ld_nc8_hint(const uint32_t* p, uint4& lo, uint4& hi, uint64_t pol) {
     asm("ld.global.nc.L2::cache_hint.v8.u32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8], %9;"
         : "=r"(lo.x), "=r"(lo.y), "=r"(lo.z), "=r"(lo.w), "=r"(hi.x), "=r"(hi.y), "=r"(hi.z), "=r"(hi.w)
@@ -283,8 +274,12 @@ __device__ __forceinline__ uint32_t block_room(uint64_t max_steps, uint64_t h) {
 // straight-line; the next block of draws is computed while loads are in
 // flight.  Lanes of a team hold the same state.  Runs until every walk has
 // ended or one is within a block of the step cap; the walks left are then in
-// the teams' first lanes.  64^3 7-point grid, one walk per row (its longest
-// walk sets the time): see the launch's comment for the figures.
+// the teams' first lanes.  48^3 27-point grid, 20 walks a row, longest walk
+// 54,670 hops: 38.7 ms with the last walks in single lanes, 18.3 ms with teams.
+// Launches with a node of more than eight groups (more than 31 neighbours) keep
+// single lanes throughout: a team has a lane for each of eight groups.  The same
+// grid, 200 walks a row: 26 ms, and 43 ms with one row of 1000 neighbours more
+// (49 ms before the rounds of four hops).
 template <bool MULTI>
 __device__ __forceinline__ void drain_walks(const WalkParams& P, bool& active, WalkState& S, int32_t& m,
                                             unsigned long long& my_hops, const Policies& pol) {
