@@ -101,7 +101,9 @@ typedef struct {
     int32_t wide_slices;     /* wide-level solves: entry slices per row (lanes per row = slices x
                                 right-hand sides, power of two <= 32); 0 = one row per warp;
                                 -1 = vector rows: one row per warp, each lane reads all
-                                right-hand sides of its entries (default -1) */
+                                right-hand sides of its entries; with solve_mode 2 and one
+                                right-hand side four rows per warp on the widest levels
+                                (default -1) */
     int32_t spmv_slices;     /* SpMV: entry slices per row (lanes per row = slices x right-hand sides, power
                                 of two <= 32); 0 = from the average row length (default 0) */
     int32_t cluster_width;   /* level schedule: levels of at most this many rows run on one thread-block
@@ -360,7 +362,8 @@ rw_status rw_probe_gather(rw_context* ctx, uint64_t buffer_bytes, int32_t access
 
 /* z = (Y^T diag(D) Y)^-1 r for nrhs node-major right-hand sides (FP64): the
  * preconditioner application inside pcg_solve (backward solve with Y^T,
- * scaling by 1/D, forward solve with Y).
+ * scaling by 1/D, forward solve with Y).  r is not checked to be finite: a
+ * non-finite entry makes the results that depend on it non-finite and no others.
  * Concurrency: every solve on a factor (this call, rw_precond_apply_static,
  * pcg_solve, rw_precond_apply_ldu, bicgstab_solve) uses the factor's own solve
  * workspace (grid-barrier words and gathered right-hand sides), so two of them on
